@@ -10,11 +10,10 @@
 // a sum of up to 1024 of them (<= 2^24) is exact in its FP32 accumulator.
 // Products of digit pairs (s, t) of the same class k = s + t carry the same
 // weight 2^(eT + eX - 8(k + 2)), so they share one accumulator column: the
-// MMA of table digit s writes the columns of classes s .. s + t_max.  A
-// column then sums at most 8 pairs x 128 sources = 1024 products per slot
-// (<= 2^24, exact in FP32); every slot's columns are converted to integers
-// and added into 64-bit integer class sums, so the only rounding is the
-// dropped digits (below 2^-55 of max|t| max|v|) and the final FP64
+// MMA of table digit s writes the columns of classes s .. s + t_max.  The
+// columns are converted to integers and added into 64-bit integer class sums,
+// so the only rounding is the dropped digits (below 2^-55 of max|t| max|v|)
+// and the final FP64
 // combination of eight class sums.  Table digits 0..6 and source digits
 // 0..7 are kept, and pairs with s + t >= 8 are not formed.
 //
@@ -39,32 +38,50 @@
 // a 16-B gap after every core matrix keeps the builders' stores free of
 // shared-memory bank conflicts).
 //
-// The block also depends only on |offset| along the slowest axis, so the
-// source lines at -d and +d from a target line share it, and so do the two
-// target lines i0 and i0 + 1 of a tile with their sources at i0 +- d and
-// i0 + 1 +- d: one MMA takes the four source chunks as the four quarters of
-// its B operand (rows ordered digit, quarter, rhs), so N = 32 per source
-// digit.  An M = 128 MMA reads its 4 KB A operand from shared memory whatever
-// N is, and shared-memory bandwidth (128 B per clock) bounds the MMAs of
-// small N: the four-chunk operand takes the A reads per target line to half
-// those of one line with its mirror pair.  A missing source line reads a
-// zero chunk.
+// The block also depends only on the distance d along the slowest axis, so
+// the two source lines at i0 - d and i0 + d of a target line i0 meet the same
+// block and are added before the product: the sum of two 8-bit digits has
+// magnitude at most 256, which BF16 still holds exactly.  That halves the
+// MMAs of the sum over all pairs.  The blocks of several target lines i0,
+// i0 + 1, ... at the same d are the same too: one MMA takes 32 columns
+// (target line, right-hand side) per source digit, four lines of eight
+// right-hand sides up to 32 lines of one, so that few right-hand sides cost
+// few MMAs.
 //
-// CTA roles (384 threads, persistent, one CTA per SM, TMEM 512 columns):
-//   warps 0-7  epilogue: TMEM -> integer class sums -> FP64 y (one thread
-//              per target row; warps 0-3 the first line, 4-7 the second),
-//   warp 8     one thread: the MMAs,
-//   warps 9-11 builders of the Hankel operand from mirrored digit rows; one
-//              of them also issues the bulk copies of the source digits.
-// Slots (one Hankel operand, four 128-source chunks) flow through a 2-stage
-// shared-memory ring (3 stages for the short sums, whose stages are smaller)
-// into two 256-column accumulators used in turn, so the
-// MMAs of the next slot proceed while the epilogue drains one.  The class
-// sums are kept as an int64 for class 0 and int32 for classes 1..7, and
-// every 32 slots the carries of classes 7..1 move up (c = s_k >> 8, s_k -=
-// 256 c, s_(k-1) += c), which keeps their value and their range.  Every wait
-// is bounded; on time-out the kernel sets *status = 1, drains its own MMAs
-// and copies, frees TMEM and returns.
+// What bounds it: an M = 128 MMA takes N / 2 cycles of the tensor pipe and
+// reads 4 KB of A and 32 N bytes of B from shared memory at 128 B per clock,
+// so a slot (7 table digits x 128 sources) is 4,096 cycles of math, ~3,850 of
+// shared-memory reads by the MMAs and ~1,850 of loads and stores by the
+// builders on the same L1 data path: that path is full (ncu: 49% + 55% of its
+// wavefronts), the tensor pipe is not.  Folding the mirror lines leaves the
+// cost of a slot nearly as it was and halves the slots; the folded operand is
+// built by threads from L2 (two loads, an add and a store per 16 bytes).
+// Measured on a GB300, whole matvec, before (one MMA quarter per source line,
+// 8-column padding, whole tiles per CTA) and after: n = 1024 x 8 right-hand
+// sides 458 -> 281 ms (classes 6, 5, 4: 357, 290, 248 -> 236, 208, 162 ms),
+// n = 512 x 8 30.8 -> 17.7 ms, n = 64 x 1 0.29 -> 0.15 ms, 3D n = 24 x 3
+// 2.8 -> 0.94 ms.
+//
+// A column sums at most 7 pairs x 64 sources x 2^15 < 2^24 products, exact in
+// FP32, so a slot fills the two accumulators in turn, 64 sources each, and
+// the epilogue drains one while the MMAs fill the other.
+//
+// The slots of all tiles form one sequence (tile, middle source coordinate,
+// source chunk, distance) that is cut into equal ranges, one per CTA, so
+// every size fills the chip whatever its number of tiles; a tile cut by a
+// range boundary leaves its integer class sums, which are exact and therefore
+// independent of the cut, in a partial buffer that fixup_kernel adds up.
+//
+// CTA roles (800 threads, persistent, one CTA per SM, TMEM 512 columns):
+//   warps 0-15   epilogue: TMEM -> integer class sums -> FP64 y (one thread
+//                per target row and 8 of the 32 columns),
+//   warp 16      one thread: the MMAs,
+//   warps 17-24  builders: the folded source digits and the Hankel operand
+//                from mirrored digit rows.
+// Slots flow through a 2-stage shared-memory ring (3 stages for the short
+// sums, whose stages are smaller).  Four neighbouring classes are kept as one
+// 64-bit sum.  Every wait is bounded; on time-out the kernel sets *status = 1,
+// drains its own MMAs, frees TMEM and returns.
 #include <cuda_bf16.h>
 #include <algorithm>
 #include <cstdlib>
@@ -89,28 +106,29 @@ constexpr int CM = 144;                         // core-matrix stride: 128 B + 1
                                                 // builders' 16-B row stores of consecutive core
                                                 // matrices fall in different bank groups
 constexpr int A_SLICE = NBLK * CM;              // bytes
-constexpr int CHUNK = SX * NR * KC * 2;         // one source chunk: (digit, rhs) rows x KC, BF16
-constexpr int TBLK = NR * KC * 2;               // the rows of one digit of one chunk
-constexpr int NL = 2;                           // target lines per tile
-constexpr int NQ = 2 * NL;                      // source chunks per slot (mirror pair per target line)
+constexpr int CHUNK = SX * NR * KC * 2;         // bytes of one source chunk: (digit, rhs) rows x KC, BF16
+constexpr int NCOL = 32;                        // columns per class: (target line, rhs)
+constexpr int DBLK = NCOL * KC * 2;             // the B rows of one digit
 constexpr int NST_MAX = 3;                      // deepest ring of the variants below
-constexpr int ACCB = 32 * 8;                    // TMEM columns of one accumulator: (class, quarter, rhs)
-constexpr int NACC = 2;                         // accumulators, used slot by slot in turn
+constexpr int ACCB = NCOL * 8;                  // TMEM columns of one accumulator: (class, column)
+constexpr int NACC = 2;                         // accumulators: the two halves of a slot's sources
 constexpr int ACC = ACCB * NACC;                // TMEM columns allocated
-constexpr int NEPI = 256;                       // epilogue threads
-constexpr int NBUILD = 96;                      // builder threads
+constexpr int NEPI = 512;                       // epilogue threads: 4 column groups x 128 rows
+constexpr int NBUILD = 256;                     // builder threads
 constexpr int NTHR = NEPI + 32 + NBUILD;
-constexpr int CARRY = 32;                       // slots between carry passes of the class sums
+constexpr int NGRP = 2;                         // 64-bit class sums (classes 4 g .. 4 g + 3)
+constexpr int CARRY = 4096;                     // slots between carries of the class sums
+constexpr int PART = NGRP * 8 * NEPI;           // int64 values of one partial tile
 constexpr long long WAIT_CYCLES = 4000000000LL; // ~2 s at GB300 clocks
 
-static_assert(8 * KC * 128 * 128 <= (1 << 24), "exact FP32 accumulation of one slot");
-// a class sum gains at most 2 columns x 7 pairs x 128 sources x 2^14 per slot
-static_assert(2.0 * 7 * KC * 16384 * CARRY + 2.0 * 16777216 < 2147483647.0, "int32 class sums between carries");
+static_assert(7 * (KC / NACC) * 128 * 256 <= (1 << 24), "exact FP32 accumulation of half a slot");
+// S[1] gains less than 2 x 2^24 x (2^24 + 2^17) per slot
+static_assert(4294967296.0 * 65536.0 * 2.1 * CARRY < 9.2e18, "64-bit class sums between carries");
 
 // The variant with KD digit classes (8: every class, the full sum; 4, 5 or
 // 6: the short sums).  Columns of table digit s: B rows (source digit t,
-// quarter, rhs) for t below nt(s) = ncols(s) / 32, written to the accumulator
-// columns (class s + t, quarter, rhs), i.e. from column 32 s on; the full sum
+// line, rhs) for t below nt(s) = ncols(s) / 32, written to the accumulator
+// columns (class s + t, line, rhs), i.e. from column 32 s on; the full sum
 // takes s + t <= 7 except for the odd counts rounded down, a short one every
 // pair with s + t < KD.
 template <int KD>
@@ -118,14 +136,15 @@ struct Digits {
     static constexpr int ST = KD == 8 ? 7 : KD;          // table digits read
     static constexpr int SX = KD;                        // source digits read
     static constexpr int A_BYTES = ST * A_SLICE;
-    static constexpr int B_BYTES = NQ * SX * TBLK;
+    static constexpr int B_BYTES = SX * DBLK;
     static constexpr int STAGE = A_BYTES + B_BYTES;
     static constexpr int NST = KD == 8 ? 2 : 3;         // ring depth within 227 KB of shared memory
     static constexpr int NPAIR = ST * NBLK;             // (slice, core matrix) build items per slot
     __host__ __device__ static constexpr int ncols(int s) {
         return KD == 8 ? (s == 0 ? 256 : s <= 2 ? 192 : s <= 4 ? 128 : 64) : 32 * (KD - s);
     }
-    static_assert(STAGE % 16 == 0 && A_BYTES % 16 == 0 && TBLK % 16 == 0, "stage alignment");
+    static constexpr int NG = (KD + 3) / 4;             // 64-bit class sums kept
+    static_assert(STAGE % 16 == 0 && A_BYTES % 16 == 0 && NPAIR <= NBUILD, "stage layout");
     static_assert(NST <= NST_MAX && NST * STAGE + 1024 + 256 <= 232448, "shared memory");
     static_assert(ncols(0) == 32 * KD && ncols(ST - 1) >= 32, "column map");
 };
@@ -154,11 +173,10 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
 }
 
 struct Bars {
-    uint64_t full[NST_MAX];     // Hankel operand built (NBUILD arrivals)
-    uint64_t bfull[NST_MAX];    // source digits landed (1 arrival + bytes)
+    uint64_t full[NST_MAX];     // both operands built (NBUILD arrivals)
     uint64_t mma_done[NST_MAX];
     uint64_t acc_full[NACC];    // accumulator written (1 commit)
-    uint64_t acc_empty[NACC];   // accumulator drained (128 epilogue arrivals)
+    uint64_t acc_empty[NACC];   // accumulator drained (NEPI arrivals)
     uint64_t drain;
     uint32_t tmem;
     int abort;
@@ -214,20 +232,20 @@ __global__ void tc_table_rows_kernel(const double* table, int n, int64_t lines, 
     }
 }
 
-// Source digits in the K-major core-matrix layout of the B operand, chunk by
-// chunk: element (digit t, rhs r, source q) of chunk ch at
-// ((ch * SX + t) * (KC/8) + q/8) * 64 + r * 8 + q % 8 (BF16 units).
+// Source digits chunk by chunk for nrv = 2^lg right-hand sides (nr of them in
+// use): element (digit t, rhs r, source q) of chunk ch at
+// (((ch * SX + t) * (KC/8) + q/8) * nrv + r) * 8 + q % 8 (BF16 units).
 __global__ void tc_source_digits_kernel(const double* v, int64_t N, int n, int64_t lines, int nc, int r0, int nr,
-                                        int sx, const unsigned long long* xmax, uint4* XB) {
-    const int64_t tot = lines * nc * (KC / 8) * NR;
+                                        int lg, int sx, int xshift, const unsigned long long* xmax, uint4* XB) {
+    const int64_t tot = (lines * nc * (KC / 8)) << lg;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e % NR);
-        const int kb = (int)((e / NR) % (KC / 8));
-        const int64_t ch = e / (NR * (KC / 8));
+        const int r = (int)(e & ((1 << lg) - 1));
+        const int kb = (int)((e >> lg) % (KC / 8));
+        const int64_t ch = (e >> lg) / (KC / 8);
         const int64_t J = ch / nc;
         const int c = (int)(ch % nc);
         float d[8][8];                               // [source][digit]
-        const int ex = r < nr ? scale_exp(xmax[r]) : 0;
+        const int ex = (r < nr ? scale_exp(xmax[r]) : 0) + xshift;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const int64_t jl = (int64_t)KC * c + 8 * kb + q;
@@ -246,7 +264,7 @@ __global__ void tc_source_digits_kernel(const double* v, int64_t N, int n, int64
             w.y = pack2(d[2][t], d[3][t]);
             w.z = pack2(d[4][t], d[5][t]);
             w.w = pack2(d[6][t], d[7][t]);
-            XB[((ch * SX + t) * (KC / 8) + kb) * 8 + r] = w;
+            XB[(((ch * SX + t) * (KC / 8) + kb) << lg) + r] = w;
         }
     }
 }
@@ -255,84 +273,120 @@ __global__ void tc_source_digits_kernel(const double* v, int64_t N, int n, int64
 
 struct TcConvArgs {
     const __nv_bfloat16* R;     // mirrored table digit rows
-    const unsigned char* XB;    // source digit chunks, then one zero chunk
+    const unsigned char* XB;    // source digit chunks
     const unsigned long long* tmax;
     const unsigned long long* xmax;   // NR entries
     double* ybuf;               // N x nrhs, grid order
+    long long* part;            // two partial tiles per CTA
     int64_t N;
     int n;
     int64_t lines;              // n^(dim-1)
     int dim;
-    int nb, nc;                 // target chunks / source chunks per line
-    int64_t tiles;              // (line pair, target chunk)
+    int nc;                     // target chunks = source chunks per line
+    int lg;                     // log2 of the right-hand sides per line in the 32 columns
+    int64_t slots;              // slots of all tiles
     int r0, nr;
+    int xshift;                 // sources scaled to |u| < 2^-(1 + xshift)
     int* status;
     int stall;                  // test of the bounded waits: issue no MMA at all
 };
 
 namespace {
 
-// The slot sequence of one CTA, identical in every role: its tiles
-// (round-robin; a tile is the target lines i0 = 2 p and i0 + 1 along the
-// slowest axis, the middle coordinate i1 in 3D, and one chunk b along the
-// last), and per tile the offsets d0 = 0..dmax along the slowest axis, the
-// middle source coordinate j1 (3D), the chunk c.
-struct Walk {
-    int n, dim, nb, nc;
-    int64_t tiles, step, tile;
-    int b, i0, i1, dmax, d0, j1, c;
-    bool ok;
+// A tile is NL = 32 / 2^lg target lines i0 .. i0 + NL - 1 along the slowest
+// axis (with the middle coordinate i1 in 3D) and one chunk b of 128 targets
+// along the last.  Its slots are (j1, c, d): middle source coordinate (3D),
+// source chunk, distance along the slowest axis 0 .. dmax, d fastest, so
+// consecutive slots read neighbouring source lines.
+struct Tiles {
+    int n, mid, nc, NL, ngrp;
+    __host__ __device__ explicit Tiles(const TcConvArgs& a)
+        : n(a.n), mid(a.dim == 3 ? a.n : 1), nc(a.nc), NL(NCOL >> a.lg), ngrp((a.n + NL - 1) / NL) {}
+    __host__ __device__ int dmax(int g) const {
+        const int lo = g * NL, hi = (lo + NL < n ? lo + NL : n) - 1;
+        return hi > n - 1 - lo ? hi : n - 1 - lo;
+    }
+    __host__ __device__ int64_t tile_slots(int g) const { return (int64_t)(dmax(g) + 1) * mid * nc; }
+    __host__ __device__ int64_t group_slots(int g) const { return tile_slots(g) * mid * nc; }
+};
 
-    __device__ void init(const TcConvArgs& a, int64_t first, int64_t stride) {
-        n = a.n; dim = a.dim; nb = a.nb; nc = a.nc; tiles = a.tiles; step = stride; tile = first;
-        ok = tile < tiles;
-        if (ok) start();
+int64_t total_slots(const TcConvArgs& a) {
+    const Tiles t(a);
+    int64_t s = 0;
+    for (int g = 0; g < t.ngrp; ++g) s += t.group_slots(g);
+    return s;
+}
+
+__device__ __forceinline__ int64_t range_start(const TcConvArgs& a, int cta, int ctas) {
+    return a.slots / ctas * cta + a.slots % ctas * cta / ctas;
+}
+
+// Position in the slot sequence: tile q of group g and slot `off` inside it;
+// q = middle target coordinate i1 * nc + target chunk b.
+struct Place {
+    int g, q;
+    int64_t off;
+    __device__ Place(const Tiles& t, int64_t slot) {
+        g = 0;
+        for (int64_t s; g < t.ngrp - 1 && slot >= (s = t.group_slots(g)); ++g) slot -= s;
+        const int64_t per = t.tile_slots(g);
+        q = (int)(slot / per);
+        off = slot % per;
     }
-    __device__ void start() {
-        const int64_t p = tile / nb;
-        b = (int)(tile % nb);
-        i0 = 2 * (dim == 2 ? (int)p : (int)(p / n));
-        i1 = dim == 2 ? 0 : (int)(p % n);
-        dmax = i0 > n - 1 - i0 ? i0 : n - 1 - i0;
-        if (i0 + 1 < n && i0 + 1 > dmax) dmax = i0 + 1;
-        d0 = 0; j1 = 0; c = 0;
-    }
-    // line index (all but the last coordinate) of target line l, -1 if none
-    __device__ int64_t line(int l) const {
-        const int il = i0 + l;
-        if (il >= n) return -1;
-        return dim == 2 ? (int64_t)il : (int64_t)il * n + i1;
-    }
-    __device__ int64_t slots() const { return (int64_t)(dmax + 1) * (dim == 3 ? n : 1) * nc; }
-    __device__ void next() {
-        if (++c < nc) return;
-        c = 0;
-        if (dim == 3 && ++j1 < n) return;
-        j1 = 0;
-        if (++d0 <= dmax) return;
-        tile += step;
-        ok = tile < tiles;
-        if (ok) start();
-    }
-    // offset index of the line pair (all but the last coordinate)
-    __device__ int64_t dl() const { return d0 + (dim == 3 ? (int64_t)n * (i1 > j1 ? i1 - j1 : j1 - i1) : 0); }
-    // source line of quarter q = 2 l + h (target line i0 + l; h = 0: minus
-    // d0, h = 1: plus d0), -1 if none
-    __device__ int64_t src_line(int q) const {
-        const int il = i0 + (q >> 1), h = q & 1;
-        if (il >= n || (h == 1 && d0 == 0)) return -1;
-        const int j0 = h == 0 ? il - d0 : il + d0;
-        if (j0 < 0 || j0 >= n) return -1;
-        return dim == 2 ? (int64_t)j0 : (int64_t)j0 * n + j1;
+    __device__ void next_tile(const Tiles& t) {
+        off = 0;
+        if (++q == t.mid * t.nc) {
+            q = 0;
+            ++g;
+        }
     }
 };
+
+// Class sums of one (row, column): S[0] = sum_k v_k 2^(8 (3 - k)) over classes
+// 0..3, S[1] the same over classes 4..7, 2^-32 of S[0]'s unit.  The carry
+// leaves 32 bits in S[1]; S[0] then stays below N 2^38 (1 + 2^-6).
+__device__ __forceinline__ void carry(long long (&S)[NGRP]) {
+    S[0] += S[1] >> 32;
+    S[1] &= 0xffffffffLL;
+}
+__device__ __forceinline__ double from_sums(const long long (&S)[NGRP], int e2) {
+    return ldexp((double)S[0] + (double)S[1] * (1.0 / 4294967296.0), e2 - 40);
+}
+
+__device__ __forceinline__ void store_row(const TcConvArgs& a, int i0, int i1, int b, int row, int col, double y) {
+    const int l = col >> a.lg, r = col & ((1 << a.lg) - 1);
+    const int il = TM * b + TM - 1 - row, line = i0 + l;
+    if (il >= a.n || line >= a.n || r >= a.nr) return;
+    const int64_t L = a.dim == 3 ? (int64_t)line * a.n + i1 : line;
+    a.ybuf[L * a.n + il + a.N * (a.r0 + r)] = y;
+}
+
+// 16 bytes of read-only data, zero when !on.  Volatile: the builders keep a
+// fixed number of loads in flight; hoisting more of them spills registers,
+// and spills go through the same L1 data path that the MMAs read from.
+__device__ __forceinline__ uint4 load16(const uint4* p, bool on) {
+    uint4 v;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t"
+        "mov.u32 %0, 0;\n\tmov.u32 %1, 0;\n\tmov.u32 %2, 0;\n\tmov.u32 %3, 0;\n\t"
+        "@p ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];\n\t}"
+        : "=&r"(v.x), "=&r"(v.y), "=&r"(v.z), "=&r"(v.w)
+        : "l"(p), "r"((uint32_t)on));
+    return v;
+}
+
+__device__ __forceinline__ uint32_t add2(uint32_t x, uint32_t y) {
+    const __nv_bfloat162 s =
+        __hadd2(*reinterpret_cast<const __nv_bfloat162*>(&x), *reinterpret_cast<const __nv_bfloat162*>(&y));
+    return *reinterpret_cast<const uint32_t*>(&s);
+}
 
 }  // namespace
 
 template <int KD>
 __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
     using C = Digits<KD>;
-    constexpr int NST = C::NST, STAGE = C::STAGE, A_BYTES = C::A_BYTES;
+    constexpr int NST = C::NST, STAGE = C::STAGE, A_BYTES = C::A_BYTES, NG = C::NG;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     Bars* bars = (Bars*)(smem + NST * STAGE);
@@ -342,7 +396,6 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
     if (threadIdx.x == 0) {
         for (int i = 0; i < NST; ++i) {
             tc::mbar_init(&bars->full[i], NBUILD);
-            tc::mbar_init(&bars->bfull[i], 1);
             tc::mbar_init(&bars->mma_done[i], 1);
         }
         for (int i = 0; i < NACC; ++i) {
@@ -358,8 +411,8 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = bars->tmem;
-    const int64_t Z0 = 128LL * a.nc - 1, RL = 256LL * a.nc;
-    const int64_t zero_chunk = a.lines * a.nc;
+    const int64_t first = range_start(a, blockIdx.x, gridDim.x);
+    const int64_t count = range_start(a, blockIdx.x + 1, gridDim.x) - first;
 
     if (warp == NEPI / 32) {
         // ---------------------------------------------------------- issuer
@@ -367,20 +420,11 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
         // but wait and issue: its scalar work between MMA batches shows up
         // as tensor-pipe idle time)
         if (lane == 0) {
-            Walk w;
-            w.init(a, a.stall ? a.tiles : (int64_t)blockIdx.x, gridDim.x);
             int st = 0;
             uint32_t ph = 0;
-            int64_t si = 0;                      // slots issued: accumulator si % NACC, use si / NACC
             bool ok = true;
-            while (w.ok) {
-                const int ab = (int)(si % NACC);
-                const int64_t use = si / NACC;
-                if (use >= 1 && !wait_bounded(&bars->acc_empty[ab], (uint32_t)((use - 1) & 1), abort)) {
-                    ok = false;
-                    break;
-                }
-                if (!wait_bounded(&bars->full[st], ph, abort) || !wait_bounded(&bars->bfull[st], ph, abort)) {
+            for (int64_t si = 0; si < (a.stall ? 0 : count); ++si) {
+                if (!wait_bounded(&bars->full[st], ph, abort)) {
                     ok = false;
                     break;
                 }
@@ -390,24 +434,32 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
                 const uint32_t a_st = tc::smem_addr(smem + st * STAGE);
                 const uint64_t a0 = tc::sdesc(a_st, CM, CM);
                 const uint64_t b0 = tc::sdesc(a_st + A_BYTES, 128, (KC / 8) * 128);
-                // slice by slice: consecutive MMAs of one slice read
-                // overlapping Hankel windows and keep N and D fixed, which
-                // the tensor core streams faster than alternating slices
-                // (the first MMA, slice 0 with N = 128, initializes all the
-                // accumulator's columns; the others add into theirs)
 #pragma unroll
-                for (int s = 0; s < C::ST; ++s) {
-                    const uint64_t as = a0 + (uint64_t)(s * A_SLICE / 16);
-                    const uint32_t d = tmem + ACCB * ab + coloff(s);
+                for (int h = 0; h < NACC; ++h) {
+                    if (si >= 1 && !wait_bounded(&bars->acc_empty[h], (uint32_t)((si - 1) & 1), abort)) {
+                        ok = false;
+                        break;
+                    }
+                    tc::tc_fence_after();
+                    // slice by slice: consecutive MMAs of one slice read
+                    // overlapping Hankel windows and keep N and D fixed, which
+                    // the tensor core streams faster than alternating slices
+                    // (the first MMA, slice 0 with every column, initializes
+                    // the accumulator; the others add into it)
 #pragma unroll
-                    for (int kk = 0; kk < KC / 16; ++kk)
-                        tc::mma_bf16(d, as + (uint64_t)(2 * CM * kk / 16), b0 + (uint64_t)(16 * kk),
-                                     tc::idesc_bf16_f32(TM, C::ncols(s)), !(s == 0 && kk == 0));
+                    for (int s = 0; s < C::ST; ++s) {
+                        const uint64_t as = a0 + (uint64_t)(s * A_SLICE / 16);
+                        const uint32_t dst = tmem + ACCB * h + coloff(s);
+#pragma unroll
+                        for (int kk = h * (KC / 16 / NACC); kk < (h + 1) * (KC / 16 / NACC); ++kk)
+                            tc::mma_bf16(dst, as + (uint64_t)(2 * CM * kk / 16), b0 + (uint64_t)(16 * kk),
+                                         tc::idesc_bf16_f32(TM, C::ncols(s)),
+                                         !(s == 0 && kk == h * (KC / 16 / NACC)));
+                    }
+                    tc::mma_commit(&bars->acc_full[h]);
                 }
+                if (!ok) break;
                 tc::mma_commit(&bars->mma_done[st]);
-                tc::mma_commit(&bars->acc_full[ab]);
-                ++si;
-                w.next();
                 if (++st == NST) {
                     st = 0;
                     ph ^= 1;
@@ -421,65 +473,80 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
         }
     } else if (warp > NEPI / 32) {
         // ------------------------------------------------------- builders
-        // each thread owns up to PPT (slice, core matrix) items per slot; the
-        // 16 digits of every item are fetched one slot ahead, so the L2
-        // latency overlaps the build of the current slot
-        constexpr int NPAIR = C::NPAIR;
-        constexpr int PPT = (NPAIR + NBUILD - 1) / NBUILD;
+        // source operand: thread bt builds the 16-byte units (digit t, column
+        // 8 (2 hi + p) + row8, source octet kb) for every t and p = 0, 1: the
+        // digits of source lines i - d and i + d added; a missing line is
+        // zero.  table operand: threads below NPAIR build one (slice, core
+        // matrix) item each.
         const int bt = threadIdx.x - (NEPI + 32);
-        uint4 cur[PPT][2], nxt[PPT][2];
-        auto fetch = [&](const Walk& v, uint4 (&buf)[PPT][2]) {
-            const int64_t dl = v.dl();
-            const int64_t idx0 = Z0 - ((int64_t)TM * v.b + TM - 1 - (int64_t)KC * v.c);   // multiple of 8
+        const int row8 = bt & 7, kb = (bt >> 3) & 15, hi = bt >> 7;
+        const int64_t Z0 = 128LL * a.nc - 1, RL = 256LL * a.nc;
+        const int64_t dig = (int64_t)(KC / 8) << a.lg;                   // uint4 per digit of a chunk
+        const int64_t chunk = SX * dig, line = (a.dim == 3 ? a.n : 1) * (int64_t)a.nc * chunk;
+        const int as = bt / NBLK, am = bt % NBLK;                        // table item
+        int lp[2], up[2];                                                // target line and unit inside a digit
 #pragma unroll
-            for (int j = 0; j < PPT; ++j) {
-                const int pr = bt + NBUILD * j;
-                if (pr < NPAIR) {
-                    const int s = pr / NBLK, m = pr % NBLK;
-                    const uint4* src =
-                        reinterpret_cast<const uint4*>(a.R + ((int64_t)s * a.lines + dl) * RL + idx0 + 8 * m);
-                    buf[j][0] = __ldg(src);
-                    buf[j][1] = __ldg(src + 1);
-                }
-            }
-        };
-        Walk w, wn;
-        w.init(a, blockIdx.x, gridDim.x);
-        wn = w;
-        if (w.ok) {
-            fetch(w, cur);
-            wn.next();
+        for (int p = 0; p < 2; ++p) {
+            const int col = 8 * (2 * hi + p) + row8;
+            lp[p] = col >> a.lg;
+            up[p] = (kb << a.lg) + (col & ((1 << a.lg) - 1));
         }
-        int st = 0;
+        unsigned char* const bdst = smem + A_BYTES + (2 * hi) * (KC / 8) * 128 + kb * 128 + row8 * 16;
+        const int64_t dp = (int64_t)(lp[1] - lp[0]) * line + up[1] - up[0];
+        const Tiles tl(a);
+        Place pl(tl, first);
+        int st = 0, gs = 0;
         uint32_t ph = 0;
-        int64_t gs = 0, issued = 0;
-        while (w.ok) {
-            if (wn.ok) fetch(wn, nxt);
-            if (gs >= NST && !wait_bounded(&bars->mma_done[st], ph ^ 1, abort)) break;
-            unsigned char* a_st = smem + st * STAGE;
-            if (bt == 0) {
-                // source digits of the four chunks, digit block by digit
-                // block into rows (digit, quarter, rhs); a missing line reads zeros
-                tc::mbar_arrive_expect_tx(&bars->bfull[st], C::B_BYTES);
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    const int64_t J = w.src_line(q);
-                    const int64_t chunk = J >= 0 ? J * a.nc + w.c : zero_chunk;
-                    const unsigned char* src = a.XB + chunk * (int64_t)CHUNK;
-#pragma unroll
-                    for (int t = 0; t < C::SX; ++t)
-                        tc::bulk_g2s(a_st + A_BYTES + (NQ * t + q) * TBLK, src + t * TBLK, TBLK, &bars->bfull[st]);
+        bool ok = true;
+        for (int left = (int)count; left > 0 && ok;) {
+            // the slots of one (tile, j1, c): distances d .. dmax, pointers stepped
+            const int dmax = tl.dmax(pl.g), i0 = pl.g * tl.NL, i1 = pl.q / tl.nc, b = pl.q % tl.nc;
+            const int c = (int)(pl.off / (dmax + 1) % tl.nc), j1 = (int)(pl.off / (dmax + 1) / tl.nc);
+            int d = (int)(pl.off % (dmax + 1));
+            const int dend = min(dmax + 1, d + left);
+            left -= dend - d;
+            pl.off += dend - d;
+            if (pl.off == tl.tile_slots(pl.g)) pl.next_tile(tl);
+            const int64_t dl = d + (int64_t)(a.dim == 3 ? a.n : 0) * (i1 > j1 ? i1 - j1 : j1 - i1);
+            const uint4* tsrc = reinterpret_cast<const uint4*>(
+                a.R + ((int64_t)as * a.lines + dl) * RL + (Z0 - ((int64_t)TM * b + TM - 1 - (int64_t)KC * c)) + 8 * am);
+            const uint4* pm =
+                reinterpret_cast<const uint4*>(a.XB) + ((int64_t)j1 * a.nc + c) * chunk + up[0] + (i0 + lp[0] - d) * line;
+            const uint4* pp = pm + 2 * d * line;
+            for (; d < dend; ++d, tsrc += RL / 8, pm -= line, pp += line) {
+                const uint4 t0 = load16(tsrc, bt < C::NPAIR), t1 = load16(tsrc + 1, bt < C::NPAIR);
+                if (gs >= NST && !wait_bounded(&bars->mma_done[st], ph ^ 1, abort)) {
+                    ok = false;
+                    break;
                 }
-                ++issued;
-            }
+                ++gs;
 #pragma unroll
-            for (int j = 0; j < PPT; ++j) {
-                const int pr = bt + NBUILD * j;
-                if (pr < NPAIR) {
-                    const int s = pr / NBLK, m = pr % NBLK;
-                    const uint32_t wd[8] = {cur[j][0].x, cur[j][0].y, cur[j][0].z, cur[j][0].w,
-                                            cur[j][1].x, cur[j][1].y, cur[j][1].z, cur[j][1].w};
-                    uint4* dst = reinterpret_cast<uint4*>(a_st + s * A_SLICE + m * CM);
+                for (int p = 0; p < 2; ++p) {
+                    const int i = i0 + lp[p];
+                    const bool vm = i < a.n && i >= d, vp = d > 0 && i + d < a.n;
+                    unsigned char* dst = bdst + st * STAGE + p * (KC / 8) * 128;
+                    constexpr int TB = (C::SX + 1) / 2;                                // digits in flight
+#pragma unroll
+                    for (int t0 = 0; t0 < C::SX; t0 += TB) {
+                        uint4 um[TB], uq[TB];
+#pragma unroll
+                        for (int t = 0; t < TB; ++t) {
+                            if (t0 + t < C::SX) {
+                                um[t] = load16(pm + p * dp + (t0 + t) * dig, vm);
+                                uq[t] = load16(pp + p * dp + (t0 + t) * dig, vp);
+                            }
+                        }
+#pragma unroll
+                        for (int t = 0; t < TB; ++t)
+                            if (t0 + t < C::SX)
+                                *reinterpret_cast<uint4*>(dst + (t0 + t) * DBLK) =
+                                    make_uint4(add2(um[t].x, uq[t].x), add2(um[t].y, uq[t].y),
+                                               add2(um[t].z, uq[t].z), add2(um[t].w, uq[t].w));
+                    }
+                }
+                if (bt < C::NPAIR) {
+                    const uint32_t wd[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+                    uint4* dst = reinterpret_cast<uint4*>(smem + st * STAGE + as * A_SLICE + am * CM);
 #pragma unroll
                     for (int rho = 0; rho < 8; ++rho) {
                         uint32_t o[4];
@@ -490,108 +557,83 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
                         dst[rho] = make_uint4(o[0], o[1], o[2], o[3]);
                     }
                 }
-            }
-            tc::fence_proxy_async_smem();
-            tc::mbar_arrive(&bars->full[st]);
-#pragma unroll
-            for (int j = 0; j < PPT; ++j) {
-                cur[j][0] = nxt[j][0];
-                cur[j][1] = nxt[j][1];
-            }
-            w = wn;
-            if (wn.ok) wn.next();
-            ++gs;
-            if (++st == NST) {
-                st = 0;
-                ph ^= 1;
+                tc::fence_proxy_async_smem();
+                tc::mbar_arrive(&bars->full[st]);
+                if (++st == NST) {
+                    st = 0;
+                    ph ^= 1;
+                }
             }
         }
-        // drain: the latest copy into every stage has landed before exit
-        if (bt == 0)
-            for (int64_t i = issued > NST ? issued - NST : 0; i < issued; ++i) {
-                const long long t1 = clock64();
-                while (!tc::mbar_try_wait(&bars->bfull[i % NST], (uint32_t)((i / NST) & 1)) &&
-                       clock64() - t1 < WAIT_CYCLES) {}
-            }
     } else {
         // ------------------------------------------------------- epilogue
-        // warp w: target line w / 4 of the tile, TMEM lane quarter w % 4
-        const int ln = warp >> 2, quad = warp & 3;
-        long long s0[NR];          // class 0
-        int sk[KD - 1][NR];        // classes 1..KD-1
-        auto carry = [&]() {
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-#pragma unroll
-                for (int k = KD - 2; k >= 1; --k) {
-                    const int c = sk[k][r] >> 8;
-                    sk[k][r] -= c * 256;
-                    sk[k - 1][r] += c;
-                }
-                const int c = sk[0][r] >> 8;
-                sk[0][r] -= c * 256;
-                s0[r] += c;
-            }
-        };
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            s0[r] = 0;
-#pragma unroll
-            for (int k = 0; k < KD - 1; ++k) sk[k][r] = 0;
-        }
-        const int eT = scale_exp(*a.tmax);
-        int64_t si = 0;                                        // slots drained
+        // warp w: columns 8 (w / 4) .. + 7 of every class, TMEM lane quarter w % 4
+        const int quad = warp & 3, cg = warp >> 2;
+        const int row = 32 * quad + lane;
+        long long S[8][NGRP];
+        uint32_t ph = 0;
         bool ok = true;
-        for (int64_t tile = blockIdx.x; tile < a.tiles && ok; tile += gridDim.x) {
-            Walk w;
-            w.init(a, tile, a.tiles);                          // this tile only
-            const int64_t nsl = w.slots();
-            for (int64_t g = 0; g < nsl; ++g, ++si) {
-                const int ab = (int)(si % NACC);
-                if (!wait_bounded(&bars->acc_full[ab], (uint32_t)((si / NACC) & 1), abort)) {
-                    ok = false;
-                    break;
-                }
-                tc::tc_fence_after();
-                // class k of this line: columns 32 k + 16 ln + (h, rhs)
-                const uint32_t tbase = tmem + ACCB * ab + 16 * ln + ((uint32_t)(32 * quad) << 16);
+        const Tiles tl(a);
+        Place pl(tl, first);
+        for (int left = (int)count; left > 0 && ok;) {
+            const int64_t per = tl.tile_slots(pl.g);
+            const int nsl = (int)(per - pl.off < left ? per - pl.off : left);
 #pragma unroll
-                for (int k = 0; k < KD; ++k) {
-                    float v[16];
-                    tc::tmem_ld16(tbase + 32 * k, v);
+            for (int e = 0; e < 8; ++e)
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        if (k == 0) s0[e % 8] += (long long)__float2int_rn(v[e]);
-                        else sk[k - 1][e % 8] += __float2int_rn(v[e]);
+                for (int g = 0; g < NGRP; ++g) S[e][g] = 0;
+            for (int s = 0; s < nsl && ok; ++s) {
+#pragma unroll 1                                // (unrolled, the sums spill)
+                for (int h = 0; h < NACC; ++h) {
+                    // (a warp gives up as one: the TMEM loads below are collective)
+                    if (!__all_sync(0xffffffffu, wait_bounded(&bars->acc_full[h], ph, abort))) {
+                        ok = false;
+                        break;
                     }
+                    tc::tc_fence_after();
+                    const uint32_t tbase = tmem + ACCB * h + 8 * cg + ((uint32_t)(32 * quad) << 16);
+#pragma unroll
+                    for (int k = 0; k < KD; k += 2) {
+                        float v[2][8];
+                        if (k + 1 < KD) tc::tmem_ld8x2(tbase + NCOL * k, tbase + NCOL * (k + 1), v[0], v[1]);
+                        else tc::tmem_ld8(tbase + NCOL * k, v[0]);
+#pragma unroll
+                        for (int u = 0; u < 2; ++u)
+                            if (k + u < KD) {
+                                const int g = (k + u) / 4, sh = 8 * (3 - (k + u) % 4);
+#pragma unroll
+                                for (int e = 0; e < 8; ++e)
+                                    S[e][g] += (long long)__float2int_rn(v[u][e]) * (1 << sh);
+                            }
+                    }
+                    tc::tc_fence_before();
+                    tc::mbar_arrive(&bars->acc_empty[h]);
                 }
-                tc::tc_fence_before();
-                tc::mbar_arrive(&bars->acc_empty[ab]);
-                if (g % CARRY == CARRY - 1) carry();
+                ph ^= 1;
+                if (s % CARRY == CARRY - 1 || s == nsl - 1) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) carry(S[e]);
+                }
             }
             if (!ok) break;
-            carry();
-            const int il = TM * w.b + TM - 1 - (32 * quad + lane);
-            const int64_t L = w.line(ln);
-            if (il < a.n && L >= 0) {
-                const int64_t gpos = L * a.n + il;
+            if (nsl == per) {
+                const int eT = scale_exp(*a.tmax);
 #pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    if (r < a.nr) {
-                        double y = 0.0, wt = ldexp(1.0, -8 * (KD - 1));
-#pragma unroll
-                        for (int k = KD - 1; k >= 1; --k, wt *= 256.0) y += (double)sk[k - 1][r] * wt;
-                        y += (double)s0[r];
-                        a.ybuf[gpos + a.N * (a.r0 + r)] = ldexp(y, eT + scale_exp(a.xmax[r]) - 16);
-                    }
+                for (int e = 0; e < 8; ++e) {
+                    const int col = 8 * cg + e, r = col & ((1 << a.lg) - 1);
+                    store_row(a, pl.g * tl.NL, pl.q / tl.nc, pl.q % tl.nc, row, col,
+                              from_sums(S[e], eT + scale_exp(a.xmax[r]) + a.xshift));
                 }
-            }
+            } else {
+                // a tile begun by an earlier CTA (0) or left to the next one (1)
+                long long* part = a.part + (int64_t)(2 * blockIdx.x + (pl.off == 0 ? 1 : 0)) * PART;
 #pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                s0[r] = 0;
+                for (int g = 0; g < NG; ++g)
 #pragma unroll
-                for (int k = 0; k < KD - 1; ++k) sk[k][r] = 0;
+                    for (int e = 0; e < 8; ++e) part[(g * 8 + e) * NEPI + threadIdx.x] = S[e][g];
             }
+            left -= nsl;
+            pl.next_tile(tl);
         }
     }
     tc::tc_fence_before();
@@ -601,6 +643,35 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
         tc::tc_fence_after();
         tc::tmem_dealloc(tmem, ACC);
     }
+}
+
+// The tiles cut by range boundaries: block x adds up the partial class sums
+// of the tile in which CTA x + 1 starts, if CTA x is the one that began it.
+__global__ void __launch_bounds__(256) tc_fixup_kernel(TcConvArgs a, int ctas, int ng) {
+    const Tiles t(a);
+    const int cta = blockIdx.x + 1;
+    const int64_t start = range_start(a, cta, ctas);
+    const Place p(t, start);
+    if (p.off == 0 || start - p.off < range_start(a, cta - 1, ctas)) return;
+    const int64_t end = start - p.off + t.tile_slots(p.g);
+    const int eT = scale_exp(*a.tmax);
+    int last = cta;
+    while (last < ctas && range_start(a, last, ctas) < end) ++last;
+    const int e = blockIdx.y * blockDim.x + threadIdx.x;       // (column of 8, epilogue thread)
+    long long S[NGRP] = {0, 0};
+#pragma unroll
+    for (int g = 0; g < NGRP; ++g) {
+        if (g >= ng) continue;
+        const long long* src = a.part + (int64_t)g * 8 * NEPI + e;
+        long long s = src[(int64_t)(2 * (cta - 1) + 1) * PART];
+#pragma unroll 8
+        for (int q = cta; q < last; ++q) s += src[(int64_t)(2 * q) * PART];
+        S[g] = s;
+    }
+    carry(S);
+    const int th = e % NEPI, col = 8 * (th >> 7) + e / NEPI, r = col & ((1 << a.lg) - 1);
+    store_row(a, p.g * t.NL, p.q / t.nc, p.q % t.nc, th & 127, col,
+              from_sums(S, eT + scale_exp(a.xmax[r]) + a.xshift));
 }
 
 // ---- host side ----------------------------------------------------------------
@@ -641,10 +712,11 @@ size_t tc_table_rows_bytes(int n, int dim) {
     return sizeof(__nv_bfloat16) * (size_t)ST * lines * 256 * nc;
 }
 
-size_t tc_source_digits_bytes(int n, int dim) {
+size_t tc_source_digits_bytes(int n, int dim, int num_sms) {
     const int nc = (n + KC - 1) / KC;
     const int64_t lines = dim == 2 ? (int64_t)n : (int64_t)n * n;
-    return (size_t)(lines * nc + 1) * CHUNK;                 // + one zero chunk
+    // + two partial tiles per CTA of the launch
+    return (size_t)(lines * nc) * CHUNK + (size_t)2 * std::max(num_sms, 1) * PART * sizeof(long long);
 }
 
 cudaError_t launch_tc_table(const double* table, int n, int dim, unsigned long long* tmax, void* R,
@@ -687,7 +759,7 @@ cudaError_t launch_direct_grid_tc(const GridDirectArgs& a, const void* R, const 
     const int64_t N = a.dim == 2 ? (int64_t)a.n * a.n : (int64_t)a.n * a.n * a.n;
     if (N == 0) return cudaSuccess;
     if (classes < 4 || classes == 7 || classes > 8) return cudaErrorInvalidValue;
-    const int nc = (a.n + KC - 1) / KC, nb = (a.n + TM - 1) / TM;
+    const int nc = (a.n + KC - 1) / KC;
     const int64_t lines = a.dim == 2 ? (int64_t)a.n : (int64_t)a.n * a.n;
     const int eb = (int)std::min<int64_t>((N * a.nrhs + 255) / 256, 152 * 16);
     void (*kfn)(TcConvArgs) = nullptr;
@@ -700,10 +772,10 @@ cudaError_t launch_direct_grid_tc(const GridDirectArgs& a, const void* R, const 
         if (e != cudaSuccess) return e;
     }
     grid_scatter_kernel_launch(a, N, eb, st);
-    {
-        cudaError_t e = cudaMemsetAsync((unsigned char*)XB + lines * nc * (int64_t)CHUNK, 0, CHUNK, st);
-        if (e != cudaSuccess) return e;
-    }
+    // the 64-bit class sums hold N 2^38 for N <= 2^24; larger sums start from
+    // smaller top digits
+    int xshift = 0;
+    while ((N >> xshift) > ((int64_t)1 << 24)) ++xshift;
     for (int r0 = 0; r0 < a.nrhs; r0 += NR) {
         const int nr = std::min(NR, a.nrhs - r0);
         cudaError_t e = cudaMemsetAsync(xmax, 0, NR * sizeof(unsigned long long), st);
@@ -711,10 +783,13 @@ cudaError_t launch_direct_grid_tc(const GridDirectArgs& a, const void* R, const 
         note_launch();
         tc_maxabs_kernel<<<(int)std::min<int64_t>((N + 255) / 256, 1024), 256, 0, st>>>(a.vbuf + N * r0, N, nr, N,
                                                                                        xmax);
-        const int64_t items = lines * nc * (KC / 8) * NR;
+        // right-hand sides of this launch, rounded up to a power of two; the
+        // rest of the 32 columns per class are target lines
+        const int lg = nr > 4 ? 3 : nr > 2 ? 2 : nr > 1 ? 1 : 0;
+        const int64_t items = (lines * nc * (KC / 8)) << lg;
         note_launch();
         tc_source_digits_kernel<<<(int)std::min<int64_t>((items + 255) / 256, 152 * 16), 256, 0, st>>>(
-            a.vbuf, N, a.n, lines, nc, r0, nr, classes, xmax, (uint4*)XB);
+            a.vbuf, N, a.n, lines, nc, r0, nr, lg, classes, xshift, xmax, (uint4*)XB);
         TcConvArgs t{};
         t.R = (const __nv_bfloat16*)R;
         t.XB = (const unsigned char*)XB;
@@ -725,9 +800,11 @@ cudaError_t launch_direct_grid_tc(const GridDirectArgs& a, const void* R, const 
         t.n = a.n;
         t.lines = lines;
         t.dim = a.dim;
-        t.nb = nb;
         t.nc = nc;
-        t.tiles = (a.dim == 2 ? (int64_t)((a.n + 1) / 2) : (int64_t)((a.n + 1) / 2) * a.n) * nb;
+        t.lg = lg;
+        t.part = (long long*)((unsigned char*)XB + lines * nc * (int64_t)CHUNK);
+        t.slots = total_slots(t);
+        t.xshift = xshift;
         t.r0 = r0;
         t.nr = nr;
         t.status = status;
@@ -738,7 +815,7 @@ cudaError_t launch_direct_grid_tc(const GridDirectArgs& a, const void* R, const 
             const char* e = getenv("HIF_TC_TEST_STALL");
             t.stall = (e && atoi(e) != 0) ? 1 : 0;
         }
-        const int grid = (int)std::min<int64_t>(t.tiles, num_sms);
+        const int grid = (int)std::min<int64_t>(t.slots, num_sms);
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         {
             std::lock_guard<std::mutex> lk(g_tm_mu);
@@ -752,6 +829,10 @@ cudaError_t launch_direct_grid_tc(const GridDirectArgs& a, const void* R, const 
         }
         note_launch();
         kfn<<<grid, NTHR, smem, st>>>(t);
+        if (grid > 1) {
+            note_launch();
+            tc_fixup_kernel<<<dim3(grid - 1, 8 * NEPI / 256), 256, 0, st>>>(t, grid, (classes + 3) / 4);
+        }
         if (e1) cudaEventRecord(e1, st);
     }
     grid_finish_kernel_launch(a, N, eb, st);

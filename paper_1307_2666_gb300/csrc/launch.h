@@ -315,7 +315,7 @@ void grid_finish_kernel_launch(const GridDirectArgs&, int64_t N, int eb, cudaStr
 // launch_tc_table with tmax its max |entry|; XB = tc_source_digits_bytes of
 // scratch, xmax 8 entries, status one int (set to 1 if a wait expired)
 size_t tc_table_rows_bytes(int n, int dim);
-size_t tc_source_digits_bytes(int n, int dim);
+size_t tc_source_digits_bytes(int n, int dim, int num_sms);
 cudaError_t launch_tc_table(const double* table, int n, int dim, unsigned long long* tmax, void* R,
                             cudaStream_t);
 // CUDA-event timing of tc_conv_kernel launches (see hif_kernel_timing)
