@@ -70,12 +70,9 @@ typedef struct {
                                other point sets always use FP64                          */
     int use_graphs;         /* capture the sweeps of each (operation, nrhs) in a CUDA graph
                                and replay it (default 1)                                   */
-    int autotune;           /* time the candidate CTA sizes of every sublevel's sweep after
-                               the factorization and keep the fastest (the sweep's
-                               arithmetic does not depend on it); in FP32 factorizations
-                               also time 16 and 32 rows per fold chunk for every box-width
-                               bucket on its first sighting in the process and keep the
-                               faster (default 1)                                         */
+    int autotune;           /* in FP32 factorizations time 16 and 32 rows per fold chunk for
+                               every box-width bucket on its first sighting in the process
+                               and keep the faster (default 1)                            */
     int symmetric;          /* 1 (default): when b == c and all weights are equal, A is
                                symmetric and the one-sided proxy matrix Y'_c = [A_{cN,c};
                                Y_{cE,c}] is compressed (Sec. 5; same ID, half the rows);
@@ -115,8 +112,8 @@ typedef struct {
 /* Defaults for dimension dim (2 or 3): occupancy 64, second_kind 1, FP64,
  * fractional levels on, proxy 64 points (2D) / 512 (3D) at radius 1.5,
  * fp32_tol_floor 2^-17, bounding-cube root box, default stream, direct sums
- * on the tensor cores (direct_precision 2), graph-replayed and autotuned
- * sweeps, symmetric shortcut and LDL on. */
+ * on the tensor cores (direct_precision 2), graph-replayed sweeps, autotuned
+ * fold chunks, symmetric shortcut and LDL on. */
 hif_status hif_options_default(int dim, hif_options* opt);
 
 /*

@@ -52,7 +52,7 @@ class Factorization:
     direct: direct sum on uniform grids, "tc" (tensor cores on exact 8-bit
     digits), "df64" (paired FP32) or "fp64".
     graphs: replay the factored-form sweeps from captured CUDA graphs.
-    autotune: pick each sublevel's sweep CTA size by timing after factoring.
+    autotune: pick the rows per fold chunk of FP32 factorizations by timing.
     kernel_id 2: the Helmholtz kernel (i/4) H_0^(1)(k r) of Sec. 5, Example 3,
     with ``wavenumber`` k; a, b, c stay real, vectors are complex (complex128
     tensors), and the library works on the real 2 x 2 embedding of the

@@ -141,13 +141,13 @@ struct SubFactor {
     std::vector<BoxFac> hbox;
     DevMem boxes, sk, rd, pool, perm;
     int max_kr2 = 0;               // max over boxes of k + 2 r
-    // sweep plan: boxes whose vectors exceed shared memory use a global work
-    // space (offsets per right-hand side); the CTA size is tuned per sublevel
+    // sweep plan: CTAs per box and CTA size; boxes whose vectors exceed shared
+    // memory use a global work space (offsets per right-hand side)
     bool global = false;
     DevMem gws_off;
     int64_t gws_units = 0;
-    int threads = 256;
-    // boxes of the one-CTA sweep kernel (sboxes) and the wide boxes whose
+    int threads = 256, cluster = 1;
+    // boxes of the cluster sweep kernel (sboxes) and the wide boxes whose
     // passes run as stage launches over the whole GPU (wboxes, work space at
     // wws_off per box in units of k + 2 r, per right-hand side)
     DevMem sboxes, wboxes, wws_off;
@@ -1361,11 +1361,17 @@ static void run_factor(hif_handle h) {
 enum { SOLVE_UP = 0, SOLVE_DOWN = 1, APPLY_UP = 2, APPLY_DOWN = 3,
        SOLVET_UP = 4, SOLVET_DOWN = 5, APPLYT_UP = 6, APPLYT_DOWN = 7 };
 
-// One sublevel in one direction for all right-hand sides (CTA size: the
-// sublevel's tuned value unless threads > 0).
+// Right-hand sides a sweep CTA holds: the power of two that covers nrhs, at
+// most 8, halved until the sublevel's largest box fits into shared memory.
+static int sweep_nc(const SubFactor& sf, int nrhs, size_t elem) {
+    int nc = nrhs > 4 ? 8 : nrhs > 2 ? 4 : nrhs;
+    while (nc > 1 && !sf.global && sweep_smem_bytes(sf.max_kr2_small, nc, sf.threads, (int)elem) > kSweepSmemMax) nc /= 2;
+    return nc;
+}
+
+// One sublevel in one direction for all right-hand sides.
 template <typename T>
-static void sweep_one(hif_handle h, SubFactor& sf, int mode, T* xw, int64_t ldx, int nrhs, int threads,
-                      cudaStream_t st) {
+static void sweep_one(hif_handle h, SubFactor& sf, int mode, T* xw, int nrhs, cudaStream_t st) {
     if (!sf.nbox) return;
     for (int r0 = 0; sf.nwide && r0 < nrhs; r0 += 16) {
         WideArgs w{};
@@ -1374,47 +1380,44 @@ static void sweep_one(hif_handle h, SubFactor& sf, int mode, T* xw, int64_t ldx,
         w.rd_ids = sf.rd.as<int>();
         w.pool = sf.pool.p;
         w.perm = sf.perm.as<int>();
-        w.x = xw + ldx * r0;
-        w.ldx = ldx;
+        w.x = xw + r0;
+        w.ldx = nrhs;
         w.nr = std::min(16, nrhs - r0);
         w.ws = h->sweep_ws.p;
         w.ws_off = sf.wws_off.as<int64_t>();
         HIF_CUDA((launch_wide_sweep<T>(w, sf.nwide, sf.wmax_k, sf.wmax_r, mode, st)));
     }
     if (!sf.nsmall) return;
-    const size_t per_col = (size_t)sf.max_kr2_small * sizeof(T);
-    const int batch = sf.global ? nrhs : (int)std::min<size_t>((size_t)nrhs, std::max<size_t>(1, (200 * 1024) / per_col));
-    for (int r0 = 0; r0 < nrhs; r0 += batch) {
-        const int nr = std::min(batch, nrhs - r0);
-        SweepArgs a{};
-        a.boxes = sf.sboxes.as<BoxFac>();
-        a.sk_ids = sf.sk.as<int>();
-        a.rd_ids = sf.rd.as<int>();
-        a.pool = sf.pool.p;
-        a.perm = sf.perm.as<int>();
-        a.x = xw + ldx * r0;
-        a.ldx = ldx;
-        a.nrhs = nr;
-        const size_t smem = sf.global ? 0 : per_col * nr + 64;
-        a.mode = mode | (int)(smem << 8);
-        a.gws = sf.global ? h->sweep_ws.p : nullptr;
-        a.gws_off = sf.global ? sf.gws_off.as<int64_t>() : nullptr;
-        HIF_CUDA((launch_sweep<T>(a, sf.nsmall, threads > 0 ? threads : sf.threads, st)));
-    }
+    const int nc = sweep_nc(sf, nrhs, sizeof(T));
+    SweepArgs a{};
+    a.boxes = sf.sboxes.as<BoxFac>();
+    a.sk_ids = sf.sk.as<int>();
+    a.rd_ids = sf.rd.as<int>();
+    a.pool = sf.pool.p;
+    a.perm = sf.perm.as<int>();
+    a.x = xw;
+    a.ldx = nrhs;
+    a.nrhs = nrhs;
+    a.mode = mode;
+    a.cluster = sf.cluster;
+    a.gws = sf.global ? h->sweep_ws.p : nullptr;
+    a.gws_off = sf.global ? sf.gws_off.as<int64_t>() : nullptr;
+    const size_t smem = sweep_smem_bytes(sf.global ? 0 : sf.max_kr2_small, nc, sf.threads, sizeof(T));
+    HIF_CUDA((launch_sweep<T>(a, sf.nsmall, nc, sf.threads, smem, st)));
 }
 
 template <typename T>
-static void sweep_seq(hif_handle h, T* xw, int64_t ldx, int nrhs, int op, cudaStream_t st) {
+static void sweep_seq(hif_handle h, T* xw, int nrhs, int op, cudaStream_t st) {
     // op: 0 solve, 1 apply, 2 solve^T, 3 apply^T
     const int up = op == 0 ? SOLVE_UP : op == 1 ? APPLY_UP : op == 2 ? SOLVET_UP : APPLYT_UP;
-    for (auto& sf : h->subs) sweep_one<T>(h, *sf, up, xw, ldx, nrhs, 0, st);
-    for (auto it = h->subs.rbegin(); it != h->subs.rend(); ++it) sweep_one<T>(h, **it, up + 1, xw, ldx, nrhs, 0, st);
+    for (auto& sf : h->subs) sweep_one<T>(h, *sf, up, xw, nrhs, st);
+    for (auto it = h->subs.rbegin(); it != h->subs.rend(); ++it) sweep_one<T>(h, **it, up + 1, xw, nrhs, st);
 }
 
 static void ensure_sweep_ws(hif_handle h, int nrhs, size_t elem) {
     int64_t need = 1;
     for (auto& sf : h->subs)
-        need = std::max({need, sf->gws_units * std::max(nrhs, 1), sf->wws_units * std::min(std::max(nrhs, 1), 16)});
+        need = std::max({need, sf->gws_units * (std::max(nrhs, 1) + 7), sf->wws_units * std::min(std::max(nrhs, 1), 16)});
     h->sweep_ws.ensure(elem * (size_t)need);
 }
 
@@ -1422,7 +1425,7 @@ static void ensure_sweep_ws(hif_handle h, int nrhs, size_t elem) {
 // (operation, nrhs, work buffer) is captured once into a CUDA graph on the
 // handle's capture stream and replayed on the handle's stream.
 template <typename T>
-static void sweep_all(hif_handle h, T* xw, int64_t ldx, int nrhs, int op) {
+static void sweep_all(hif_handle h, T* xw, int nrhs, int op) {
     ensure_sweep_ws(h, nrhs, sizeof(T));
     double sweep_bytes = 0.0;
     if (prof_enabled())
@@ -1430,8 +1433,8 @@ static void sweep_all(hif_handle h, T* xw, int64_t ldx, int nrhs, int op) {
             sweep_bytes += sizeof(T) * (sf->sweep_factor_elems + 4.0 * sf->sweep_vec_elems * nrhs) +
                            sizeof(int) * sf->sweep_perm_ints;
     ProfRange pr(PROF_SWEEP, h->st, 0.0, sweep_bytes);
-    if (!h->opt.use_graphs || ldx != h->N) {
-        sweep_seq<T>(h, xw, ldx, nrhs, op, h->st);
+    if (!h->opt.use_graphs) {
+        sweep_seq<T>(h, xw, nrhs, op, h->st);
         return;
     }
     SweepGraph* g = nullptr;
@@ -1443,7 +1446,7 @@ static void sweep_all(hif_handle h, T* xw, int64_t ldx, int nrhs, int op) {
         HIF_CUDA(cudaStreamBeginCapture(h->cap_st, cudaStreamCaptureModeThreadLocal));
         cudaGraph_t graph = nullptr;
         try {
-            sweep_seq<T>(h, xw, ldx, nrhs, op, h->cap_st);
+            sweep_seq<T>(h, xw, nrhs, op, h->cap_st);
         } catch (...) {
             cudaStreamEndCapture(h->cap_st, &graph);
             if (graph) cudaGraphDestroy(graph);
@@ -1468,9 +1471,8 @@ static void sweep_all(hif_handle h, T* xw, int64_t ldx, int nrhs, int op) {
     g_launches.fetch_add(g->kernels);
 }
 
-// After the factorization: the global work-space offsets of every sublevel,
-// and (with autotune) the CTA size of each sublevel's sweep, picked by timing
-// one solve sweep per candidate on the work vector.
+// After the factorization: the launch shape and the global work-space offsets
+// of every sublevel's sweep.
 template <typename T>
 static void prepare_sweeps(hif_handle h) {
     const cudaStream_t st = h->st;
@@ -1483,12 +1485,16 @@ static void prepare_sweeps(hif_handle h) {
             sf.sweep_perm_ints += r;
             sf.sweep_vec_elems += k + r;
         }
-        // wide LU boxes take the stage path (HIF_SWEEP_WIDE: the k + r above
-        // which a box is wide)
-        const int wide_min = env_int("HIF_SWEEP_WIDE", 768);
+        // LU boxes above 8,192 rows take the stage path over the whole GPU
+        // (HIF_SWEEP_WIDE: another line).  The cluster kernel was the faster
+        // of the two at every width measured: 64-bit n = 200, boxes of up to
+        // 1,153 rows, 3.8 ms with every box above 768 rows on the stage path
+        // and 1.6 ms with none; 3D n = 32, up to 1,968 rows, 5.2 and 1.7 ms.
+        const int wide_min = env_int("HIF_SWEEP_WIDE", 8192);
         std::vector<BoxFac> sb, wb;
         std::vector<int64_t> woffs;
         sf.wmax_k = sf.wmax_r = sf.max_kr2_small = 0;
+        int max_kr = 0;
         sf.wws_units = 0;
         for (const BoxFac& bf : sf.hbox) {
             if (!bf.ldl && bf.k + bf.r > wide_min) {
@@ -1500,6 +1506,7 @@ static void prepare_sweeps(hif_handle h) {
             } else {
                 sb.push_back(bf);
                 sf.max_kr2_small = std::max(sf.max_kr2_small, bf.k + 2 * bf.r);
+                max_kr = std::max(max_kr, bf.k + bf.r);
             }
         }
         sf.nsmall = (int)sb.size();
@@ -1507,7 +1514,18 @@ static void prepare_sweeps(hif_handle h) {
         upload(sf.sboxes, sb, st);
         upload(sf.wboxes, wb, st);
         upload(sf.wws_off, woffs, st);
-        sf.global = (size_t)sf.max_kr2_small * sizeof(T) > 200 * 1024;
+        // CTAs per box: until the sublevel has eight per SM, while each keeps
+        // 64 of the box's rows
+        sf.cluster = 1;
+        while (sf.cluster < 8 && 2 * sf.cluster * sf.nsmall <= 8 * h->num_sms && max_kr > 64 * sf.cluster) sf.cluster *= 2;
+        // (512 threads with 16 loads in flight each: wide boxes that have their
+        // SMs to themselves.  n = 512, one 64-bit right-hand side: 16 boxes of
+        // ~1,050 rows 137 -> 80 us, but 64 boxes of ~770 rows 112 -> 158 us)
+        sf.threads = max_kr <= 96                                                               ? 128
+                     : sf.cluster == 8 && max_kr > 512 && sf.cluster * sf.nsmall <= h->num_sms ? 512
+                                                                                                : 256;
+        sf.global = sweep_smem_bytes(sf.max_kr2_small, 1, sf.threads, sizeof(T)) > kSweepSmemMax;
+        if (sf.global) sf.cluster = 1;
         sf.gws_units = 0;
         if (!sf.global || !sf.nsmall) continue;
         std::vector<int64_t> offs(sb.size());
@@ -1519,37 +1537,6 @@ static void prepare_sweeps(hif_handle h) {
         upload(sf.gws_off, offs, st);
         sf.gws_units = tot;
     }
-    if (!h->opt.autotune) return;
-    const int64_t N = h->N;
-    h->work.ensure(sizeof(T) * N);
-    T* xw = h->work.as<T>();
-    HIF_CUDA(cudaMemsetAsync(xw, 0, sizeof(T) * N, st));
-    ensure_sweep_ws(h, 1, sizeof(T));
-    cudaEvent_t e0, e1;
-    HIF_CUDA(cudaEventCreate(&e0));
-    HIF_CUDA(cudaEventCreate(&e1));
-    const int cand[3] = {128, 256, 512};
-    for (auto& sp : h->subs) {
-        SubFactor& sf = *sp;
-        if (!sf.nsmall) continue;
-        float best = 1e30f;
-        for (int c : cand) {
-            float t = 0.f;
-            for (int rep = 0; rep < 2; ++rep) {           // the first run warms the factor data
-                HIF_CUDA(cudaEventRecord(e0, st));
-                sweep_one<T>(h, sf, SOLVE_UP, xw, N, 1, c, st);
-                HIF_CUDA(cudaEventRecord(e1, st));
-                HIF_CUDA(cudaEventSynchronize(e1));
-                HIF_CUDA(cudaEventElapsedTime(&t, e0, e1));
-            }
-            if (t < best) {
-                best = t;
-                sf.threads = c;
-            }
-        }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
 }
 
 static void apply_op(hif_handle h, const double* in, double* out, int64_t nrhs, int64_t ld, int op) {
@@ -1579,15 +1566,15 @@ static void apply_op(hif_handle h, const double* in, double* out, int64_t nrhs, 
     if (h->precision == 0) {
         h->work.ensure(sizeof(double) * N * nrhs);
         double* xw = h->work.as<double>();
-        HIF_CUDA(launch_to_work<double>(din_p, ldi, xw, N, N, (int)nrhs, st));
-        sweep_all<double>(h, xw, N, (int)nrhs, op);
-        HIF_CUDA(launch_from_work<double>(xw, N, dout_p, ldo, N, (int)nrhs, st));
+        HIF_CUDA(launch_to_work<double>(din_p, ldi, xw, N, (int)nrhs, st));
+        sweep_all<double>(h, xw, (int)nrhs, op);
+        HIF_CUDA(launch_from_work<double>(xw, dout_p, ldo, N, (int)nrhs, st));
     } else {
         h->work.ensure(sizeof(float) * N * nrhs);
         float* xw = h->work.as<float>();
-        HIF_CUDA(launch_to_work<float>(din_p, ldi, xw, N, N, (int)nrhs, st));
-        sweep_all<float>(h, xw, N, (int)nrhs, op);
-        HIF_CUDA(launch_from_work<float>(xw, N, dout_p, ldo, N, (int)nrhs, st));
+        HIF_CUDA(launch_to_work<float>(din_p, ldi, xw, N, (int)nrhs, st));
+        sweep_all<float>(h, xw, (int)nrhs, op);
+        HIF_CUDA(launch_from_work<float>(xw, dout_p, ldo, N, (int)nrhs, st));
     }
     if (!dout)
         HIF_CUDA(cudaMemcpy2DAsync(out, sizeof(double) * ld, dout_p, sizeof(double) * N, sizeof(double) * N, nrhs,
@@ -1679,15 +1666,15 @@ static void fac_dev(hif_handle h, int op, const double* b, double* x, int nrhs) 
     if (h->precision == 0) {
         h->work.ensure(sizeof(double) * N * nrhs);
         double* xw = h->work.as<double>();
-        HIF_CUDA(launch_to_work<double>(b, N, xw, N, N, nrhs, st));
-        sweep_all<double>(h, xw, N, nrhs, op);
-        HIF_CUDA(launch_from_work<double>(xw, N, x, N, N, nrhs, st));
+        HIF_CUDA(launch_to_work<double>(b, N, xw, N, nrhs, st));
+        sweep_all<double>(h, xw, nrhs, op);
+        HIF_CUDA(launch_from_work<double>(xw, x, N, N, nrhs, st));
     } else {
         h->work.ensure(sizeof(float) * N * nrhs);
         float* xw = h->work.as<float>();
-        HIF_CUDA(launch_to_work<float>(b, N, xw, N, N, nrhs, st));
-        sweep_all<float>(h, xw, N, nrhs, op);
-        HIF_CUDA(launch_from_work<float>(xw, N, x, N, N, nrhs, st));
+        HIF_CUDA(launch_to_work<float>(b, N, xw, N, nrhs, st));
+        sweep_all<float>(h, xw, nrhs, op);
+        HIF_CUDA(launch_from_work<float>(xw, x, N, N, nrhs, st));
     }
 }
 

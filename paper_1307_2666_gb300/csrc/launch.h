@@ -74,12 +74,13 @@ struct SweepArgs {
     const int* rd_ids;
     const void* pool;
     const int* perm;
-    void* x;                // working vectors, N x nrhs column-major (factor precision)
+    void* x;                // working vectors, ldx apart per DOF, right-hand sides adjacent (factor precision)
     int64_t ldx;
     int nrhs;
     int mode;               // see k_sweep.cu
-    void* gws;              // non-null: per-box vectors in global memory at gws_off[box] * nrhs
-    const int64_t* gws_off; // (boxes too large for shared memory); offsets per right-hand side
+    int cluster;            // CTAs per box (1, 2, 4, 8)
+    void* gws;              // non-null: per-box vectors in global memory at gws_off[box] * nrhs (rounded up
+    const int64_t* gws_off; // to the launch's nc; boxes too large for shared memory, one CTA each)
 };
 
 // ---- large boxes: unpivoted blocked QR to the n x n factor R (k_bigqr.cu)
@@ -223,9 +224,13 @@ template <typename T> cudaError_t launch_id(const IdArgs&, int ngroups, size_t s
 template <typename T> cudaError_t launch_elim(const ElimArgs&, int nbox, int num_sms, cudaStream_t);
 
 // sweeps
-// threads: CTA size, a multiple of 32 up to 512 (the sweep's arithmetic does
-// not depend on it)
-template <typename T> cudaError_t launch_sweep(const SweepArgs&, int nbox, int threads, cudaStream_t);
+// nc: right-hand sides held per CTA (1, 2, 4, 8); threads: CTA size, a
+// multiple of 32 up to 512; smem: sweep_smem_bytes of the largest k + 2 r
+// (0 units of k + 2 r with gws)
+constexpr size_t kSweepSmemMax = 224 * 1024;
+size_t sweep_smem_bytes(int k2r, int nc, int threads, int elem);
+template <typename T>
+cudaError_t launch_sweep(const SweepArgs&, int nbox, int nc, int threads, size_t smem, cudaStream_t);
 
 // Wide boxes of a sublevel: the pass as stage launches over (box, row tile).
 // ws holds per box (k + 2 r) x nr values from ws_off[box] * nr; nr <= 16.
@@ -245,10 +250,10 @@ template <typename T>
 cudaError_t launch_wide_sweep(const WideArgs&, int nwide, int max_k, int max_r, int mode, cudaStream_t);
 
 // vectors and direct sums (FP64 inputs)
-template <typename T> cudaError_t launch_to_work(const double* src, int64_t lds, T* dst, int64_t ldd,
-                                                 int64_t N, int nrhs, cudaStream_t);
-template <typename T> cudaError_t launch_from_work(const T* src, int64_t lds, double* dst, int64_t ldd,
-                                                   int64_t N, int nrhs, cudaStream_t);
+template <typename T> cudaError_t launch_to_work(const double* src, int64_t lds, T* dst, int64_t N, int nrhs,
+                                                 cudaStream_t);
+template <typename T> cudaError_t launch_from_work(const T* src, double* dst, int64_t ldd, int64_t N, int nrhs,
+                                                   cudaStream_t);
 
 struct DirectArgs {
     GeomDev g;
