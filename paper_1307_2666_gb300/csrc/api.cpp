@@ -130,7 +130,7 @@ struct Segment {
 };
 
 struct FactorScratch {
-    DevMem d_ed, d_ed_big, d_eg, ews, piv, ldl_fail, gemm_probs, elim_order, elim_next;
+    DevMem d_ed, d_ed_big, d_eg, ews, piv, ldl_fail, gemm_probs, elim_order, elim_next, elim_fail_idx;
 };
 
 constexpr int KIND_TOP = 3;   // the top blocks, eliminated as boxes without skeletons
@@ -552,57 +552,89 @@ static void launch_elims(hif_handle h, SubFactor& sf, const std::vector<ElimDesc
     // the LU fallback of LDL boxes can be exercised on any problem
     ea.ldl_alpha = (1.0 + std::sqrt(17.0)) / 8.0;
     if (const char* v = std::getenv("HIF_LDL_TEST_ALPHA")) ea.ldl_alpha = std::atof(v);
-    // work list of the persistent launch: boxes by (k + r)^3 descending
-    {
-        std::vector<int> order(ed.size());
-        for (size_t q = 0; q < ed.size(); ++q) order[q] = (int)q;
+    // Boxes above mid_n take the batched multi-CTA stages with the large ones
+    // (LDL kept), the others one CTA each.  Batched, n = 64 (64-bit, 4 boxes of
+    // 348, a top block of 388) went from 89 to 12 ms of elimination, 24
+    // problems of n <= 256 (32-bit) from 134 to 27 ms; between 40 and 160 the
+    // line moves the totals by less than 2%.
+    const bool tc_gemm = env_int("HIF_TC_GEMM", 0) != 0;
+    const int mid_n = tc_gemm ? 1 << 30 : env_int("HIF_ELIM_MID", 96);
+    const int be_max_r = be_factor_max_r<T>();
+    std::vector<ElimDesc> batch;
+    std::vector<int> fail_idx, order;
+    double work_batch = work[1], work_cta = work[0];
+    for (size_t q = 0; q < ed.size(); ++q) {
+        if (ed[q].k + ed[q].r > mid_n && ed[q].r <= be_max_r) {
+            batch.push_back(ed[q]);
+            fail_idx.push_back((int)q);
+            const double kk = ed[q].k, rr = ed[q].r;
+            const double w = 6.0 * (kk * kk * rr + kk * rr * rr) + 2.0 / 3.0 * rr * rr * rr;
+            work_batch += w;
+            work_cta -= w;
+        } else {
+            order.push_back((int)q);
+        }
+    }
+    for (const ElimDesc& e : ed_big) {
+        batch.push_back(e);
+        fail_idx.push_back(-1);
+    }
+    if (!order.empty()) {
+        // work list of the persistent launch: boxes by (k + r)^3 descending
         std::stable_sort(order.begin(), order.end(), [&](int u, int v) {
             return ed[u].k + ed[u].r > ed[v].k + ed[v].r;
         });
         upload(S.elim_order, order, st);
         S.elim_next.ensure(sizeof(int));
         ea.order = S.elim_order.as<int>();
-        ea.nitems = (int)ed.size();
+        ea.nitems = (int)order.size();
         ea.next_item = S.elim_next.as<int>();
+        ProfRange pr(PROF_ELIM, st, std::max(work_cta, 0.0), 0.0);
+        HIF_CUDA((launch_elim<T>(ea, (int)order.size(), h->num_sms, st)));
     }
-    {
-        ProfRange pr(PROF_ELIM, st, work[0], 0.0);
-        HIF_CUDA((launch_elim<T>(ea, (int)ed.size(), h->num_sms, st)));
-    }
-    if (!ed_big.empty()) {
-        upload(S.d_ed_big, ed_big, st);
-        int mxn = 0, mxk = 0, mxr = 0;
-        for (const ElimDesc& eb : ed_big) {
-            mxn = std::max(mxn, eb.k + eb.r);
-            mxk = std::max(mxk, eb.k);
-            mxr = std::max(mxr, eb.r);
+    if (!batch.empty()) {
+        upload(S.d_ed_big, batch, st);
+        upload(S.elim_fail_idx, fail_idx, st);
+        if (tc_gemm) S.gemm_probs.ensure(sizeof(TcGemmProb) * 5 * batch.size());
+        ProfRange pr(PROF_BIG_ELIM, st, work_batch, 0.0);
+        constexpr size_t kGridMax = 65535;          // boxes per launch (grid y and z)
+        for (size_t q0 = 0; q0 < batch.size(); q0 += kGridMax) {
+            BatchElimArgs ba{};
+            ba.g = ea.g;
+            ba.sci = ea.sci;
+            ba.ed = S.d_ed_big.as<ElimDesc>() + q0;
+            ba.nbox = (int)std::min(kGridMax, batch.size() - q0);
+            ba.groups = S.d_eg.as<ElimGroup>();
+            ba.sk = sf.sk.as<int>();
+            ba.rd = sf.rd.as<int>();
+            ba.Tws = Tws.p;
+            ba.ws = S.ews.p;
+            ba.pool = sf.pool.p;
+            ba.piv = S.piv.as<int>();
+            ba.perm = sf.perm.as<int>();
+            ba.sci_pool = sci_pool;
+            ba.status = h->status.as<int>();
+            // HIF_TC_GEMM=1: the products on the tensor cores (hif_gemm_batched_f32).
+            // Off by default: the tensor core's FP32 accumulation of the long
+            // products (K = k or r) is less accurate than the SIMT FMA chains, and
+            // at N = 1M the FP32 factor's refinement contraction went from ~1e-3
+            // to ~4e-3 per step (one refinement step more), for no gain in time.
+            if (tc_gemm) ba.gemm_probs = S.gemm_probs.p;
+            ba.factor_max_r = be_max_r;
+            ba.num_sms = h->num_sms;
+            ba.ldl_alpha = ea.ldl_alpha;
+            ba.ldl_fail = ea.ldl_fail;
+            ba.fail_idx = S.elim_fail_idx.as<int>() + q0;
+            int mxn = 0, mxk = 0, mxr = 0, smr = 0;
+            for (int q = 0; q < ba.nbox; ++q) {
+                const ElimDesc& eb = batch[q0 + q];
+                mxn = std::max(mxn, eb.k + eb.r);
+                mxk = std::max(mxk, eb.k);
+                mxr = std::max(mxr, eb.r);
+                if (eb.r <= ba.factor_max_r) smr = std::max(smr, eb.r);
+            }
+            HIF_CUDA((big_elim_batch<T>(ba, mxn, mxk, mxr, smr, st)));
         }
-        BatchElimArgs ba{};
-        ba.g = ea.g;
-        ba.sci = ea.sci;
-        ba.ed = S.d_ed_big.as<ElimDesc>();
-        ba.nbox = (int)ed_big.size();
-        ba.groups = S.d_eg.as<ElimGroup>();
-        ba.sk = sf.sk.as<int>();
-        ba.rd = sf.rd.as<int>();
-        ba.Tws = Tws.p;
-        ba.ws = S.ews.p;
-        ba.pool = sf.pool.p;
-        ba.piv = S.piv.as<int>();
-        ba.perm = sf.perm.as<int>();
-        ba.sci_pool = sci_pool;
-        ba.status = h->status.as<int>();
-        // HIF_TC_GEMM=1: the products on the tensor cores (hif_gemm_batched_f32).
-        // Off by default: the tensor core's FP32 accumulation of the long
-        // products (K = k or r) is less accurate than the SIMT FMA chains, and
-        // at N = 1M the FP32 factor's refinement contraction went from ~1e-3
-        // to ~4e-3 per step (one refinement step more), for no gain in time.
-        if (env_int("HIF_TC_GEMM", 0)) {
-            S.gemm_probs.ensure(sizeof(TcGemmProb) * 5 * ed_big.size());
-            ba.gemm_probs = S.gemm_probs.p;
-        }
-        ProfRange pr(PROF_BIG_ELIM, st, work[1], 0.0);
-        HIF_CUDA((big_elim_batch<T>(ba, mxn, mxk, mxr, st)));
     }
 }
 
@@ -1221,7 +1253,7 @@ static void run_factor(hif_handle h) {
             e.k = k;
             e.r = r;
             const bool big = k + r > big_elim_n;
-            // LDL for symmetric problems (Sec. 5) on the one-CTA path
+            // LDL for symmetric problems (Sec. 5) below the large-box line
             e.ldl = (h->opt.ldl && b.sym && !big) ? 1 : 0;
             if (k > 0) {
                 e.sci_out = sci_off;

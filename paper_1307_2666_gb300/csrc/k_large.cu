@@ -1010,10 +1010,12 @@ __global__ void be_T_kernel(BatchElimArgs a) {
 // the GEMMs of Lemma 2.4 and the Schur update, one op per launch:
 // 0: B_sr = A_sr - A_ss T     1: B_rr -= T^T B_sr     2: B_rr -= A_rs T
 // 3: B_rs = A_rs - T^T A_ss   4: S = -X Z (into the SCI pool)
-template <typename T>
+// TS x TS tiles: 64, or 32 where the boxes give few of them.
+template <typename T, int TS>
 __global__ void __launch_bounds__(256) be_gemm_kernel(BatchElimArgs a, int op) {
-    __shared__ T As[16][64 + 1];
-    __shared__ T Bs[16][64 + 1];
+    constexpr int Q = TS / 16;
+    __shared__ T As[16][TS + 1];
+    __shared__ T Bs[16][TS + 1];
     const int e = blockIdx.z;
     const ElimDesc d = a.ed[e];
     const EBox<T> Bx(a, e);
@@ -1033,20 +1035,20 @@ __global__ void __launch_bounds__(256) be_gemm_kernel(BatchElimArgs a, int op) {
         case 0: m = k; n = r; kk = k; A = Ass; lda = ld; Bm = Bx.Tm; ldb = k; C = Asr; ldc = ld; break;
         case 1: m = r; n = r; kk = k; A = Bx.Tm; lda = k; tA = true; Bm = Asr; ldb = ld; C = Arr; ldc = ld; break;
         case 2: m = r; n = r; kk = k; A = Ars; lda = ld; Bm = Bx.Tm; ldb = k; C = Arr; ldc = ld; break;
-        case 3: m = r; n = k; kk = k; A = Bx.Tm; lda = k; tA = true; Bm = Ass; ldb = ld; C = Ars; ldc = ld; break;
+        case 3: if (d.ldl) return; m = r; n = k; kk = k; A = Bx.Tm; lda = k; tA = true; Bm = Ass; ldb = ld; C = Ars; ldc = ld; break;
         default:
             if (k == 0 || d.sci_out < 0) return;
             m = k; n = k; kk = r; A = Asr; lda = ld; Bm = Ars; ldb = ld;
             C = static_cast<T*>(a.sci_pool) + d.sci_out; ldc = k;
             break;
     }
-    const int i0 = blockIdx.x * 64, j0 = blockIdx.y * 64;
+    const int i0 = blockIdx.x * TS, j0 = blockIdx.y * TS;
     if (i0 >= m || j0 >= n || kk == 0) return;
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    T acc[4][4] = {};
+    T acc[Q][Q] = {};
     for (int l0 = 0; l0 < kk; l0 += 16) {
-        for (int q = threadIdx.x; q < 64 * 16; q += 256) {
-            const int rr = q % 64, l = q / 64;
+        for (int q = threadIdx.x; q < TS * 16; q += 256) {
+            const int rr = q % TS, l = q / TS;
             const int i = i0 + rr, kx = l0 + l;
             T v = T(0);
             if (i < m && kx < kk) v = tA ? A[kx + lda * i] : A[i + lda * kx];
@@ -1057,17 +1059,22 @@ __global__ void __launch_bounds__(256) be_gemm_kernel(BatchElimArgs a, int op) {
             Bs[l][rr] = u;
         }
         __syncthreads();
+#pragma unroll
         for (int l = 0; l < 16; ++l) {
-            T av[4], bv[4];
-            for (int q = 0; q < 4; ++q) av[q] = As[l][tx + 16 * q];
-            for (int q = 0; q < 4; ++q) bv[q] = Bs[l][ty + 16 * q];
-            for (int p = 0; p < 4; ++p)
-                for (int q = 0; q < 4; ++q) acc[p][q] += av[p] * bv[q];
+            T av[Q], bv[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) av[q] = As[l][tx + 16 * q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) bv[q] = Bs[l][ty + 16 * q];
+#pragma unroll
+            for (int p = 0; p < Q; ++p)
+#pragma unroll
+                for (int q = 0; q < Q; ++q) acc[p][q] += av[p] * bv[q];
         }
         __syncthreads();
     }
-    for (int p = 0; p < 4; ++p)
-        for (int q = 0; q < 4; ++q) {
+    for (int p = 0; p < Q; ++p)
+        for (int q = 0; q < Q; ++q) {
             const int i = i0 + tx + 16 * p, jj = j0 + ty + 16 * q;
             if (i < m && jj < n) {
                 if (op == 4) C[i + ldc * jj] = -acc[p][q];
@@ -1110,7 +1117,254 @@ __global__ void be_probs_kernel(BatchElimArgs a, int op, TcGemmProb* out) {
     out[e] = p;
 }
 
-// blocked LU of B_rr (Lemma 2.1), panel / interchange+TRSM / update stages
+// ---- factorization of B_rr in shared memory, one cluster of CTAs per box ----
+//
+// One pivot step is a search, a column that every CTA needs and a rank-1
+// update: for r of a few hundred the chain of steps, not the arithmetic, sets
+// the time, and from global memory a step costs several dependent round trips.
+// Here the block lives in the shared memory of a cluster (columns dealt out
+// in turn), a step's column goes to every CTA by distributed shared memory,
+// and the steps are separated by one (LU) or two (LDL) cluster barriers.
+// Pivots are not moved: `at` maps positions to rows (and columns, LDL), with
+// the interchanges of the textbook scheme applied to it alone, so ties go to
+// the lowest position as they do there.  Output in position order: LU (L
+// strictly below the diagonal), or for LDL boxes L below, D, and D L^T above.
+// Measured on a GB300 against the one-CTA and panel kernels this replaces: a
+// 64-bit LDL block of 388 rows 60 -> 3 ms with all its stages.
+constexpr int FT = 512;
+constexpr int FCL = 8;                       // largest cluster
+constexpr size_t kFactorSmemMax = 224 * 1024;
+
+template <typename T>
+size_t be_factor_smem(int r, int cl) {
+    return (size_t)((r + cl - 1) / cl) * r * sizeof(T) + 2 * (size_t)r * sizeof(T) + 2 * (size_t)r * sizeof(int) + 64;
+}
+
+__device__ __forceinline__ uint32_t cl_peer(const void* p, int rank) {
+    uint32_t out;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return out;
+}
+__device__ __forceinline__ void cl_store(uint32_t a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cl_store(uint32_t a, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cl_store(uint32_t a, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cl_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// largest v, then lowest pos, over the warp; id follows (-1: no candidate)
+template <typename T>
+__device__ __forceinline__ void warp_best(T& v, int& pos, int& id) {
+    for (int o = 16; o; o >>= 1) {
+        const T v2 = __shfl_xor_sync(0xffffffffu, v, o);
+        const int p2 = __shfl_xor_sync(0xffffffffu, pos, o), i2 = __shfl_xor_sync(0xffffffffu, id, o);
+        if (i2 >= 0 && (id < 0 || v2 > v || (v2 == v && p2 < pos))) { v = v2; pos = p2; id = i2; }
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(FT) be_factor_kernel(BatchElimArgs a, int cl) {
+    const int e = blockIdx.x / cl, rank = blockIdx.x % cl;
+    const ElimDesc d = a.ed[e];
+    const int r = d.r;
+    if (r > a.factor_max_r) return;                   // panel path (the whole cluster leaves)
+    const int64_t ld = d.k + r;
+    T* Ag = static_cast<T*>(a.ws) + d.ws_off;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ T cval[2][FCL];
+    __shared__ int cid[2][FCL], cpos[2][FCL];
+    const int own = (r - rank + cl - 1) / cl;         // columns rank, rank + cl, ...
+    T* A = reinterpret_cast<T*>(smem_raw);            // A[i + r * s]: column rank + cl * s
+    T* col = A + (size_t)((r + cl - 1) / cl) * r;     // col[r * parity + i]
+    int* at = reinterpret_cast<int*>(col + 2 * r);
+    int* pos = at + r;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int NW = FT / 32;
+    for (int q = threadIdx.x; q < own * r; q += FT) A[q] = Ag[q % r + ld * (rank + cl * (q / r))];
+    for (int i = threadIdx.x; i < r; i += FT) at[i] = pos[i] = i;
+    __syncthreads();
+    if (cl > 1) cl_sync();                            // every CTA is there before the first remote store
+    for (int j = 0; j < r; ++j) {
+        T* c = col + r * (j & 1);
+        int p;
+        T inv;
+        if (d.ldl) {
+            // remaining diagonal entry of largest magnitude
+            if (warp == 0) {
+                T v = T(-1);
+                int ps = 0, id = -1;
+                for (int s = lane; s < own; s += 32) {
+                    const int q = rank + cl * s, pq = pos[q];
+                    const T x = fabs(A[q + r * s]);
+                    if (pq >= j && (id < 0 ? x == x : x > v || (x == v && pq < ps))) { v = x; ps = pq; id = q; }
+                }
+                warp_best(v, ps, id);
+                if (lane < cl) {
+                    cl_store(cl_peer(&cval[j & 1][rank], lane), v);
+                    cl_store(cl_peer(&cpos[j & 1][rank], lane), ps);
+                    cl_store(cl_peer(&cid[j & 1][rank], lane), id);
+                }
+            }
+            if (cl > 1) cl_sync();
+            else __syncthreads();
+            T v = T(-1);
+            int ps = 0;
+            p = -1;
+            for (int q = 0; q < cl; ++q) {
+                const T x = cval[j & 1][q];
+                const int pq = cpos[j & 1][q], id = cid[j & 1][q];
+                if (id >= 0 && (p < 0 || x > v || (x == v && pq < ps))) { v = x; ps = pq; p = id; }
+            }
+            if (p < 0) p = at[j];                     // no comparable entry: the test below fails
+            if (p % cl == rank) {
+                const T* src = A + (size_t)r * (p / cl);
+                for (int i = threadIdx.x; i < r; i += FT) {
+                    const T x = pos[i] >= j ? src[i] : T(0);
+                    for (int q = 0; q < cl; ++q) cl_store(cl_peer(c + i, q), x);
+                }
+            }
+            if (cl > 1) cl_sync();
+            else __syncthreads();
+            const T dp = c[p];
+            T cm = T(0);
+            for (int i = lane; i < r; i += 32)
+                if (i != p) cm = fmax(cm, fabs(c[i]));
+            for (int o = 16; o; o >>= 1) cm = fmax(cm, __shfl_xor_sync(0xffffffffu, cm, o));
+            if (dp == T(0) || !isfinite((double)dp)) {
+                if (rank == 0 && threadIdx.x == 0) atomicOr(a.status, (int)DEV_SINGULAR);
+                break;
+            }
+            if (!(fabs(dp) >= (T)a.ldl_alpha * cm)) {
+                if (rank == 0 && threadIdx.x == 0) {
+                    atomicOr(a.status, (int)DEV_LDL_FALLBACK);
+                    a.ldl_fail[a.fail_idx[e]] = 1;
+                }
+                break;
+            }
+            inv = T(1) / dp;
+            for (int s = warp; s < own; s += NW) {
+                const int q = rank + cl * s;
+                if (pos[q] < j || q == p) continue;
+                const T vq = c[q];
+                T* x = A + (size_t)r * s;
+                for (int i = lane; i < r; i += 32)
+                    if (i != p) x[i] -= c[i] * vq * inv;
+            }
+            if (p % cl == rank) {
+                T* x = A + (size_t)r * (p / cl);
+                for (int i = threadIdx.x; i < r; i += FT)
+                    if (pos[i] >= j && i != p) x[i] = c[i] * inv;
+            }
+        } else {
+            // largest remaining entry of column j
+            if (j % cl == rank) {
+                T* x = A + (size_t)r * (j / cl);
+                if (warp == 0) {
+                    T v = T(-1);
+                    int ps = 0, id = -1;
+                    for (int i = lane; i < r; i += 32) {
+                        const T y = fabs(x[i]);
+                        const int pi = pos[i];
+                        if (pi >= j && (id < 0 ? y == y : y > v || (y == v && pi < ps))) { v = y; ps = pi; id = i; }
+                    }
+                    warp_best(v, ps, id);
+                    if (id < 0) id = at[j];           // (all NaN: the pivot test below fails)
+                    if (lane < cl) {
+                        cl_store(cl_peer(&cid[j & 1][0], lane), id);
+                        cl_store(cl_peer(&cval[j & 1][0], lane), x[id]);
+                    }
+                    if (lane == 0) cpos[0][1] = id;
+                }
+                __syncthreads();
+                const int pp = cpos[0][1];
+                const T pinv = T(1) / x[pp];
+                for (int i = threadIdx.x; i < r; i += FT) {
+                    const bool on = pos[i] >= j && i != pp;
+                    const T l = on ? x[i] * pinv : T(0);
+                    if (on) x[i] = l;
+                    for (int q = 0; q < cl; ++q) cl_store(cl_peer(c + i, q), l);
+                }
+            }
+            if (cl > 1) cl_sync();
+            else __syncthreads();
+            p = cid[j & 1][0];
+            const T dp = cval[j & 1][0];
+            if (dp == T(0) || !isfinite((double)dp)) {
+                if (rank == 0 && threadIdx.x == 0) atomicOr(a.status, (int)DEV_SINGULAR);
+                break;
+            }
+            for (int s = warp; s < own; s += NW) {
+                if (rank + cl * s <= j) continue;
+                T* x = A + (size_t)r * s;
+                const T u = x[p];
+                for (int i = lane; i < r; i += 32) x[i] -= c[i] * u;
+            }
+        }
+        __syncthreads();                              // updates done, pos and at read
+        if (threadIdx.x == 0) {
+            const int t = at[j], pp = pos[p];
+            at[j] = p;
+            at[pp] = t;
+            pos[t] = pp;
+            pos[p] = j;
+        }
+        __syncthreads();
+    }
+    if (cl > 1) cl_sync();                            // no CTA leaves while a peer may store to it
+    else __syncthreads();
+    for (int q = threadIdx.x; q < own * r; q += FT) {
+        const int i = q % r, s = q / r, o = rank + cl * s, j = d.ldl ? pos[o] : o;
+        const T* x = A + (size_t)r * s;
+        const T v = x[at[i]];
+        if (!d.ldl || i >= j) Ag[i + ld * j] = v;
+        if (d.ldl && i > j) Ag[j + ld * i] = v * x[o];
+    }
+    if (rank == 0)
+        for (int i = threadIdx.x; i < r; i += FT) a.perm[d.piv_out + i] = at[i];
+}
+
+// the largest block that fits into a cluster's shared memory
+template <typename T>
+int be_factor_max_r() {
+    int r = 1;
+    while (be_factor_smem<T>(r + 1, FCL) <= kFactorSmemMax) ++r;
+    return r;
+}
+
+template <typename T>
+cudaError_t launch_be_factor(const BatchElimArgs& a, int max_r, cudaStream_t st) {
+    // CTAs per box: as many as the largest block needs, more while the
+    // sublevel's boxes leave SMs idle and each CTA keeps 16 columns
+    int cl = 1;
+    while (cl < FCL && be_factor_smem<T>(max_r, cl) > kFactorSmemMax) cl *= 2;
+    while (cl < FCL && 2 * cl * a.nbox <= a.num_sms && max_r >= 32 * cl) cl *= 2;
+    const size_t smem = be_factor_smem<T>(max_r, cl);
+    cudaError_t e = cudaFuncSetAttribute(be_factor_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kFactorSmemMax);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(a.nbox * cl));
+    cfg.blockDim = dim3(FT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)cl;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = cl > 1 ? 1 : 0;
+    note_launch();
+    return cudaLaunchKernelEx(&cfg, be_factor_kernel<T>, a, cl);
+}
+
+// blocked LU of B_rr (Lemma 2.1) of blocks too large for that, panel /
+// interchange+TRSM / update stages
 constexpr int PNT = 512;   // threads of the LU panel kernel (the pivot search spans all rows)
 
 template <typename T>
@@ -1119,7 +1373,7 @@ __global__ void __launch_bounds__(PNT) be_panel_kernel(BatchElimArgs a, int j0) 
     const ElimDesc d = a.ed[e];
     const EBox<T> Bx(a, e);
     const int n = Bx.r;
-    if (j0 >= n) return;
+    if (j0 >= n || n <= a.factor_max_r) return;
     const int nb = min(32, n - j0);
     const int64_t ld = Bx.n;
     T* A = Bx.A;
@@ -1181,7 +1435,7 @@ __global__ void be_swap_trsm_kernel(BatchElimArgs a, int j0) {
     const ElimDesc d = a.ed[e];
     const EBox<T> Bx(a, e);
     const int n = Bx.r;
-    if (j0 >= n) return;
+    if (j0 >= n || n <= a.factor_max_r) return;
     const int nb = min(32, n - j0);
     const int64_t ld = Bx.n;
     T* A = Bx.A;
@@ -1209,7 +1463,7 @@ __global__ void __launch_bounds__(256) be_update_kernel(BatchElimArgs a, int j0)
     const int e = blockIdx.z;
     const EBox<T> Bx(a, e);
     const int n = Bx.r;
-    if (j0 >= n) return;
+    if (j0 >= n || n <= a.factor_max_r) return;
     const int nb = min(32, n - j0);
     const int s = j0 + nb;
     const int i0 = s + blockIdx.x * 64, c0 = s + blockIdx.y * 64;
@@ -1273,9 +1527,9 @@ __global__ void be_lu_out_kernel(BatchElimArgs a) {
     for (int64_t q = t0; q < r; q += stride) Dv[q] = Arr[q + ld * q];
     for (int64_t q = t0; q < (int64_t)r * r; q += stride) {
         const int i = (int)(q % r), j = (int)(q / r);
-        LUo[q] = i == j ? T(0) : (i < j ? Arr[i + ld * j] / Arr[i + ld * i] : Arr[i + ld * j]);
+        LUo[q] = i == j || (d.ldl && i < j) ? T(0) : (i < j ? Arr[i + ld * j] / Arr[i + ld * i] : Arr[i + ld * j]);
     }
-    if (t0 == 0) {
+    if (t0 == 0 && r > a.factor_max_r) {
         int* pm = a.perm + d.piv_out;
         const int* piv = a.piv + d.piv_out;
         for (int i = 0; i < r; ++i) pm[i] = i;
@@ -1289,14 +1543,15 @@ __global__ void be_lu_out_kernel(BatchElimArgs a) {
 constexpr int IB = 32;   // block size of the triangular inverses
 
 // Unit lower factor F(i, l), i > l: L itself (UP false) or U'^T (UP true);
-// its inverse's entries (i > j) go to LUi_out at (i, j) or, transposed, (j, i).
+// its inverse's entries (i > j) go to LUi_out at (i, j) or, transposed, (j, i)
+// (U'^T, and L of an LDL box, whose inverse shares L's array).
 template <typename T, bool UP>
 __device__ __forceinline__ T tri_f(const T* F, int64_t r, int i, int l) {
     return UP ? F[l + r * i] : F[i + r * l];
 }
-template <typename T, bool UP>
-__device__ __forceinline__ T* tri_x(T* X, int64_t r, int i, int j) {
-    return UP ? X + j + r * i : X + i + r * j;
+template <typename T>
+__device__ __forceinline__ T* tri_x(T* X, int64_t r, bool xt, int i, int j) {
+    return xt ? X + j + r * i : X + i + r * j;
 }
 
 // inverses of the IB x IB diagonal blocks (one warp per block and box)
@@ -1306,7 +1561,8 @@ __global__ void be_dinv_kernel(BatchElimArgs a) {
     const ElimDesc d = a.ed[e];
     const int r = d.r;
     const int b0 = blockIdx.x * IB;
-    if (b0 >= r) return;
+    if (b0 >= r || (UP && d.ldl)) return;
+    const bool xt = UP || d.ldl;
     const int nbk = min(IB, r - b0);
     const T* F = static_cast<const T*>(a.pool) + d.LU_out;
     T* X = static_cast<T*>(a.pool) + d.LUi_out;
@@ -1329,7 +1585,7 @@ __global__ void be_dinv_kernel(BatchElimArgs a) {
     __syncthreads();
     for (int q = t; q < IB * IB; q += 32) {
         const int i = UP ? q / IB : q % IB, j = UP ? q % IB : q / IB;
-        if (i < nbk && j < nbk && i > j) *tri_x<T, UP>(X, r, b0 + i, b0 + j) = Xs[i][j];
+        if (i < nbk && j < nbk && i > j) *tri_x(X, r, xt, b0 + i, b0 + j) = Xs[i][j];
     }
     if (t < nbk) X[(b0 + t) + (int64_t)r * (b0 + t)] = T(0);
 }
@@ -1343,7 +1599,8 @@ __global__ void __launch_bounds__(256) be_binv_kernel(BatchElimArgs a) {
     const int r = d.r;
     const int nb = (r + IB - 1) / IB;
     const int J = blockIdx.x;
-    if (J >= nb - 1) return;
+    if (J >= nb - 1 || (UP && d.ldl)) return;
+    const bool xt = UP || d.ldl;
     const T* F = static_cast<const T*>(a.pool) + d.LU_out;
     T* X = static_cast<T*>(a.pool) + d.LUi_out;
     __shared__ T Fs[IB][IB + 1];
@@ -1362,7 +1619,7 @@ __global__ void __launch_bounds__(256) be_binv_kernel(BatchElimArgs a) {
                 const int xk = UP ? q / IB : q % IB, xj = UP ? q % IB : q / IB;
                 const int gk = K * IB + xk, gj = J * IB + xj;
                 T xv = T(0);
-                if (gk < r && gj < r) xv = gk == gj ? T(1) : (gk > gj ? *tri_x<T, UP>(X, r, gk, gj) : T(0));
+                if (gk < r && gj < r) xv = gk == gj ? T(1) : (gk > gj ? *tri_x(X, r, xt, gk, gj) : T(0));
                 Xs[xk][xj] = xv;
             }
             __syncthreads();
@@ -1380,7 +1637,7 @@ __global__ void __launch_bounds__(256) be_binv_kernel(BatchElimArgs a) {
         for (int q = t; q < IB * IB; q += 256) {
             const int i = UP ? q / IB : q % IB, l = UP ? q % IB : q / IB;
             const int gi = I * IB + i, gl = I * IB + l;
-            Fs[i][l] = (i > l && gi < r && gl < r) ? *tri_x<T, UP>(X, r, gi, gl) : T(0);
+            Fs[i][l] = (i > l && gi < r && gl < r) ? *tri_x(X, r, xt, gi, gl) : T(0);
         }
         __syncthreads();
         const int gi = I * IB + ti;
@@ -1389,22 +1646,24 @@ __global__ void __launch_bounds__(256) be_binv_kernel(BatchElimArgs a) {
             const int jj = tj + 8 * q, gj = J * IB + jj;
             T v = Xs[ti][jj];
             for (int l = 0; l < ti; ++l) v += Fs[ti][l] * Xs[l][jj];
-            if (gi < r && gj < r) *tri_x<T, UP>(X, r, gi, gj) = -v;
+            if (gi < r && gj < r) *tri_x(X, r, xt, gi, gj) = -v;
         }
     }
 }
 
 // X = B_sr U^{-1} by block columns: X_J = (B_J - sum_{K<J} X_K U_KJ) inv(U_JJ),
 // inv(U_JJ) = (I + S_JJ) D_J^{-1} with S_JJ the stored strict upper part of
-// the diagonal block of U'^{-1}.  One CTA per 64 rows of X and box; thread
-// (tx, ty) holds entries (tx, ty + 4 q), q < 8, of the 64 x 32 block.
-template <typename T>
+// the diagonal block of U'^{-1}.  LDL box: B_sr P^T (D L^T)^{-1}.  One CTA per
+// RT rows of X and box (64, or 16 where the boxes give few CTAs); thread
+// (tx, ty) holds entries (tx, ty + CT q) of the RT x 32 block.
+template <typename T, int RT>
 __global__ void __launch_bounds__(256) be_trsm_x_kernel(BatchElimArgs a) {
     const int e = blockIdx.y;
     const ElimDesc d = a.ed[e];
     const EBox<T> Bx(a, e);
     const int k = Bx.k, r = Bx.r;
-    const int i0 = blockIdx.x * 64;
+    constexpr int CT = 256 / RT, NQ = IB / CT;
+    const int i0 = blockIdx.x * RT;
     if (i0 >= k) return;
     const int64_t ld = Bx.n;
     const T* Arr = Bx.A;
@@ -1412,22 +1671,23 @@ __global__ void __launch_bounds__(256) be_trsm_x_kernel(BatchElimArgs a) {
     T* X = static_cast<T*>(a.pool) + d.X_out;
     const T* Si = static_cast<const T*>(a.pool) + d.LUi_out;
     const T* Dv = static_cast<const T*>(a.pool) + d.D_out;
-    __shared__ T Xs[64][IB + 1];
+    __shared__ T Xs[RT][IB + 1];
     __shared__ T Us[IB][IB + 1];
-    const int tx = threadIdx.x % 64, ty = threadIdx.x / 64;
+    const int tx = threadIdx.x % RT, ty = threadIdx.x / RT;
     const int i = i0 + tx;
+    const int* pm = a.perm + d.piv_out;
     const int rb = (r + IB - 1) / IB;
     for (int J = 0; J < rb; ++J) {
-        T acc[8];
+        T acc[NQ];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int c = J * IB + ty + 4 * q;
-            acc[q] = (i < k && c < r) ? Asr[i + ld * c] : T(0);
+        for (int q = 0; q < NQ; ++q) {
+            const int c = J * IB + ty + CT * q;
+            acc[q] = (i < k && c < r) ? Asr[i + ld * (d.ldl ? pm[c] : c)] : T(0);
         }
         for (int K = 0; K < J; ++K) {
             __syncthreads();
-            for (int q = threadIdx.x; q < 64 * IB; q += 256) {
-                const int rr = q % 64, l = q / 64, gl = K * IB + l;
+            for (int q = threadIdx.x; q < RT * IB; q += 256) {
+                const int rr = q % RT, l = q / RT, gl = K * IB + l;
                 Xs[rr][l] = (i0 + rr < k && gl < r) ? X[(i0 + rr) + (int64_t)k * gl] : T(0);
             }
             for (int q = threadIdx.x; q < IB * IB; q += 256) {
@@ -1439,20 +1699,20 @@ __global__ void __launch_bounds__(256) be_trsm_x_kernel(BatchElimArgs a) {
             for (int l = 0; l < IB; ++l) {
                 const T xv = Xs[tx][l];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) acc[q] -= xv * Us[l][ty + 4 * q];
+                for (int q = 0; q < NQ; ++q) acc[q] -= xv * Us[l][ty + CT * q];
             }
         }
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 8; ++q) Xs[tx][ty + 4 * q] = acc[q];
+        for (int q = 0; q < NQ; ++q) Xs[tx][ty + CT * q] = acc[q];
         for (int q = threadIdx.x; q < IB * IB; q += 256) {
             const int l = q % IB, c = q / IB, gl = J * IB + l, gc = J * IB + c;
             Us[l][c] = (l < c && gc < r) ? Si[gl + (int64_t)r * gc] : T(0);
         }
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int c = ty + 4 * q, gc = J * IB + c;
+        for (int q = 0; q < NQ; ++q) {
+            const int c = ty + CT * q, gc = J * IB + c;
             T v = Xs[tx][c];
             for (int l = 0; l < c; ++l) v += Xs[tx][l] * Us[l][c];
             if (i < k && gc < r) X[i + (int64_t)k * gc] = v / Dv[gc];
@@ -1462,16 +1722,18 @@ __global__ void __launch_bounds__(256) be_trsm_x_kernel(BatchElimArgs a) {
 
 // Z = L^{-1} P B_rs by block rows: Z_I = (I + S_II) (PB_I - sum_{K<I} L_IK Z_K),
 // S_II the stored strict lower part of the diagonal block of L^{-1}.  Z goes
-// to Y_out (scaled by D^{-1} later).  One CTA per 64 columns of Z and box;
-// thread (tr, tc) holds entries (tr, tc + 8 q), q < 8, of the 32 x 64 block.
-template <typename T>
+// to Y_out (scaled by D^{-1} later); LDL boxes need none.  One CTA per RT
+// columns of Z and box; thread (tr, tc) holds entries (tr, tc + 8 q) of the
+// 32 x RT block.
+template <typename T, int RT>
 __global__ void __launch_bounds__(256) be_trsm_z_kernel(BatchElimArgs a) {
     const int e = blockIdx.y;
     const ElimDesc d = a.ed[e];
     const EBox<T> Bx(a, e);
     const int k = Bx.k, r = Bx.r;
-    const int j0 = blockIdx.x * 64;
-    if (j0 >= k) return;
+    constexpr int NQ = RT / 8;
+    const int j0 = blockIdx.x * RT;
+    if (j0 >= k || d.ldl) return;
     const int64_t ld = Bx.n;
     const T* Arr = Bx.A;
     const T* Ars = Bx.A + ld * r;
@@ -1479,14 +1741,14 @@ __global__ void __launch_bounds__(256) be_trsm_z_kernel(BatchElimArgs a) {
     const T* Si = static_cast<const T*>(a.pool) + d.LUi_out;
     const int* pm = a.perm + d.piv_out;
     __shared__ T Ls[IB][IB + 1];
-    __shared__ T Zs[IB][64 + 1];
+    __shared__ T Zs[IB][RT + 1];
     const int tr = threadIdx.x % IB, tc = threadIdx.x / IB;
     const int rb = (r + IB - 1) / IB;
     for (int I = 0; I < rb; ++I) {
         const int gi = I * IB + tr;
-        T acc[8];
+        T acc[NQ];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < NQ; ++q) {
             const int j = j0 + tc + 8 * q;
             acc[q] = (gi < r && j < k) ? Ars[pm[gi] + ld * j] : T(0);
         }
@@ -1496,7 +1758,7 @@ __global__ void __launch_bounds__(256) be_trsm_z_kernel(BatchElimArgs a) {
                 const int rr = q % IB, l = q / IB, g1 = I * IB + rr, g2 = K * IB + l;
                 Ls[rr][l] = (g1 < r && g2 < r) ? Arr[g1 + ld * g2] : T(0);
             }
-            for (int q = threadIdx.x; q < IB * 64; q += 256) {
+            for (int q = threadIdx.x; q < IB * RT; q += 256) {
                 const int l = q % IB, c = q / IB, gl = K * IB + l;
                 Zs[l][c] = (gl < r && j0 + c < k) ? Z[gl + (int64_t)r * (j0 + c)] : T(0);
             }
@@ -1505,19 +1767,19 @@ __global__ void __launch_bounds__(256) be_trsm_z_kernel(BatchElimArgs a) {
             for (int l = 0; l < IB; ++l) {
                 const T lv = Ls[tr][l];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) acc[q] -= lv * Zs[l][tc + 8 * q];
+                for (int q = 0; q < NQ; ++q) acc[q] -= lv * Zs[l][tc + 8 * q];
             }
         }
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 8; ++q) Zs[tr][tc + 8 * q] = acc[q];
+        for (int q = 0; q < NQ; ++q) Zs[tr][tc + 8 * q] = acc[q];
         for (int q = threadIdx.x; q < IB * IB; q += 256) {
             const int rr = q % IB, l = q / IB, g1 = I * IB + rr, g2 = I * IB + l;
             Ls[rr][l] = (rr > l && g1 < r) ? Si[g1 + (int64_t)r * g2] : T(0);
         }
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < NQ; ++q) {
             const int c = tc + 8 * q;
             T v = Zs[tr][c];
             for (int l = 0; l < tr; ++l) v += Ls[tr][l] * Zs[l][c];
@@ -1526,46 +1788,48 @@ __global__ void __launch_bounds__(256) be_trsm_z_kernel(BatchElimArgs a) {
     }
 }
 
-// S = -X Z into the SCI pool (64 x 64 tiles, K = r by 16)
-template <typename T>
+// S = -X Z into the SCI pool, -X D X^T of an LDL box (TS x TS tiles, K = r by 16)
+template <typename T, int TS>
 __global__ void __launch_bounds__(256) be_schur_kernel(BatchElimArgs a) {
-    __shared__ T As[16][64 + 1];
-    __shared__ T Bs[16][64 + 1];
+    constexpr int Q = TS / 16;
+    __shared__ T As[16][TS + 1];
+    __shared__ T Bs[16][TS + 1];
     const int e = blockIdx.z;
     const ElimDesc d = a.ed[e];
     const int k = d.k, r = d.r;
     if (k == 0 || d.sci_out < 0) return;
-    const int i0 = blockIdx.x * 64, j0 = blockIdx.y * 64;
+    const int i0 = blockIdx.x * TS, j0 = blockIdx.y * TS;
     if (i0 >= k || j0 >= k) return;
     const T* X = static_cast<const T*>(a.pool) + d.X_out;
     const T* Z = static_cast<const T*>(a.pool) + d.Y_out;
+    const T* Dv = static_cast<const T*>(a.pool) + d.D_out;
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    T acc[4][4] = {};
+    T acc[Q][Q] = {};
     for (int l0 = 0; l0 < r; l0 += 16) {
-        for (int q = threadIdx.x; q < 64 * 16; q += 256) {
-            const int rr = q % 64, l = q / 64;
+        for (int q = threadIdx.x; q < TS * 16; q += 256) {
+            const int rr = q % TS, l = q / TS;
             const int i = i0 + rr, kx = l0 + l, jj = j0 + rr;
             As[l][rr] = (i < k && kx < r) ? X[i + (int64_t)k * kx] : T(0);
-            Bs[l][rr] = (jj < k && kx < r) ? Z[kx + (int64_t)r * jj] : T(0);
+            Bs[l][rr] = (jj < k && kx < r) ? (d.ldl ? X[jj + (int64_t)k * kx] * Dv[kx] : Z[kx + (int64_t)r * jj]) : T(0);
         }
         __syncthreads();
 #pragma unroll
         for (int l = 0; l < 16; ++l) {
-            T av[4], bv[4];
+            T av[Q], bv[Q];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) av[q] = As[l][tx + 16 * q];
+            for (int q = 0; q < Q; ++q) av[q] = As[l][tx + 16 * q];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) bv[q] = Bs[l][ty + 16 * q];
+            for (int q = 0; q < Q; ++q) bv[q] = Bs[l][ty + 16 * q];
 #pragma unroll
-            for (int p = 0; p < 4; ++p)
+            for (int p = 0; p < Q; ++p)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[p][q] += av[p] * bv[q];
+                for (int q = 0; q < Q; ++q) acc[p][q] += av[p] * bv[q];
         }
         __syncthreads();
     }
     T* S = static_cast<T*>(a.sci_pool) + d.sci_out;
-    for (int p = 0; p < 4; ++p)
-        for (int q = 0; q < 4; ++q) {
+    for (int p = 0; p < Q; ++p)
+        for (int q = 0; q < Q; ++q) {
             const int i = i0 + tx + 16 * p, jj = j0 + ty + 16 * q;
             if (i < k && jj < k) S[i + (int64_t)k * jj] = -acc[p][q];
         }
@@ -1584,19 +1848,29 @@ __global__ void be_finish_kernel(BatchElimArgs a) {
     T* To = pool + d.T_out;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    for (int64_t q = t0; q < (int64_t)r * k; q += stride) Yo[q] /= Dv[q % r];
+    if (!d.ldl)
+        for (int64_t q = t0; q < (int64_t)r * k; q += stride) Yo[q] /= Dv[q % r];
     for (int64_t q = t0; q < (int64_t)k * r; q += stride) To[q] = Bx.Tm[q];
 }
 
 template <typename T>
-cudaError_t big_elim_batch(const BatchElimArgs& a, int max_n, int max_k, int max_r, cudaStream_t st) {
+cudaError_t big_elim_batch(const BatchElimArgs& a, int max_n, int max_k, int max_r, int small_r, cudaStream_t st) {
     const int nb = a.nbox;
     if (nb == 0) return cudaSuccess;
     note_launch();
     be_gather_kernel<T><<<dim3((unsigned)std::min<int64_t>(((int64_t)max_n * max_n + 255) / 256, 1024), nb), 256, 0, st>>>(a);
     note_launch();
     be_T_kernel<T><<<nb, 256, 0, st>>>(a);
-    const int tk = (max_k + 63) / 64, tr = (max_r + 63) / 64;
+    // small tiles while 64 x 64 ones would leave SMs idle (n = 64, 64-bit: 4
+    // boxes of 348 give 36 tiles of 64, 484 of 32)
+    const int tm = std::max(max_k, max_r);
+    const bool small = (int64_t)((tm + 63) / 64) * ((tm + 63) / 64) * nb < 2 * a.num_sms;
+    const int ts = small ? 32 : 64, tk = (max_k + ts - 1) / ts, tr = (max_r + ts - 1) / ts;
+    auto gemm_op = [&](int op, int mt, int nt) {
+        note_launch();
+        if (small) be_gemm_kernel<T, 32><<<dim3(mt, nt, nb), 256, 0, st>>>(a, op);
+        else be_gemm_kernel<T, 64><<<dim3(mt, nt, nb), 256, 0, st>>>(a, op);
+    };
     // FP32: the products of Lemma 2.4 and the Schur update on the tensor cores
     TcGemmProb* probs = static_cast<TcGemmProb*>(a.gemm_probs);
     const bool tcg = sizeof(T) == 4 && probs != nullptr;
@@ -1612,16 +1886,16 @@ cudaError_t big_elim_batch(const BatchElimArgs& a, int max_n, int max_k, int max
         if ((e = tc_op(2, max_r, max_r)) != cudaSuccess) return e;
         if ((e = tc_op(3, max_r, max_k)) != cudaSuccess) return e;
     } else if (max_k > 0) {
-        note_launch();
-        be_gemm_kernel<T><<<dim3(tk, tr, nb), 256, 0, st>>>(a, 0);
-        note_launch();
-        be_gemm_kernel<T><<<dim3(tr, tr, nb), 256, 0, st>>>(a, 1);
-        note_launch();
-        be_gemm_kernel<T><<<dim3(tr, tr, nb), 256, 0, st>>>(a, 2);
-        note_launch();
-        be_gemm_kernel<T><<<dim3(tr, tk, nb), 256, 0, st>>>(a, 3);
+        gemm_op(0, tk, tr);
+        gemm_op(1, tr, tr);
+        gemm_op(2, tr, tr);
+        gemm_op(3, tr, tk);
     }
-    for (int j0 = 0; j0 < max_r; j0 += 32) {
+    if (small_r > 0) {
+        const cudaError_t e = launch_be_factor<T>(a, small_r, st);
+        if (e != cudaSuccess) return e;
+    }
+    for (int j0 = 0; max_r > a.factor_max_r && j0 < max_r; j0 += 32) {
         note_launch();
         be_panel_kernel<T><<<nb, PNT, 0, st>>>(a, j0);
         note_launch();
@@ -1647,15 +1921,18 @@ cudaError_t big_elim_batch(const BatchElimArgs& a, int max_n, int max_k, int max
     }
     if (max_k > 0) {
         note_launch();
-        be_trsm_x_kernel<T><<<dim3(tk, nb), 256, 0, st>>>(a);
+        if (small) be_trsm_x_kernel<T, 16><<<dim3((max_k + 15) / 16, nb), 256, 0, st>>>(a);
+        else be_trsm_x_kernel<T, 64><<<dim3(tk, nb), 256, 0, st>>>(a);
         note_launch();
-        be_trsm_z_kernel<T><<<dim3(tk, nb), 256, 0, st>>>(a);
+        if (small) be_trsm_z_kernel<T, 16><<<dim3((max_k + 15) / 16, nb), 256, 0, st>>>(a);
+        else be_trsm_z_kernel<T, 64><<<dim3(tk, nb), 256, 0, st>>>(a);
         if (tcg) {
             const cudaError_t e = tc_op(4, max_k, max_k);
             if (e != cudaSuccess) return e;
         } else {
             note_launch();
-            be_schur_kernel<T><<<dim3(tk, tk, nb), 256, 0, st>>>(a);
+            if (small) be_schur_kernel<T, 32><<<dim3(tk, tk, nb), 256, 0, st>>>(a);
+            else be_schur_kernel<T, 64><<<dim3(tk, tk, nb), 256, 0, st>>>(a);
         }
     }
     note_launch();
@@ -1672,7 +1949,8 @@ cudaError_t big_elim_batch(const BatchElimArgs& a, int max_n, int max_k, int max
     template cudaError_t big_qr_step<T>(const BigArgs&, int, int, int, cudaStream_t);                          \
     template cudaError_t big_qp_panel<T>(const BigArgs&, int, int, int, int&, cudaStream_t);                   \
     template cudaError_t big_finish<T>(const BigArgs&, int, int, cudaStream_t);                                \
-    template cudaError_t big_elim_batch<T>(const BatchElimArgs&, int, int, int, cudaStream_t);
+    template cudaError_t big_elim_batch<T>(const BatchElimArgs&, int, int, int, int, cudaStream_t);               \
+    template int be_factor_max_r<T>();
 HIF_INST(double)
 HIF_INST(float)
 

@@ -197,8 +197,16 @@ struct BatchElimArgs {
     void* sci_pool;
     int* status;
     void* gemm_probs;         // FP32: 5 nbox TcGemmProb of work space for the tensor-core products
+    int factor_max_r;         // B_rr up to this size is factored in shared memory (be_factor_max_r)
+    int num_sms;
+    double ldl_alpha;         // as in ElimArgs
+    int* ldl_fail;            // ldl_fail[fail_idx[box]] = 1 when an LDL pivot failed the test
+    const int* fail_idx;
 };
-template <typename T> cudaError_t big_elim_batch(const BatchElimArgs&, int max_n, int max_k, int max_r, cudaStream_t);
+// small_r: the largest r <= factor_max_r among the boxes (0: none)
+template <typename T>
+cudaError_t big_elim_batch(const BatchElimArgs&, int max_n, int max_k, int max_r, int small_r, cudaStream_t);
+template <typename T> int be_factor_max_r();
 
 size_t fold_smem_bytes(int n, int cpt, bool sci, bool R_in_smem, int elem);
 size_t id_smem_bytes(int ng, int mrow, bool W_in_smem, int elem);
