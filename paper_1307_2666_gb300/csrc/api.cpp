@@ -1018,10 +1018,43 @@ static void run_factor(hif_handle h) {
         });
         upload(d_small_groups, small_groups, st);
         Rws.ensure(sizeof(T) * std::max<int64_t>(Roff, 1));
+        // small boxes by width bucket, and the CTAs per box of each
         const bool grams = h->second_kind && any_sci;
+        struct Bucket { FoldArgs fa; int count, w, cpt, rc; size_t smem; };
+        std::vector<Bucket> buckets;
+        int max_split = 1;
+        {
+            int64_t at = 0;
+            const int widths[] = {32, 64, 96, 128, 160, 192, 224, 256, 512, 1024};
+            for (int w : widths) {
+                if (at >= (int64_t)small_boxes.size()) break;
+                const int64_t b0 = at;
+                int64_t pairs = 0;
+                while (at < (int64_t)small_boxes.size() && bd[small_sorted[at]].n <= w) {
+                    const BoxDesc& b = bd[small_sorted[at++]];
+                    pairs += (b.sym ? 1 : 2) * (int64_t)(b.m_near + h->P);
+                }
+                if (at == b0) continue;
+                const int cpt = fold_cpt(w, (int)sizeof(T));
+                if (cpt == 0) fail(HIF_EINVAL, "box too wide for the fold kernel");
+                Bucket bk{FoldArgs{}, (int)(at - b0), w, cpt, 0, 0};
+                bk.fa.box_list = d_small_sorted.as<int>() + b0;
+                bk.smem = fold_smem_bytes(w, cpt, grams, true, sizeof(T));
+                bk.fa.R_in_smem = bk.smem <= 220 * 1024;
+                if (!bk.fa.R_in_smem) bk.smem = fold_smem_bytes(w, cpt, grams, false, sizeof(T));
+                if (bk.smem > 220 * 1024) fail(HIF_EINVAL, "box too large for the fold kernel");
+                bk.fa.split = cpt == 1 && bk.fa.R_in_smem
+                                  ? fold_split(w, (pairs / bk.count + 31) / 32, bk.count, h->num_sms, (int)sizeof(T))
+                                  : 1;
+                if (const int fs = env_int("HIF_FOLD_SPLIT", 0); fs > 0 && cpt == 1 && bk.fa.R_in_smem) bk.fa.split = fs;
+                max_split = std::max(max_split, bk.fa.split);
+                buckets.push_back(bk);
+            }
+            if (at != (int64_t)small_boxes.size()) fail(HIF_EINVAL, "box too wide for the fold kernel");
+        }
         if (grams) {
-            GKws.ensure(sizeof(T) * Roff);
-            GSws.ensure(sizeof(T) * Roff);
+            GKws.ensure(sizeof(T) * Roff * max_split);
+            GSws.ensure(sizeof(T) * Roff * max_split);
         }
         Tws.ensure(sizeof(T) * std::max<int64_t>(Toff, 1));
         perm_out.ensure(sizeof(int) * std::max<size_t>(p.cols.size(), 1));
@@ -1050,26 +1083,14 @@ static void run_factor(hif_handle h) {
                 // handle's; the rows per chunk of each one-column-per-thread
                 // bucket are autotuned once per process (and precision, width)
                 ProfRange pr(PROF_FOLD, st, fold_flops, 0.0);
-                struct Bucket { FoldArgs fa; int count, w, cpt, rc; size_t smem; };
-                std::vector<Bucket> buckets;
-                int64_t at = 0;
-                const int widths[] = {32, 64, 96, 128, 160, 192, 224, 256, 512, 1024};
-                for (int w : widths) {
-                    if (at >= (int64_t)small_boxes.size()) break;
-                    const int64_t b0 = at;
-                    while (at < (int64_t)small_boxes.size() && bd[small_sorted[at]].n <= w) ++at;
-                    if (at == b0) continue;
-                    const int cpt = fold_cpt(w, (int)sizeof(T));
-                    if (cpt == 0) fail(HIF_EINVAL, "box too wide for the fold kernel");
-                    Bucket bk{fa, (int)(at - b0), w, cpt, 0, 0};
-                    bk.fa.box_list = d_small_sorted.as<int>() + b0;
-                    bk.smem = fold_smem_bytes(w, cpt, grams, true, sizeof(T));
-                    bk.fa.R_in_smem = bk.smem <= 220 * 1024;
-                    if (!bk.fa.R_in_smem) bk.smem = fold_smem_bytes(w, cpt, grams, false, sizeof(T));
-                    if (bk.smem > 220 * 1024) fail(HIF_EINVAL, "box too large for the fold kernel");
-                    buckets.push_back(bk);
+                for (Bucket& bk : buckets) {
+                    FoldArgs f = fa;
+                    f.box_list = bk.fa.box_list;
+                    f.R_in_smem = bk.fa.R_in_smem;
+                    f.split = bk.fa.split;
+                    f.gram_stride = Roff;
+                    bk.fa = f;
                 }
-                if (at != (int64_t)small_boxes.size()) fail(HIF_EINVAL, "box too wide for the fold kernel");
                 // autotune (synchronous, first sighting of a bucket only)
                 std::vector<char> done(buckets.size(), 0);
                 for (size_t q = 0; q < buckets.size(); ++q) {

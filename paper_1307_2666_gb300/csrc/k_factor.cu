@@ -57,9 +57,38 @@ __device__ inline T* align_ptr(unsigned char*& p, size_t count) {
 // second-kind mode the chunk's kernel and SCI parts also pass through shared
 // memory for the Gram matrices of Y^K and Y^S inside each column group
 // (Sec. 4.4), stored diagonal-major: G[l][l + t] at t * n + l.
+//
+// What bounds it: the chain of m n / RC column steps, not the arithmetic.  Two
+// things shorten it.
+//  - Rows are split over a cluster of args.split CTAs, each folding its share
+//    of the chunks into an R of its own; the R factors are then folded
+//    together in pairs through distributed shared memory (a row of an upper
+//    triangle starts at its diagonal, so a merge is n^2 / (2 RC) steps).  The
+//    split is chosen per bucket (fold_split).
+//  - In 64 bits a warp instruction occupies its scheduler's FP64 unit for 64
+//    cycles, so the owner's 2 RC operations on its column alone took as long
+//    as a warp's whole update; its warp now takes the column a row per lane.
+// Measured on a GB300, all folds of a factorization: 64-bit n = 64 22 -> 5.6 ms
+// (17 without the split), n = 200 with b != c 131 -> 81, Helmholtz n = 64 165
+// -> 42; 32-bit 3D n = 32 45 -> 29, n = 1024 187 -> 160 (forcing a split of 8
+// everywhere: 397).
+template <typename T>
+__device__ __forceinline__ T ld_peer(const T* p, int rank) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    T v;
+    if constexpr (sizeof(T) == 8) asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    else asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void fold_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 template <typename T, int RC, int CPT>
 __global__ void __launch_bounds__(256, CPT == 1 ? 2 : 1) fold_kernel(FoldArgs args) {
-    const BoxDesc bx = args.boxes[args.box_list[blockIdx.x]];
+    const int nsplit = CPT == 1 ? args.split : 1, rank = CPT == 1 ? blockIdx.x % nsplit : 0;
+    const BoxDesc bx = args.boxes[args.box_list[blockIdx.x / nsplit]];
     const int n = bx.n;
     const int NT = blockDim.x;
     const bool sym = bx.sym != 0;               // one row per pair: Y'_c
@@ -83,8 +112,9 @@ __global__ void __launch_bounds__(256, CPT == 1 ? 2 : 1) fold_kernel(FoldArgs ar
     T* CS = grams ? align_ptr<T>(sp, (size_t)RC * n) : nullptr;
     T* const Rglob = static_cast<T*>(args.Rws) + bx.R_off;
     T* const Rpack = args.R_in_smem ? align_ptr<T>(sp, (size_t)n * (n + 1) / 2) : nullptr;
-    T* GK = grams ? static_cast<T*>(args.GKws) + bx.R_off : nullptr;
-    T* GS = grams ? static_cast<T*>(args.GSws) + bx.R_off : nullptr;
+    // (each CTA of a split sums its own Grams; added up at the end)
+    T* GK = grams ? static_cast<T*>(args.GKws) + bx.R_off + rank * args.gram_stride : nullptr;
+    T* GS = grams ? static_cast<T*>(args.GSws) + bx.R_off + rank * args.gram_stride : nullptr;
 
     const double c0 = bx.ctr[0], c1 = bx.ctr[1], c2 = dim == 3 ? bx.ctr[2] : 0.0;
     // column data of this thread's columns
@@ -124,8 +154,108 @@ __global__ void __launch_bounds__(256, CPT == 1 ? 2 : 1) fold_kernel(FoldArgs ar
     const int* near = args.near + bx.near_off;
     const int npairs = bx.m_near + args.P;
     T c[CPT][RC];
-    for (int p0 = 0; p0 < npairs; p0 += ppc) {
-        const int np = min(ppc, npairs - p0);
+    // folds the chunk in c (rows below the first j0 of R) into R: Householder
+    // QR of [R; C], steps j0 ..
+    auto fold_chunk = [&](int j0) {
+        T rcur[CPT];
+#pragma unroll
+        for (int q = 0; q < CPT; ++q) {
+            const int l = threadIdx.x + q * NT;
+            rcur[q] = l < n && j0 <= l ? Rcol[q][j0 * rstride] : T(0);
+        }
+        for (int j = j0; j < n; ++j) {
+            const int buf = j & 1;
+            // the next step's R[j + 1][l], read a step ahead (only this thread writes it)
+            T rnext[CPT];
+#pragma unroll
+            for (int q = 0; q < CPT; ++q) {
+                const int l = threadIdx.x + q * NT;
+                rnext[q] = (l < n && j + 1 <= l) ? Rcol[q][(j + 1) * rstride] : T(0);
+            }
+            const int oq = j / NT;                   // the owner's slot
+            if (sizeof(T) == 8 && CPT == 1) {
+                // 64 bits: the owner's warp forms the reflector, row i on lane i
+                if (threadIdx.x / 32 == j / 32) {
+                    const int lane = threadIdx.x & 31;
+                    T* v = vbuf + buf * RC;
+                    if (lane == j % 32) {
+#pragma unroll
+                        for (int i = 0; i < RC; ++i) v[i] = c[0][i];
+                    }
+                    const T alpha = __shfl_sync(0xffffffffu, rcur[0], j % 32);
+                    __syncwarp();
+                    const T x = lane < RC ? v[lane] : T(0);
+                    const T ss = warp_sum(x * x);
+                    T tau = T(0), beta = alpha;
+                    if (ss != T(0)) {
+                        beta = -copysign(sqrt(alpha * alpha + ss), alpha);
+                        tau = (beta - alpha) / beta;
+                        const T scal = T(1) / (alpha - beta);
+                        if (lane < RC) v[lane] = x * scal;
+                    }
+                    if (lane == j % 32) {
+                        if (ss != T(0)) Rcol[0][j * rstride] = beta;
+                        taub[buf] = tau;
+                    }
+                }
+            } else if (threadIdx.x == j % NT) {
+#pragma unroll
+                for (int q = 0; q < CPT; ++q) {
+                    if (q != oq) continue;
+                    T q0 = T(0), q1 = T(0), q2 = T(0), q3 = T(0);
+#pragma unroll
+                    for (int i = 0; i < RC; i += 4) {
+                        q0 += c[q][i] * c[q][i];
+                        if (i + 1 < RC) q1 += c[q][i + 1] * c[q][i + 1];
+                        if (i + 2 < RC) q2 += c[q][i + 2] * c[q][i + 2];
+                        if (i + 3 < RC) q3 += c[q][i + 3] * c[q][i + 3];
+                    }
+                    const T ss = (q0 + q1) + (q2 + q3);
+                    T tau = T(0);
+                    if (ss != T(0)) {
+                        const T alpha = rcur[q];
+                        const T beta = -copysign(sqrt(alpha * alpha + ss), alpha);
+                        tau = (beta - alpha) / beta;
+                        const T scal = T(1) / (alpha - beta);
+                        Rcol[q][j * rstride] = beta;
+#pragma unroll
+                        for (int i = 0; i < RC; ++i) vbuf[buf * RC + i] = c[q][i] * scal;
+                    }
+                    taub[buf] = tau;
+                }
+            }
+            __syncthreads();
+            const T tau = taub[buf];
+            if (tau != T(0)) {
+                const T* v = vbuf + buf * RC;
+#pragma unroll
+                for (int q = 0; q < CPT; ++q) {
+                    const int l = threadIdx.x + q * NT;
+                    if (l > j && l < n) {
+                        T w0 = rcur[q], w1 = T(0), w2 = T(0), w3 = T(0);
+#pragma unroll
+                        for (int i = 0; i < RC; i += 4) {
+                            w0 += v[i] * c[q][i];
+                            if (i + 1 < RC) w1 += v[i + 1] * c[q][i + 1];
+                            if (i + 2 < RC) w2 += v[i + 2] * c[q][i + 2];
+                            if (i + 3 < RC) w3 += v[i + 3] * c[q][i + 3];
+                        }
+                        const T w = ((w0 + w1) + (w2 + w3)) * tau;
+                        Rcol[q][j * rstride] = rcur[q] - w;
+#pragma unroll
+                        for (int i = 0; i < RC; ++i) c[q][i] -= w * v[i];
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < CPT; ++q) rcur[q] = rnext[q];
+        }
+    };
+    const int nchunks = (npairs + ppc - 1) / ppc;
+    const int pbeg = (int)((int64_t)nchunks * rank / nsplit) * ppc;
+    const int pend = min(npairs, (int)((int64_t)nchunks * (rank + 1) / nsplit) * ppc);
+    for (int p0 = pbeg; p0 < pend; p0 += ppc) {
+        const int np = min(ppc, pend - p0);
         __syncthreads();                        // previous chunk's row data and Gram reads done
         for (int q = threadIdx.x; q < ppc; q += NT) {
             const int p = p0 + q;
@@ -204,72 +334,37 @@ __global__ void __launch_bounds__(256, CPT == 1 ? 2 : 1) fold_kernel(FoldArgs ar
                 }
             }
         }
-        // ---- fold the chunk into R: Householder QR of [R; C]
-        T rcur[CPT];
+        fold_chunk(0);
+    }
+    if (nsplit > 1) {
+        // the R factors folded together in pairs: rank 2 s q takes rank 2 s q + s
+        for (int s = 1; s < nsplit; s *= 2) {
+            fold_cluster_sync();
+            if (rank % (2 * s) != 0 || rank + s >= nsplit) continue;
+            const int l = threadIdx.x;
+            for (int i0 = 0; i0 < n; i0 += RC) {
 #pragma unroll
-        for (int q = 0; q < CPT; ++q) rcur[q] = threadIdx.x + q * NT < n ? Rcol[q][0] : T(0);
-        for (int j = 0; j < n; ++j) {
-            const int buf = j & 1;
-            // the next step's R[j + 1][l], read a step ahead (only this thread writes it)
-            T rnext[CPT];
-#pragma unroll
-            for (int q = 0; q < CPT; ++q) {
-                const int l = threadIdx.x + q * NT;
-                rnext[q] = (l < n && j + 1 <= l) ? Rcol[q][(j + 1) * rstride] : T(0);
+                for (int i = 0; i < RC; ++i)
+                    c[0][i] = l < n && i0 + i <= l ? ld_peer(Rcol[0] + i0 + i, rank + s) : T(0);
+                __syncthreads();                     // the previous chunk's last reflector has been read
+                fold_chunk(i0);
             }
-            const int oq = j / NT;                   // the owner's slot
-            if (threadIdx.x == j % NT) {
-#pragma unroll
-                for (int q = 0; q < CPT; ++q) {
-                    if (q != oq) continue;
-                    T q0 = T(0), q1 = T(0), q2 = T(0), q3 = T(0);
-#pragma unroll
-                    for (int i = 0; i < RC; i += 4) {
-                        q0 += c[q][i] * c[q][i];
-                        if (i + 1 < RC) q1 += c[q][i + 1] * c[q][i + 1];
-                        if (i + 2 < RC) q2 += c[q][i + 2] * c[q][i + 2];
-                        if (i + 3 < RC) q3 += c[q][i + 3] * c[q][i + 3];
-                    }
-                    const T ss = (q0 + q1) + (q2 + q3);
-                    T tau = T(0);
-                    if (ss != T(0)) {
-                        const T alpha = rcur[q];
-                        const T beta = -copysign(sqrt(alpha * alpha + ss), alpha);
-                        tau = (beta - alpha) / beta;
-                        const T scal = T(1) / (alpha - beta);
-                        Rcol[q][j * rstride] = beta;
-#pragma unroll
-                        for (int i = 0; i < RC; ++i) vbuf[buf * RC + i] = c[q][i] * scal;
-                    }
-                    taub[buf] = tau;
-                }
-            }
-            __syncthreads();
-            const T tau = taub[buf];
-            if (tau != T(0)) {
-                const T* v = vbuf + buf * RC;
-#pragma unroll
-                for (int q = 0; q < CPT; ++q) {
-                    const int l = threadIdx.x + q * NT;
-                    if (l > j && l < n) {
-                        T w0 = rcur[q], w1 = T(0), w2 = T(0), w3 = T(0);
-#pragma unroll
-                        for (int i = 0; i < RC; i += 4) {
-                            w0 += v[i] * c[q][i];
-                            if (i + 1 < RC) w1 += v[i + 1] * c[q][i + 1];
-                            if (i + 2 < RC) w2 += v[i + 2] * c[q][i + 2];
-                            if (i + 3 < RC) w3 += v[i + 3] * c[q][i + 3];
-                        }
-                        const T w = ((w0 + w1) + (w2 + w3)) * tau;
-                        Rcol[q][j * rstride] = rcur[q] - w;
-#pragma unroll
-                        for (int i = 0; i < RC; ++i) c[q][i] -= w * v[i];
-                    }
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < CPT; ++q) rcur[q] = rnext[q];
         }
+        fold_cluster_sync();                         // no CTA leaves while its R or Grams are read
+        if (grams)
+            for (int e = rank * NT + threadIdx.x; e < n * n; e += nsplit * NT) {
+                if (e / n + e % n >= n) continue;    // diagonal-major: (t, l), l + t < n
+                T* gk = static_cast<T*>(args.GKws) + bx.R_off + e;
+                T* gs = static_cast<T*>(args.GSws) + bx.R_off + e;
+                T k = gk[0], v = gs[0];
+                for (int q = 1; q < nsplit; ++q) {
+                    k += gk[q * args.gram_stride];
+                    v += gs[q * args.gram_stride];
+                }
+                gk[0] = k;
+                gs[0] = v;
+            }
+        if (rank != 0) return;
     }
     if (args.R_in_smem)
 #pragma unroll
@@ -861,9 +956,39 @@ static cudaError_t launch_fold_cfg(const FoldArgs& a, int nbox, int threads, siz
     cudaError_t e = cudaFuncSetAttribute(fold_kernel<T, RC, CPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(nbox * a.split));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)a.split;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = a.split > 1 ? 1 : 0;
     note_launch();
-    fold_kernel<T, RC, CPT><<<nbox, threads, smem, st>>>(a);
-    return cudaGetLastError();
+    return cudaLaunchKernelEx(&cfg, fold_kernel<T, RC, CPT>, a);
+}
+
+// CTAs per box for `count` boxes of up to n columns and `chunks` row chunks
+// each: the split of the smallest steps x waves, steps = a CTA's share of the
+// chunks and the merges of a triangle into another, waves of one 256-thread
+// CTA per SM (two in 32 bits).  A split has to save a tenth at least.
+int fold_split(int n, int64_t chunks, int count, int num_sms, int elem) {
+    const int64_t per_wave = (int64_t)num_sms * (elem == 8 ? 1 : 2) * std::max(1, 256 / std::max(n, 32));
+    int best = 1;
+    double cost1 = 0.0, least = 0.0;
+    for (int s = 1; s <= 8; s *= 2) {
+        const double steps = (double)((chunks + s - 1) / s) * n + (double)(s == 8 ? 3 : s / 2) * n * n / 64.0;
+        const double cost = steps * std::ceil((double)count * s / per_wave);
+        if (s == 1) cost1 = least = cost;
+        if (cost < least && cost < 0.9 * cost1) {
+            least = cost;
+            best = s;
+        }
+    }
+    return best;
 }
 
 // threads: the launch's largest box width rounded up to a warp (<= 256) for
@@ -871,7 +996,9 @@ static cudaError_t launch_fold_cfg(const FoldArgs& a, int nbox, int threads, siz
 template <typename T>
 cudaError_t launch_fold(const FoldArgs& a, int nbox, int threads, int cpt, size_t smem, cudaStream_t st, int rc) {
     if (nbox == 0) return cudaSuccess;
-    if (threads < 32 || threads > 256 || threads % 32) return cudaErrorInvalidValue;
+    if (threads < 32 || threads > 256 || threads % 32 || a.split < 1 || a.split > 8 ||
+        (a.split > 1 && (cpt != 1 || !a.R_in_smem)))
+        return cudaErrorInvalidValue;
     if (cpt == 1 && rc == 16) return launch_fold_cfg<T, 16, 1>(a, nbox, threads, smem, st);
     if constexpr (sizeof(T) == 4) {
         if (cpt == 1) return launch_fold_cfg<T, 32, 1>(a, nbox, threads, smem, st);

@@ -22,6 +22,8 @@ struct FoldArgs {
     int bpairs;
     int second_kind;
     int R_in_smem;
+    int split;                // CTAs (a cluster) per box, 1, 2, 4 or 8
+    int64_t gram_stride;      // between the Grams of the CTAs of a split
     void* Rws;
     void* GKws;
     void* GSws;
@@ -226,6 +228,7 @@ template <typename T> cudaError_t launch_r_colmajor(const void* R, int n, void* 
 
 // columns per thread of the fold kernel for a box of n columns (0: too wide)
 int fold_cpt(int n, int elem);
+int fold_split(int n, int64_t chunks, int count, int num_sms, int elem);
 template <typename T>
 cudaError_t launch_fold(const FoldArgs&, int nbox, int threads, int cpt, size_t smem, cudaStream_t, int rc = 0);
 template <typename T> cudaError_t launch_id(const IdArgs&, int ngroups, size_t smem, int num_sms, cudaStream_t);
