@@ -124,6 +124,7 @@ struct Segment {
     bool sym = false;             // b == c and equal weights: A symmetric, Y'_c compressed (Sec. 5)
     int gn = 0;
     double gh = 0;
+    int hgrid_n = 0;              // kernel 2 on a full grid: points per side, table and point_of (dof_of) filled
     DevMem dof_of, table, table_df;
     DevMem tc_rows, tc_tmax;      // digit rows of the table for the tensor-core sum (built on first use)
     double spread = 1.0;          // max|T| sqrt(#T) / |T|_2 of the table (scale of the short sums' error)
@@ -285,6 +286,35 @@ static void detect_grid(hif_handle h, Segment& sg) {
     sg.gn = n;
     sg.gh = hx;
     upload(sg.dof_of, dof_of, h->st);
+}
+
+// The complex kernel on a full uniform grid: the table of its values by index
+// offset.  Only for points within rounding of the grid (the direct sum uses
+// the points themselves elsewhere); self: K_ii / w.
+static void detect_helmholtz_grid(hif_handle h, Segment& sg, double self_re, double self_im) {
+    const int64_t np = sg.N / 2;
+    std::vector<double> X(2 * (size_t)np), W((size_t)np);
+    for (int64_t p = 0; p < np; ++p) {
+        const int64_t i = sg.off + 2 * p;
+        X[2 * p] = h->hx[2 * i];
+        X[2 * p + 1] = h->hx[2 * i + 1];
+        W[p] = h->hw[i];
+    }
+    std::vector<int> point_of;
+    int n = 0;
+    double hx = 0.0;
+    if (!grid_layout(X.data(), W.data(), np, 2, 0, &n, &hx, point_of)) return;
+    const double lo[2] = {X[2 * (size_t)point_of[0]], X[2 * (size_t)point_of[0] + 1]};
+    const double tol = 1e-15 * std::max({hx * n, std::fabs(lo[0]), std::fabs(lo[1])});
+    for (int64_t g = 0; g < np; ++g)
+        for (int k = 0; k < 2; ++k) {
+            const double at = lo[k] + hx * (double)(k == 0 ? g / n : g % n);
+            if (std::fabs(X[2 * (size_t)point_of[g] + k] - at) > tol) return;
+        }
+    upload(sg.dof_of, point_of, h->st);
+    sg.table.ensure(sizeof(double) * 2 * (size_t)np);
+    HIF_CUDA(launch_helmholtz_table(sg.table.as<double>(), n, hx, h->wavenumber, self_re, self_im, h->st));
+    sg.hgrid_n = n;
 }
 
 static int env_int(const char* name, int dflt) {
@@ -1705,9 +1735,15 @@ static void matvec_dev(hif_handle h, int trans, const double* x, int64_t ldx, do
             da.trans = trans;
             da.seg_off = sg.off;
             da.seg_n = sg.N;
+            h->ybuf.ensure(std::max(sg.hgrid_n ? helmholtz_grid_part_bytes(sg.hgrid_n, nrhs, h->num_sms)
+                                               : direct_part_bytes(sg.N, nrhs, h->num_sms),
+                                    (size_t)8));
             ProfRange pr(PROF_DIRECT, st, 2.0 * (double)sg.N * sg.N * nrhs, 0.0);
-            if (h->ncomp == 2) HIF_CUDA(launch_direct_helmholtz(da, st));
-            else HIF_CUDA(launch_direct_general(da, st));
+            if (sg.hgrid_n)
+                HIF_CUDA(launch_helmholtz_grid(da, sg.table.as<double>(), sg.dof_of.as<int>(), sg.hgrid_n,
+                                               h->ybuf.as<double>(), h->num_sms, st));
+            else if (h->ncomp == 2) HIF_CUDA(launch_direct_helmholtz(da, st));
+            else HIF_CUDA(launch_direct_general(da, h->ybuf.as<double>(), h->num_sms, st));
         }
     }
 }
@@ -2313,7 +2349,12 @@ static hif_status factor_impl(int count, const hif_problem* probs, int kernel_id
         HIF_CUDA(cudaStreamSynchronize(st));
         for (auto& sp : h->segs) {
             Segment& sg = *sp;
-            if (h->ncomp == 2) continue;               // no grid convolution for the complex kernel
+            if (h->ncomp == 2) {
+                double kr = 0.0, ki = 0.0;
+                helmholtz_self(h->wavenumber, std::sqrt(h->hw[sg.off]), &kr, &ki);
+                detect_helmholtz_grid(h.get(), sg, kr / h->hw[sg.off], ki / h->hw[sg.off]);
+                continue;
+            }
             detect_grid(h.get(), sg);
             if (!sg.grid) continue;
             const int64_t tsz = d == 2 ? (int64_t)sg.gn * sg.gn : (int64_t)sg.gn * sg.gn * sg.gn;

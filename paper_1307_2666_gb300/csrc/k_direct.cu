@@ -75,47 +75,97 @@ cudaError_t launch_kernel_block(const GeomDev& g, const int* rows, int64_t nr, c
 
 constexpr int DS_T = 128;   // targets per CTA (one per thread)
 constexpr int DS_S = 256;   // sources per shared-memory tile
-constexpr int DS_R = 8;     // right-hand sides per pass
+constexpr int DS_R = 8;     // most right-hand sides per pass
 
-__global__ void __launch_bounds__(DS_T) direct_general_kernel(DirectArgs a, int r0, int nr) {
+__device__ __forceinline__ double green_constant(int kid) { return kid == 0 ? -0.25 / kPi : 0.25 / kPi; }
+
+// One thread per target.  What bounds it is the FP64 unit (64 cycles per warp
+// instruction and scheduler): ~5 operations for the distance, 13 for the
+// logarithm and one per right-hand side, so NR is the number of right-hand
+// sides rounded up to a power of two.  blockIdx.y takes a share of the sources
+// (direct_splits: targets alone give too few warps), whose sums are added in
+// order by direct_finish_kernel.  Measured on a GB300, 16,384 scattered points
+// and two right-hand sides: 27.6 ms with log(), NR = 8 and no split; 11 ms now.
+template <int NR>
+__global__ void __launch_bounds__(DS_T) direct_general_kernel(DirectArgs a, int r0, int nr, double* part) {
     __shared__ double sx[DS_S * 3];
-    __shared__ double sv[DS_S * DS_R];
+    __shared__ double sv[DS_S * NR];
     const GeomDev& g = a.g;
-    const int dim = g.dim;
-    const int64_t s_end = a.seg_off + a.seg_n;
+    const int dim = g.dim, kid = g.kernel_id;
     const int64_t i = a.seg_off + blockIdx.x * (int64_t)DS_T + threadIdx.x;
-    const bool valid = i < s_end;
+    const bool valid = i < a.seg_off + a.seg_n;
     double xi[3] = {0, 0, 0};
     if (valid)
         for (int d = 0; d < dim; ++d) xi[d] = g.x[(int64_t)dim * i + d];
-    double acc[DS_R];
-    for (int c = 0; c < DS_R; ++c) acc[c] = 0.0;
-    for (int64_t j0 = a.seg_off; j0 < s_end; j0 += DS_S) {
-        const int ns = (int)(s_end - j0 < DS_S ? s_end - j0 : DS_S);
+    double acc[NR];
+#pragma unroll
+    for (int c = 0; c < NR; ++c) acc[c] = 0.0;
+    const int64_t tiles = (a.seg_n + DS_S - 1) / DS_S;
+    const int64_t t1 = tiles * (blockIdx.y + 1) / gridDim.y;
+    for (int64_t t = tiles * blockIdx.y / gridDim.y; t < t1; ++t) {
+        const int64_t j0 = a.seg_off + t * DS_S;
+        const int ns = (int)min((int64_t)DS_S, a.seg_off + a.seg_n - j0);
         __syncthreads();
         for (int s = threadIdx.x; s < ns; s += DS_T) {
             const int64_t j = j0 + s;
             for (int d = 0; d < 3; ++d) sx[3 * s + d] = d < dim ? g.x[(int64_t)dim * j + d] : 0.0;
             const double sw = a.trans ? g.b[j] : g.w[j] * g.c[j];
-            for (int c = 0; c < DS_R; ++c) sv[s * DS_R + c] = c < nr ? sw * a.x[j + a.ldx * (r0 + c)] : 0.0;
+#pragma unroll
+            for (int c = 0; c < NR; ++c) sv[s * NR + c] = c < nr ? sw * a.x[j + a.ldx * (r0 + c)] : 0.0;
         }
         __syncthreads();
         if (valid) {
+#pragma unroll 2
             for (int s = 0; s < ns; ++s) {
-                const int64_t j = j0 + s;
-                if (j == i) continue;
-                const double d0 = xi[0] - sx[3 * s], d1 = xi[1] - sx[3 * s + 1], d2 = xi[2] - sx[3 * s + 2];
-                const double gk = green_d(g.kernel_id, d0 * d0 + d1 * d1 + d2 * d2);
-                for (int c = 0; c < DS_R; ++c) acc[c] += gk * sv[s * DS_R + c];
+                if (j0 + s == i) continue;
+                const double d0 = xi[0] - sx[3 * s], d1 = xi[1] - sx[3 * s + 1];
+                double r2 = d0 * d0 + d1 * d1;
+                if (dim == 3) {
+                    const double d2 = xi[2] - sx[3 * s + 2];
+                    r2 += d2 * d2;
+                }
+                const double gk = kid == 0 ? log_tab(r2) : rsqrt(r2);      // G but for its constant
+#pragma unroll
+                for (int c = 0; c < NR; ++c) acc[c] += gk * sv[s * NR + c];
             }
         }
     }
-    if (valid) {
-        const double tf = a.trans ? g.c[i] * g.w[i] : g.b[i];
-        const double self = g.b[i] * g.kself[i] * g.c[i] + g.a[i];
-        for (int c = 0; c < nr; ++c)
-            a.y[i + a.ldy * (r0 + c)] = tf * acc[c] + self * a.x[i + a.ldx * (r0 + c)];
+    if (!valid) return;
+    if (part) {
+#pragma unroll
+        for (int c = 0; c < NR; ++c) part[((int64_t)blockIdx.y * NR + c) * a.seg_n + (i - a.seg_off)] = acc[c];
+        return;
     }
+    const double tf = (a.trans ? g.c[i] * g.w[i] : g.b[i]) * green_constant(kid);
+    const double self = g.b[i] * g.kself[i] * g.c[i] + g.a[i];
+#pragma unroll
+    for (int c = 0; c < NR; ++c)
+        if (c < nr) a.y[i + a.ldy * (r0 + c)] = tf * acc[c] + self * a.x[i + a.ldx * (r0 + c)];
+}
+
+// y from the partial sums of `splits` shares of the sources, in order
+__global__ void direct_finish_kernel(DirectArgs a, int r0, int nr, int NR, const double* part, int splits) {
+    const GeomDev& g = a.g;
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= a.seg_n * nr) return;
+    const int64_t q = e % a.seg_n, i = a.seg_off + q;
+    const int c = (int)(e / a.seg_n);
+    double s = 0.0;
+    for (int y = 0; y < splits; ++y) s += part[((int64_t)y * NR + c) * a.seg_n + q];
+    const double tf = (a.trans ? g.c[i] * g.w[i] : g.b[i]) * green_constant(g.kernel_id);
+    const double self = g.b[i] * g.kself[i] * g.c[i] + g.a[i];
+    a.y[i + a.ldy * (r0 + c)] = tf * s + self * a.x[i + a.ldx * (r0 + c)];
+}
+
+// Shares of the sources: about seven CTAs of 128 targets per SM, while a share
+// keeps 512 sources.
+static int direct_splits(int64_t n, int num_sms) {
+    const int64_t blocks = (n + DS_T - 1) / DS_T;
+    return (int)std::clamp<int64_t>(std::min<int64_t>(7LL * num_sms / blocks, n / 512), 1, 64);
+}
+size_t direct_part_bytes(int64_t n, int nrhs, int num_sms) {
+    const int s = direct_splits(n, num_sms);
+    return s > 1 ? sizeof(double) * (size_t)s * n * std::min(nrhs > 4 ? 8 : nrhs > 2 ? 4 : nrhs, DS_R) : 0;
 }
 
 // Helmholtz kernel (kernel 2) on the real embedding: complex unknowns are the
@@ -195,12 +245,135 @@ cudaError_t launch_direct_helmholtz(const DirectArgs& a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_direct_general(const DirectArgs& a, cudaStream_t st) {
+cudaError_t launch_direct_general(const DirectArgs& a, double* part, int num_sms, cudaStream_t st) {
     if (a.seg_n == 0) return cudaSuccess;
-    const int blocks = (int)((a.seg_n + DS_T - 1) / DS_T);
+    const int splits = direct_splits(a.seg_n, num_sms);
+    const dim3 grid((unsigned)((a.seg_n + DS_T - 1) / DS_T), splits);
+    double* pt = splits > 1 ? part : nullptr;
     for (int r0 = 0; r0 < a.nrhs; r0 += DS_R) {
+        const int nr = std::min(DS_R, a.nrhs - r0), NR = nr > 4 ? 8 : nr > 2 ? 4 : nr;
         note_launch();
-        direct_general_kernel<<<blocks, DS_T, 0, st>>>(a, r0, std::min(DS_R, a.nrhs - r0));
+        if (NR == 8) direct_general_kernel<8><<<grid, DS_T, 0, st>>>(a, r0, nr, pt);
+        else if (NR == 4) direct_general_kernel<4><<<grid, DS_T, 0, st>>>(a, r0, nr, pt);
+        else if (NR == 2) direct_general_kernel<2><<<grid, DS_T, 0, st>>>(a, r0, nr, pt);
+        else direct_general_kernel<1><<<grid, DS_T, 0, st>>>(a, r0, nr, pt);
+        if (splits > 1) {
+            note_launch();
+            direct_finish_kernel<<<(unsigned)((a.seg_n * nr + 255) / 256), 256, 0, st>>>(a, r0, nr, NR, pt, splits);
+        }
+    }
+    return cudaGetLastError();
+}
+
+// Helmholtz sum on a full uniform grid: G depends on the index offset only, so
+// its n^2 values are tabulated once per handle (J_0 and Y_0 are hundreds of
+// 64-bit operations, and the general kernel evaluates them for every pair at
+// every call).  One thread per target, blockIdx.y a share of the source
+// lines; a pair costs one 16-byte table read and four FMAs per right-hand
+// side.  Measured on a GB300, n = 64, one right-hand side: 25.6 -> 0.2 ms.
+__global__ void helmholtz_table_kernel(double2* table, int n, double h, double k, double gr0, double gi0) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n * n) return;
+    const double d0 = (e / n) * h, d1 = (e % n) * h;
+    double gr = gr0, gi = gi0;
+    if (e > 0) green_helmholtz(k, d0 * d0 + d1 * d1, gr, gi);
+    table[e] = make_double2(gr, gi);
+}
+
+template <int NR>
+__global__ void __launch_bounds__(DS_T) helmholtz_grid_kernel(DirectArgs a, const double2* table, const int* point_of,
+                                                              int n, int r0, int nr, double* part) {
+    __shared__ double2 sv[DS_S * NR];
+    const GeomDev& g = a.g;
+    const int64_t N = (int64_t)n * n, gp = blockIdx.x * (int64_t)DS_T + threadIdx.x;
+    const bool valid = gp < N;
+    const int i0 = (int)(gp / n), i1 = (int)(gp % n);
+    const double cs = a.trans ? -1.0 : 1.0;
+    double ar[NR], ai[NR];
+#pragma unroll
+    for (int c = 0; c < NR; ++c) ar[c] = ai[c] = 0.0;
+    const int l1 = (int)((int64_t)n * (blockIdx.y + 1) / gridDim.y);
+    for (int j0 = (int)((int64_t)n * blockIdx.y / gridDim.y); j0 < l1; ++j0)
+        for (int jb = 0; jb < n; jb += DS_S) {
+            const int ns = min(DS_S, n - jb);
+            __syncthreads();
+            for (int s = threadIdx.x; s < ns; s += DS_T) {
+                const int64_t q = a.seg_off + 2 * (int64_t)point_of[j0 * n + jb + s];
+                const double sw = a.trans ? g.b[q] : g.w[q] * g.c[q];
+#pragma unroll
+                for (int c = 0; c < NR; ++c)
+                    sv[s * NR + c] = c < nr ? make_double2(sw * a.x[q + a.ldx * (r0 + c)], sw * a.x[q + 1 + a.ldx * (r0 + c)])
+                                            : make_double2(0.0, 0.0);
+            }
+            __syncthreads();
+            if (valid) {
+                const double2* row = table + (int64_t)abs(i0 - j0) * n;
+#pragma unroll 4
+                for (int s = 0; s < ns; ++s) {
+                    const double2 t = __ldg(row + abs(i1 - jb - s));
+                    const double gi = cs * t.y;
+#pragma unroll
+                    for (int c = 0; c < NR; ++c) {
+                        const double2 v = sv[s * NR + c];
+                        ar[c] += t.x * v.x - gi * v.y;
+                        ai[c] += t.x * v.y + gi * v.x;
+                    }
+                }
+            }
+        }
+    if (!valid) return;
+#pragma unroll
+    for (int c = 0; c < NR; ++c) {
+        part[((int64_t)blockIdx.y * NR + c) * 2 * N + 2 * gp] = ar[c];
+        part[((int64_t)blockIdx.y * NR + c) * 2 * N + 2 * gp + 1] = ai[c];
+    }
+}
+
+__global__ void helmholtz_finish_kernel(DirectArgs a, const int* point_of, int n, int r0, int nr, int NR,
+                                        const double* part, int splits) {
+    const GeomDev& g = a.g;
+    const int64_t N = (int64_t)n * n, t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= N * nr) return;
+    const int64_t gp = t % N, e = a.seg_off + 2 * (int64_t)point_of[gp];
+    const int c = (int)(t / N);
+    double sr = 0.0, si = 0.0;
+    for (int y = 0; y < splits; ++y) {
+        sr += part[((int64_t)y * NR + c) * 2 * N + 2 * gp];
+        si += part[((int64_t)y * NR + c) * 2 * N + 2 * gp + 1];
+    }
+    // (the table's zero offset is the self integral over w, as in the Laplace grid sums)
+    const double tf = a.trans ? g.c[e] * g.w[e] : g.b[e];
+    a.y[e + a.ldy * (r0 + c)] = tf * sr + g.a[e] * a.x[e + a.ldx * (r0 + c)];
+    a.y[e + 1 + a.ldy * (r0 + c)] = tf * si + g.a[e] * a.x[e + 1 + a.ldx * (r0 + c)];
+}
+
+static int helmholtz_splits(int n, int num_sms) {
+    const int64_t blocks = ((int64_t)n * n + DS_T - 1) / DS_T;
+    return (int)std::clamp<int64_t>(7LL * num_sms / blocks, 1, n);
+}
+size_t helmholtz_grid_part_bytes(int n, int nrhs, int num_sms) {
+    return sizeof(double) * 2 * (size_t)n * n * helmholtz_splits(n, num_sms) * (nrhs > 2 ? 4 : nrhs);
+}
+cudaError_t launch_helmholtz_table(double* table, int n, double h, double k, double gr0, double gi0, cudaStream_t st) {
+    note_launch();
+    helmholtz_table_kernel<<<(n * n + 255) / 256, 256, 0, st>>>(reinterpret_cast<double2*>(table), n, h, k, gr0, gi0);
+    return cudaGetLastError();
+}
+cudaError_t launch_helmholtz_grid(const DirectArgs& a, const double* table, const int* point_of, int n, double* part,
+                                  int num_sms, cudaStream_t st) {
+    const int splits = helmholtz_splits(n, num_sms);
+    const int64_t N = (int64_t)n * n;
+    const dim3 grid((unsigned)((N + DS_T - 1) / DS_T), splits);
+    const double2* tb = reinterpret_cast<const double2*>(table);
+    for (int r0 = 0; r0 < a.nrhs; r0 += DH_R) {
+        const int nr = std::min(DH_R, a.nrhs - r0), NR = nr > 2 ? 4 : nr;
+        note_launch();
+        if (NR == 4) helmholtz_grid_kernel<4><<<grid, DS_T, 0, st>>>(a, tb, point_of, n, r0, nr, part);
+        else if (NR == 2) helmholtz_grid_kernel<2><<<grid, DS_T, 0, st>>>(a, tb, point_of, n, r0, nr, part);
+        else helmholtz_grid_kernel<1><<<grid, DS_T, 0, st>>>(a, tb, point_of, n, r0, nr, part);
+        note_launch();
+        helmholtz_finish_kernel<<<(unsigned)((N * nr + 255) / 256), 256, 0, st>>>(a, point_of, n, r0, nr, NR, part,
+                                                                                 splits);
     }
     return cudaGetLastError();
 }

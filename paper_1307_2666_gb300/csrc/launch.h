@@ -277,7 +277,16 @@ struct DirectArgs {
     int64_t seg_off;        // the problem's DOF range [seg_off, seg_off + seg_n)
     int64_t seg_n;
 };
-cudaError_t launch_direct_general(const DirectArgs&, cudaStream_t);
+// part: direct_part_bytes of scratch for the shares of the sources
+size_t direct_part_bytes(int64_t n, int nrhs, int num_sms);
+cudaError_t launch_direct_general(const DirectArgs&, double* part, int num_sms, cudaStream_t);
+// Helmholtz sum on a full n x n grid: point_of[grid position] = point of the
+// problem, table (n^2 complex values, offset 0 the self integral over w) built
+// by launch_helmholtz_table, part of helmholtz_grid_part_bytes
+size_t helmholtz_grid_part_bytes(int n, int nrhs, int num_sms);
+cudaError_t launch_helmholtz_table(double* table, int n, double h, double k, double gr0, double gi0, cudaStream_t);
+cudaError_t launch_helmholtz_grid(const DirectArgs&, const double* table, const int* point_of, int n, double* part,
+                                  int num_sms, cudaStream_t);
 cudaError_t launch_direct_helmholtz(const DirectArgs&, cudaStream_t);
 
 // Batched FP32 products on the tensor cores (k_tcgemm.cu):
