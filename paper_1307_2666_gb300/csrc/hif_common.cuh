@@ -5,15 +5,14 @@
 #include <cuda_runtime.h>
 
 #include "hif_types.h"
-#include "log_tab.cuh"
 
 namespace hif {
 
 // ---------------------------------------------------------------- kernels --
 
-__device__ inline double green_d(int kernel_id, double r2) {
+__host__ __device__ inline double green_d(int kernel_id, double r2) {
     // G of Eq. (1.4) from the squared distance: -log(r)/(2 pi) = -log(r^2)/(4 pi)
-    return kernel_id == 0 ? -log_tab(r2) * (0.25 / kPi) : (0.25 / kPi) * rsqrt(r2);
+    return kernel_id == 0 ? -log(r2) * (0.25 / kPi) : (0.25 / kPi) / sqrt(r2);
 }
 
 __device__ inline float green_f(int kernel_id, float r2) {

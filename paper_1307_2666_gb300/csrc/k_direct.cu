@@ -14,6 +14,7 @@
 
 #include "hif_common.cuh"
 #include "launch.h"
+#include "log_tab.cuh"
 
 namespace hif {
 
