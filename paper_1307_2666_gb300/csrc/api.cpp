@@ -331,8 +331,8 @@ struct BigBuffers {
 // The column-pivoted QR of all large groups of a sublevel: by panels of
 // HIF_BIG_QP_NB pivots (blocked, one trailing product per panel) or, at 1,
 // one launch pair per pivot.  Default: panels of 32 in FP32; one pivot per
-// step in FP64, whose exact norms at every step keep the rank decisions of
-// the symmetric and full proxy matrices identical at eps = 1e-9 (the blocked
+// step in FP64, whose norms (kNormKeep) keep the rank decisions of the
+// symmetric and full proxy matrices identical at eps = 1e-9 (the blocked
 // update's rounding moved one decision at the threshold by one).
 template <typename T>
 static void run_big_pivoted_qr(BigArgs& a, BigBuffers& B, const std::vector<BigGroup>& bgv, int max_n, int maxk,
@@ -345,14 +345,12 @@ static void run_big_pivoted_qr(BigArgs& a, BigBuffers& B, const std::vector<BigG
     if (nbq > 1) {
         B.F.ensure(sizeof(T) * std::max<int64_t>(voff, 1) * nbq);
         B.gv.ensure(sizeof(T) * 32 * std::max(ng, 1));
-        B.nrm0.ensure(sizeof(double) * std::max<int64_t>(voff, 1));
         a.F = B.F.p;
         a.gv = B.gv.p;
-        a.nrm0 = B.nrm0.as<double>();
         a.nb = nbq;
-    } else {
-        a.nrm0 = nullptr;
     }
+    B.nrm0.ensure(sizeof(double) * std::max<int64_t>(voff, 1));
+    a.nrm0 = B.nrm0.as<double>();
     HIF_CUDA((big_qr_init<T>(a, ng, max_n, st)));
     if (nbq > 1) {
         int step = 0;

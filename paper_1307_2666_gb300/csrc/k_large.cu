@@ -9,8 +9,8 @@
 //  * big_step /      column-pivoted Householder QR (Lemma 2.2), one pair of
 //    big_update      launches per pivot step for all large groups at once: one
 //                    CTA per group picks the pivot and forms the reflector, a
-//                    warp per remaining column applies it and recomputes the
-//                    column norm in FP64;
+//                    warp per remaining column applies it and brings the
+//                    column norm up to date in FP64 (kNormKeep);
 //  * big_T           T = R1^{-1} R2 and the skeleton / redundant order;
 //  * gemm / trsm / elimination helpers: Lemma 2.4 blocks, Lemma 2.1 LU
 //                    (blocked, multi-CTA) and the Schur update for one large
@@ -215,23 +215,26 @@ __global__ void big_norm_init_kernel(BigArgs a) {
     s = warp_sum(s);
     if (lane == 0) {
         a.nrm[G.vec_off + l] = s;
-        if (a.nrm0) a.nrm0[G.vec_off + l] = s;
+        a.nrm0[G.vec_off + l] = s;
         a.perm[G.vec_off + l] = l;
     }
 }
 
+constexpr int BST = 256;   // threads of the step kernel: one CTA walks the pivot column of m rows
+
 template <typename T>
-__global__ void __launch_bounds__(256) big_step_kernel(BigArgs a, int j) {
+__global__ void __launch_bounds__(BST) big_step_kernel(BigArgs a, int j) {
     const BigGroup G = a.groups[blockIdx.x];
     BigState* S = a.state + blockIdx.x;
     if (S->stop) return;
     T* W = static_cast<T*>(a.YK) + G.y_off;
     const int64_t ld = G.ld;
     double* nrm = a.nrm + G.vec_off;
+    double* nrm0 = a.nrm0 + G.vec_off;
     int* perm = a.perm + G.vec_off;
-    __shared__ double redv[256];
-    __shared__ int redi[256];
-    __shared__ T hs[256];
+    __shared__ double redv[BST];
+    __shared__ int redi[BST];
+    __shared__ T hs[BST];
     const int kmax = min(G.m, G.n);
     if (j >= kmax) {
         if (threadIdx.x == 0) S->stop = 1;
@@ -278,7 +281,8 @@ __global__ void __launch_bounds__(256) big_step_kernel(BigArgs a, int j) {
     __syncthreads();
     if (threadIdx.x == 0 && p != j) {
         const int t = perm[j]; perm[j] = perm[p]; perm[p] = t;
-        const double tn = nrm[j]; nrm[j] = nrm[p]; nrm[p] = tn;
+        double tn = nrm[j]; nrm[j] = nrm[p]; nrm[p] = tn;
+        tn = nrm0[j]; nrm0[j] = nrm0[p]; nrm0[p] = tn;
     }
     // reflector for W[j:, j]
     T s = T(0);
@@ -333,30 +337,25 @@ __global__ void __launch_bounds__(256) big_update_kernel(BigArgs a, int j) {
         __syncwarp();
         if (lane == 0) col[j] -= w;
     }
-    double s = 0.0;
-    if constexpr (sizeof(T) == 4) {
-        // FP32 factorization: the update and the new norm in one pass, each
-        // lane's share of the norm summed in FP32 (its ~m/32 squares are FP32
-        // data) and the lanes in FP64 -- a warp-wide FP64 FMA in the loop
-        // would bind the step to the FP64 pipe
-        float sf = 0.f;
-        for (int i = j + 1 + lane; i < G.m; i += 32) {
-            const float c = tau != T(0) ? col[i] - w * v[i] : col[i];
-            if (tau != T(0)) col[i] = c;
-            sf = fmaf(c, c, sf);
-        }
-        s = (double)sf;
-    } else {
-        if (tau != T(0))
-            for (int i = j + 1 + lane; i < G.m; i += 32) col[i] -= w * v[i];
-        // FP64: the new norm in its own pass
+    if (tau != T(0))
+        for (int i = j + 1 + lane; i < G.m; i += 32) col[i] -= w * v[i];
+    // the square of the new norm (see kNormKeep)
+    double* nrm = a.nrm + G.vec_off + l;
+    double* nrm0 = a.nrm0 + G.vec_off + l;
+    __syncwarp();
+    const double rj = (double)col[j];
+    double s = fmax(*nrm - rj * rj, 0.0);
+    __syncwarp();
+    if (!(s >= kNormKeep * *nrm0)) {
+        s = 0.0;
         for (int i = j + 1 + lane; i < G.m; i += 32) {
             const double c = (double)col[i];
             s += c * c;
         }
+        s = warp_sum(s);
+        if (lane == 0) *nrm0 = s;
     }
-    s = warp_sum(s);
-    if (lane == 0) a.nrm[G.vec_off + l] = s;
+    if (lane == 0) *nrm = s;
 }
 
 // ---------------------------------------- blocked pivoted QR (panels) ----
@@ -765,7 +764,7 @@ cudaError_t big_qr_init(const BigArgs& a, int ngroups, int max_n, cudaStream_t s
 template <typename T>
 cudaError_t big_qr_step(const BigArgs& a, int ngroups, int max_n, int j, cudaStream_t st) {
     note_launch();
-    big_step_kernel<T><<<ngroups, 256, 0, st>>>(a, j);
+    big_step_kernel<T><<<ngroups, BST, 0, st>>>(a, j);
     const int cols = max_n - j - 1;
     if (cols > 0) {
         dim3 g((cols + 7) / 8, ngroups);
