@@ -587,7 +587,9 @@ static void launch_elims(hif_handle h, SubFactor& sf, const std::vector<ElimDesc
     // line moves the totals by less than 2%.
     const bool tc_gemm = env_int("HIF_TC_GEMM", 0) != 0;
     const int mid_n = tc_gemm ? 1 << 30 : env_int("HIF_ELIM_MID", 96);
-    const int be_max_r = be_factor_max_r<T>();
+    // (HIF_ELIM_CLUSTER_R: a lower line between the cluster's shared memory and
+    // the panels, for tests)
+    const int be_max_r = std::min(be_factor_max_r<T>(), std::max(1, env_int("HIF_ELIM_CLUSTER_R", 1 << 30)));
     std::vector<ElimDesc> batch;
     std::vector<int> fail_idx, order;
     double work_batch = work[1], work_cta = work[0];

@@ -677,9 +677,16 @@ cudaError_t big_qp_panel(const BigArgs& a, int ngroups, int max_n, int max_m, in
     return cudaGetLastError();
 }
 
-// T = R1^{-1} R2 (redundant columns in ascending original order), outputs
+// T = R1^{-1} R2 (redundant columns in ascending original order), outputs.
+// One CTA per TW redundant columns, by blocks of 32 rows from the last: the
+// products with the rows already solved, then the triangular block itself, a
+// column per lane.  (One thread per column read R1 row by row from global
+// memory: 3D n = 32, k ~ 900, 32-bit, 27.6 ms for the sublevels' large groups,
+// 0.8 now; n = 200, 64-bit, 14.6 and 3.4.)
+constexpr int TW = 8;
+
 template <typename T>
-__global__ void big_T_kernel(BigArgs a) {
+__global__ void __launch_bounds__(256) big_T_kernel(BigArgs a) {
     const BigGroup G = a.groups[blockIdx.y];
     const GroupDesc gd = a.gdesc[G.group];
     const int k = a.state[blockIdx.y].k;
@@ -689,21 +696,56 @@ __global__ void big_T_kernel(BigArgs a) {
     const int* perm = a.perm + G.vec_off;
     T* Tout = static_cast<T*>(a.Tws) + gd.T_off;
     int* pout = a.perm_out + gd.perm_off;
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.k_out[G.group] = k;
-    if (l < k) pout[l] = perm[l];
-    if (l >= r) return;
-    const int o = perm[k + l];
-    int pos = 0;
-    for (int q = 0; q < r; ++q) pos += perm[k + q] < o;
-    pout[k + pos] = o;
-    // back substitution in a local copy held in the T output column
-    T* tcol = Tout + (int64_t)k * pos;
-    const T* rcol = W + ld * (k + l);
-    for (int i = k - 1; i >= 0; --i) {
-        T v = rcol[i];
-        for (int q = i + 1; q < k; ++q) v -= W[i + ld * q] * tcol[q];
-        tcol[i] = v / W[i + ld * i];
+    const int t = threadIdx.x, l0 = blockIdx.x * TW;
+    if (l0 == 0 && t == 0) a.k_out[G.group] = k;
+    for (int l = l0 + t; l < min(l0 + TW, k); l += 256) pout[l] = perm[l];
+    if (l0 >= r) return;
+    __shared__ T Rs[32][33];
+    __shared__ T Xs[32][TW + 1];
+    __shared__ int pos[TW];
+    const int ti = t % 32, tj = t / 32, l = l0 + tj;          // one warp per column
+    {
+        const int o = l < r ? perm[k + l] : 0;
+        int c = 0;
+        for (int q = ti; l < r && q < r; q += 32) c += perm[k + q] < o;
+        for (int off = 16; off; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
+        if (ti == 0 && l < r) {
+            pos[tj] = c;
+            pout[k + c] = o;
+        }
+    }
+    __syncthreads();
+    T* tcol = l < r ? Tout + (int64_t)k * pos[tj] : nullptr;
+    const int nb = (k + 31) / 32;
+    for (int I = nb - 1; I >= 0; --I) {
+        const int gi = 32 * I + ti;
+        T acc = gi < k && l < r ? W[gi + ld * (k + l)] : T(0);
+        for (int K = nb - 1; K >= I; --K) {
+            __syncthreads();
+            for (int q = t; q < 1024; q += 256) {
+                const int i = q % 32, c = q / 32, ri = 32 * I + i, rc = 32 * K + c;
+                Rs[i][c] = ri < k && rc < k ? W[ri + ld * rc] : T(0);
+            }
+            const int gk = 32 * K + ti;
+            if (K > I) Xs[ti][tj] = gk < k && l < r ? tcol[gk] : T(0);
+            __syncthreads();
+            if (K == I) break;
+#pragma unroll
+            for (int c = 0; c < 32; ++c) acc -= Rs[ti][c] * Xs[c][tj];
+        }
+        // the triangular block: the column's warp, from the last row up
+        const int last = min(31, k - 1 - 32 * I);
+        T x = T(0);
+        const T di = ti <= last ? Rs[ti][ti] : T(1), ri = T(1) / di;
+        for (int i = last; i >= 0; --i) {
+            // acc / di: the reciprocal and one correction step
+            T v = acc * ri;
+            v = fma(fma(-v, di, acc), ri, v);
+            v = __shfl_sync(0xffffffffu, v, i);
+            if (ti == i) x = v;
+            if (ti < i) acc -= Rs[ti][i] * v;
+        }
+        if (gi < k && l < r) tcol[gi] = x;
     }
 }
 
@@ -777,9 +819,9 @@ cudaError_t big_qr_step(const BigArgs& a, int ngroups, int max_n, int j, cudaStr
 template <typename T>
 cudaError_t big_finish(const BigArgs& a, int ngroups, int max_n, cudaStream_t st) {
     if (ngroups == 0) return cudaSuccess;
-    dim3 g((max_n + 127) / 128, ngroups);
+    dim3 g((max_n + TW - 1) / TW, ngroups);
     note_launch();
-    big_T_kernel<T><<<g, 128, 0, st>>>(a);
+    big_T_kernel<T><<<g, 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -1428,6 +1470,102 @@ __global__ void __launch_bounds__(PNT) be_panel_kernel(BatchElimArgs a, int j0) 
     }
 }
 
+// The same panel with its rows dealt to a cluster of PCL CTAs, in shared memory:
+// every CTA sends its best candidate of the column with its row, and the CTA
+// that holds row j that row too, to all the others, so that a column costs one
+// cluster barrier.  (The one-CTA panel in global memory took ~12 us a column:
+// 61 ms of the 3D n = 32 elimination.)
+constexpr int PCL = 8;
+
+template <typename T>
+size_t be_panel_smem(int rows) {
+    return (size_t)((rows + PCL - 1) / PCL) * 33 * sizeof(T);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) be_panel_cluster_kernel(BatchElimArgs a, int j0) {
+    const int e = blockIdx.x / PCL, rank = blockIdx.x % PCL;
+    const ElimDesc d = a.ed[e];
+    const EBox<T> Bx(a, e);
+    const int n = Bx.r;
+    if (j0 >= n || n <= a.factor_max_r) return;           // the whole cluster
+    const int nb = min(32, n - j0), rows = n - j0, per = (rows + PCL - 1) / PCL;
+    const int i0 = j0 + rank * per, own = max(0, min(per, n - i0));
+    const int64_t ld = Bx.n;
+    T* A = Bx.A;
+    int* piv = a.piv + d.piv_out;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* P = reinterpret_cast<T*>(smem_raw);                // P[33 i + c]: row i0 + i, column j0 + c
+    __shared__ T crow[2][PCL][32], jrow[2][32], cval[2][PCL], wv[8];
+    __shared__ int cid[2][PCL], wi[8];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    for (int q = t; q < own * nb; q += 256) P[33 * (q % own) + q / own] = A[i0 + q % own + ld * (j0 + q / own)];
+    __syncthreads();
+    cl_sync();
+    bool bad = false;
+    for (int c = 0; c < nb; ++c) {
+        const int j = j0 + c, buf = c & 1;
+        T best = T(-1);
+        int bi = -1, dummy = 0;
+        for (int i = t; i < own; i += 256) {
+            const T v = fabs(P[33 * i + c]);
+            if (i0 + i >= j && (bi < 0 ? v == v : v > best)) { best = v; bi = i0 + i; }
+        }
+        dummy = bi;                                       // ties: lowest row
+        warp_best(best, dummy, bi);
+        if (lane == 0) { wv[warp] = best; wi[warp] = bi; }
+        __syncthreads();
+        // warp q sends this CTA's candidate (and row j) to CTA q
+        best = lane < 8 ? wv[lane] : T(-1);
+        bi = dummy = lane < 8 ? wi[lane] : -1;
+        warp_best(best, dummy, bi);
+        if (bi >= 0) cl_store(cl_peer(&crow[buf][rank][lane], warp), lane < nb ? P[33 * (bi - i0) + lane] : T(0));
+        if (lane == 0) {
+            cl_store(cl_peer(&cval[buf][rank], warp), best);
+            cl_store(cl_peer(&cid[buf][rank], warp), bi);
+        }
+        if (j >= i0 && j < i0 + own && lane < nb) cl_store(cl_peer(&jrow[buf][lane], warp), P[33 * (j - i0) + lane]);
+        cl_sync();
+        int p = -1, pr = 0;
+        best = T(-1);
+        for (int q = 0; q < PCL; ++q) {
+            const int id = cid[buf][q];
+            const T v = cval[buf][q];
+            if (id >= 0 && (p < 0 || v > best || (v == best && id < p))) { best = v; p = id; pr = q; }
+        }
+        if (p < 0) p = j;                                 // all NaN: the test below fails
+        const T* prow = best >= T(0) ? crow[buf][pr] : jrow[buf];
+        if (rank == 0 && t == 0) piv[j] = p;
+        const T dg = prow[c];
+        if (dg == T(0) || !isfinite((double)dg)) {
+            if (rank == 0 && t == 0) atomicOr(a.status, (int)DEV_SINGULAR);
+            bad = true;
+            break;
+        }
+        const T inv = T(1) / dg;
+        for (int i = t; i < own; i += 256) {
+            const int g = i0 + i;
+            T* x = P + 33 * i;
+            if (g == p && p != j)
+                for (int q = 0; q < nb; ++q) x[q] = jrow[buf][q];
+            if (g == j)
+                for (int q = 0; q < nb; ++q) x[q] = prow[q];
+            if (g <= j) continue;
+            const T l = x[c] * inv;
+            x[c] = l;
+            for (int q = c + 1; q < nb; ++q) x[q] -= l * prow[q];
+        }
+        __syncthreads();
+    }
+    cl_sync();                                            // no CTA leaves while a peer may store to it
+    if (bad) {
+        for (int j = j0 + t; rank == 0 && j < j0 + nb; j += 256)
+            if (j > j0) piv[j] = j;
+        return;
+    }
+    for (int q = t; q < own * nb; q += 256) A[i0 + q % own + ld * (j0 + q / own)] = P[33 * (q % own) + q / own];
+}
+
 template <typename T>
 __global__ void be_swap_trsm_kernel(BatchElimArgs a, int j0) {
     const int e = blockIdx.y;
@@ -1501,9 +1639,8 @@ __global__ void __launch_bounds__(256) be_update_kernel(BatchElimArgs a, int j0)
 // With P B_rr = L U = L D U' (L, U' unit triangular), Lemma 2.4's blocks
 // are X = B_sr U^{-1}, Z = L^{-1} P B_rs, the Schur update S = -X Z, and the
 // sweeps keep Y = D^{-1} Z and the unit triangular inverses L^{-1}, U'^{-1}.
-// The inverses are formed by IB x IB blocks: the diagonal blocks by
-// substitution, then every block column J below the diagonal as
-// X_IJ = -inv(F_II) sum_{K=J..I-1} F_IK X_KJ (F = L, or U'^T for the upper
+// The inverses are formed from the diagonal IB x IB blocks up, by substitution
+// and then by doubling (be_inv_level_kernel; F = L, or U'^T for the upper
 // factor).  X and Z are blocked substitutions (only the IB x IB diagonal
 // blocks enter through their inverses: multiplying by the whole explicit
 // inverse measured a less accurate FP32 factor), S a tiled product.
@@ -1589,64 +1726,70 @@ __global__ void be_dinv_kernel(BatchElimArgs a) {
     if (t < nbk) X[(b0 + t) + (int64_t)r * (b0 + t)] = T(0);
 }
 
-// block column J of the inverse, blocks I = J+1.. in order (one CTA per
-// block column and box; 256 threads, 4 entries of the 32 x 32 block each)
-template <typename T, bool UP>
-__global__ void __launch_bounds__(256) be_binv_kernel(BatchElimArgs a) {
-    const int e = blockIdx.y;
+// From the inverses of the diagonal blocks of size s to those of size 2 s:
+// with F = [F11 0; F21 F22] the block below is -inv(F22) (F21 inv(F11)).
+// PH 1: T = F21 inv(F11), into B_rr's work space (no longer needed); PH 2:
+// X21 = -inv(F22) T.  One CTA per 32 x 32 tile, pair of blocks and box, so a
+// level fills the GPU.  (Block column by block column, each one a chain over
+// its blocks, the 3D n = 32 inverses took 39 ms, the n = 200 64-bit ones 21;
+// with the cluster panels the eliminations went from 123 to 46 and from 92 to
+// 70 ms.)
+template <typename T, bool UP, int PH>
+__global__ void __launch_bounds__(256) be_inv_level_kernel(BatchElimArgs a, int s) {
+    const int e = blockIdx.z;
     const ElimDesc d = a.ed[e];
-    const int r = d.r;
-    const int nb = (r + IB - 1) / IB;
-    const int J = blockIdx.x;
-    if (J >= nb - 1 || (UP && d.ldl)) return;
+    const int r = d.r, nt = s / IB;
+    const int ti0 = blockIdx.x % nt, tj0 = blockIdx.x / nt;
+    const int b = 2 * s * blockIdx.y, i0 = b + s + IB * ti0, j0 = b + IB * tj0;
+    if (i0 >= r || (UP && d.ldl)) return;
     const bool xt = UP || d.ldl;
     const T* F = static_cast<const T*>(a.pool) + d.LU_out;
     T* X = static_cast<T*>(a.pool) + d.LUi_out;
-    __shared__ T Fs[IB][IB + 1];
-    __shared__ T Xs[IB][IB + 1];
-    const int t = threadIdx.x;
-    const int ti = t % IB, tj = t / IB;          // entries (ti, tj + 8 q)
-    for (int I = J + 1; I < nb; ++I) {
-        T acc[4] = {T(0), T(0), T(0), T(0)};
-        for (int K = J; K < I; ++K) {
-            __syncthreads();
-            for (int q = t; q < IB * IB; q += 256) {
-                const int i = UP ? q / IB : q % IB, l = UP ? q % IB : q / IB;
-                const int gi = I * IB + i, gl = K * IB + l;
-                Fs[i][l] = (gi < r && gl < r) ? tri_f<T, UP>(F, r, gi, gl) : T(0);
-                // X_KJ (unit diagonal, zero above)
-                const int xk = UP ? q / IB : q % IB, xj = UP ? q % IB : q / IB;
-                const int gk = K * IB + xk, gj = J * IB + xj;
-                T xv = T(0);
-                if (gk < r && gj < r) xv = gk == gj ? T(1) : (gk > gj ? *tri_x(X, r, xt, gk, gj) : T(0));
-                Xs[xk][xj] = xv;
-            }
-            __syncthreads();
-#pragma unroll 8
-            for (int l = 0; l < IB; ++l) {
-                const T f = Fs[ti][l];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[q] += f * Xs[l][tj + 8 * q];
-            }
-        }
-        // X_IJ = -(I + S_II) acc, S_II the stored strict part of inv(F_II)
+    const EBox<T> Bx(a, e);
+    T* Tm = Bx.A;
+    const int64_t ld = Bx.n;
+    __shared__ T Ls[IB][IB + 1];
+    __shared__ T Rs[IB][IB + 1];
+    const int t = threadIdx.x, ti = t % IB, tj = t / IB;          // entries (ti, tj + 8 q)
+    T acc[4] = {T(0), T(0), T(0), T(0)};
+    // entry (i, j) of the unit lower inverse inside a diagonal block of size s
+    auto inv_at = [&](int i, int j) -> T {
+        return i < r && j < r ? (i == j ? T(1) : i > j ? *tri_x(X, r, xt, i, j) : T(0)) : T(0);
+    };
+    const int k0 = PH == 1 ? tj0 : 0, k1 = PH == 1 ? nt : ti0 + 1;
+    for (int K = k0; K < k1; ++K) {
+        const int g0 = (PH == 1 ? b : b + s) + IB * K;            // rows of the right operand
         __syncthreads();
-#pragma unroll
-        for (int q = 0; q < 4; ++q) Xs[ti][tj + 8 * q] = acc[q];
         for (int q = t; q < IB * IB; q += 256) {
-            const int i = UP ? q / IB : q % IB, l = UP ? q % IB : q / IB;
-            const int gi = I * IB + i, gl = I * IB + l;
-            Fs[i][l] = (i > l && gi < r && gl < r) ? *tri_x(X, r, xt, gi, gl) : T(0);
+            const int u = q % IB, v = q / IB;
+            {
+                // coalesced along the stored rows
+                const int i = (PH == 1 ? UP : xt) ? v : u, l = (PH == 1 ? UP : xt) ? u : v;
+                const int gi = i0 + i, gl = g0 + l;
+                Ls[i][l] = PH == 1 ? (gi < r && gl < r ? tri_f<T, UP>(F, r, gi, gl) : T(0)) : inv_at(gi, gl);
+            }
+            {
+                const bool tr = PH == 1 && xt;
+                const int l = tr ? v : u, c = tr ? u : v;
+                const int gl = g0 + l, gc = j0 + c;
+                Rs[l][c] = PH == 1 ? inv_at(gl, gc) : gl < r ? Tm[gl + ld * gc] : T(0);
+            }
         }
         __syncthreads();
-        const int gi = I * IB + ti;
+#pragma unroll 8
+        for (int l = 0; l < IB; ++l) {
+            const T f = Ls[ti][l];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int jj = tj + 8 * q, gj = J * IB + jj;
-            T v = Xs[ti][jj];
-            for (int l = 0; l < ti; ++l) v += Fs[ti][l] * Xs[l][jj];
-            if (gi < r && gj < r) *tri_x(X, r, xt, gi, gj) = -v;
+            for (int q = 0; q < 4; ++q) acc[q] += f * Rs[l][tj + 8 * q];
         }
+    }
+    const int gi = i0 + ti;
+    if (gi >= r) return;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int gj = j0 + tj + 8 * q;
+        if (PH == 1) Tm[gi + ld * gj] = acc[q];
+        else *tri_x(X, r, xt, gi, gj) = -acc[q];
     }
 }
 
@@ -1895,8 +2038,27 @@ cudaError_t big_elim_batch(const BatchElimArgs& a, int max_n, int max_k, int max
         if (e != cudaSuccess) return e;
     }
     for (int j0 = 0; max_r > a.factor_max_r && j0 < max_r; j0 += 32) {
+        const size_t ps = be_panel_smem<T>(max_r - j0);
         note_launch();
-        be_panel_kernel<T><<<nb, PNT, 0, st>>>(a, j0);
+        if (ps <= 200 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(be_panel_cluster_kernel<T>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+            if (e != cudaSuccess) return e;
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3((unsigned)(nb * PCL));
+            cfg.blockDim = dim3(256);
+            cfg.dynamicSmemBytes = ps;
+            cfg.stream = st;
+            cudaLaunchAttribute at{};
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = PCL;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            if ((e = cudaLaunchKernelEx(&cfg, be_panel_cluster_kernel<T>, a, j0)) != cudaSuccess) return e;
+        } else {
+            be_panel_kernel<T><<<nb, PNT, 0, st>>>(a, j0);
+        }
         note_launch();
         be_swap_trsm_kernel<T><<<dim3((max_r + 127) / 128, nb), 128, 0, st>>>(a, j0);
         const int rest = max_r - j0 - 32;
@@ -1912,19 +2074,17 @@ cudaError_t big_elim_batch(const BatchElimArgs& a, int max_n, int max_k, int max
     be_dinv_kernel<T, false><<<dim3(rb, nb), 32, 0, st>>>(a);
     note_launch();
     be_dinv_kernel<T, true><<<dim3(rb, nb), 32, 0, st>>>(a);
-    if (rb > 1) {
-        note_launch();
-        be_binv_kernel<T, false><<<dim3(rb - 1, nb), 256, 0, st>>>(a);
-        note_launch();
-        be_binv_kernel<T, true><<<dim3(rb - 1, nb), 256, 0, st>>>(a);
-    }
     if (max_k > 0) {
+        // rows (columns) of a substitution's CTA: 64, or 16 while 64 would
+        // leave SMs without one (n = 200, 64-bit: 16 boxes of k ~ 500)
+        const int rt = (int64_t)((max_k + 63) / 64) * nb < 2 * a.num_sms ? 16 : 64;
+        const dim3 gt((max_k + rt - 1) / rt, nb);
         note_launch();
-        if (small) be_trsm_x_kernel<T, 16><<<dim3((max_k + 15) / 16, nb), 256, 0, st>>>(a);
-        else be_trsm_x_kernel<T, 64><<<dim3(tk, nb), 256, 0, st>>>(a);
+        if (rt == 16) be_trsm_x_kernel<T, 16><<<gt, 256, 0, st>>>(a);
+        else be_trsm_x_kernel<T, 64><<<gt, 256, 0, st>>>(a);
         note_launch();
-        if (small) be_trsm_z_kernel<T, 16><<<dim3((max_k + 15) / 16, nb), 256, 0, st>>>(a);
-        else be_trsm_z_kernel<T, 64><<<dim3(tk, nb), 256, 0, st>>>(a);
+        if (rt == 16) be_trsm_z_kernel<T, 16><<<gt, 256, 0, st>>>(a);
+        else be_trsm_z_kernel<T, 64><<<gt, 256, 0, st>>>(a);
         if (tcg) {
             const cudaError_t e = tc_op(4, max_k, max_k);
             if (e != cudaSuccess) return e;
@@ -1933,6 +2093,19 @@ cudaError_t big_elim_batch(const BatchElimArgs& a, int max_n, int max_k, int max
             if (small) be_schur_kernel<T, 32><<<dim3(tk, tk, nb), 256, 0, st>>>(a);
             else be_schur_kernel<T, 64><<<dim3(tk, tk, nb), 256, 0, st>>>(a);
         }
+    }
+    // inverses of the unit triangular factors, by doubling the inverted blocks
+    for (int s = IB; s < max_r; s *= 2) {
+        const int nt = s / IB;
+        const dim3 g(nt * nt, (max_r + 2 * s - 1) / (2 * s), nb);
+        note_launch();
+        be_inv_level_kernel<T, false, 1><<<g, 256, 0, st>>>(a, s);
+        note_launch();
+        be_inv_level_kernel<T, false, 2><<<g, 256, 0, st>>>(a, s);
+        note_launch();
+        be_inv_level_kernel<T, true, 1><<<g, 256, 0, st>>>(a, s);
+        note_launch();
+        be_inv_level_kernel<T, true, 2><<<g, 256, 0, st>>>(a, s);
     }
     note_launch();
     be_finish_kernel<T><<<dim3((unsigned)std::clamp<int64_t>(((int64_t)max_k * max_r + 255) / 256, 1, 512), nb), 256,

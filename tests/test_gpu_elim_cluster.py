@@ -38,3 +38,29 @@ def test_cluster_elimination_matches_one_cta(monkeypatch, n, dim, general, preci
     tol = 1e-12 if precision == "fp64" else 1e-4
     for p, q in zip(*out):
         assert float((p - q).abs().max()) <= tol * float(q.abs().max())
+
+
+@pytest.mark.parametrize("n,dim,precision", [(64, 2, "fp64"), (40, 2, "fp32"), (12, 3, "fp64")])
+def test_panel_elimination_matches_cluster(monkeypatch, n, dim, precision):
+    # LU blocks above HIF_ELIM_CLUSTER_R rows by panels of 32 columns: blocks of
+    # one panel and of several, ragged last panels, the top block
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1307_2666_gb300 as P
+    pb = hi.volume_problem(n, dim, smooth_seed=41 + n)
+    c = 1.0 + 0.5 * hi.smooth_field(pb.points, 96)
+    T = lambda v: torch.as_tensor(np.ascontiguousarray(v), dtype=torch.float64, device="cuda:0")
+    x = T(hi.gaussian_rhs(pb.N, 3, n))
+    monkeypatch.setenv("HIF_ELIM_MID", "0")
+    monkeypatch.setenv("HIF_BIG_ELIM", "24")
+    out = []
+    for line in ("100000", "33", "8"):
+        monkeypatch.setenv("HIF_ELIM_CLUSTER_R", line)
+        fac = P.Factorization(T(pb.points), T(pb.weights), T(pb.a), T(pb.b), T(c), pb.kernel_id, 1e-6,
+                              proxy_dirs=pb.proxy if dim == 3 else None, precision=precision)
+        out.append([getattr(fac, op)(x) for op in ("solve", "apply", "solve_transpose", "apply_transpose")])
+        fac.close()
+    tol = 1e-12 if precision == "fp64" else 1e-4
+    for other in out[1:]:
+        for p, q in zip(other, out[0]):
+            assert float((p - q).abs().max()) <= tol * float(q.abs().max())
