@@ -441,6 +441,7 @@ static void run_big_id(hif_handle h, size_t tau, const std::vector<BoxDesc>& bd,
     B.nrm.ensure(sizeof(double) * std::max<int64_t>(voff, 1));
     B.perm.ensure(sizeof(int) * std::max<int64_t>(voff, 1));
     BigArgs a{};
+    a.num_sms = h->num_sms;
     a.g = geom(h);
     a.sci = scidev(h, (int)tau);
     a.boxes = d_boxes.as<BoxDesc>();
@@ -758,6 +759,7 @@ static void run_big_id_R(hif_handle h, const std::vector<BoxDesc>& bd, const std
     ga.tol_floor = tol_floor;
     HIF_CUDA((launch_gram_tol<T>(ga, ng, max_ng, st)));
     BigArgs a{};
+    a.num_sms = h->num_sms;
     a.groups = B.bg.as<BigGroup>();
     a.state = B.state.as<BigState>();
     a.gdesc = d_groups.as<GroupDesc>();

@@ -271,11 +271,26 @@ __global__ void __launch_bounds__(BST) big_step_kernel(BigArgs a, int j) {
         }
         return;
     }
-    if (p != j) {
-        for (int i = threadIdx.x; i < G.m; i += blockDim.x) {
-            const T t = W[i + ld * j];
-            W[i + ld * j] = W[i + ld * p];
-            W[i + ld * p] = t;
+    // columns j and p swapped, and the sum of squares below row j of the new
+    // column j; SU rows per thread in flight (one CTA walks the m rows)
+    constexpr int SU = 8;
+    T s = T(0);
+    for (int i0 = threadIdx.x; i0 < G.m; i0 += BST * SU) {
+        T xj[SU], xp[SU];
+#pragma unroll
+        for (int u = 0; u < SU; ++u) {
+            const int i = i0 + BST * u;
+            xj[u] = i < G.m ? W[i + ld * j] : T(0);
+            xp[u] = i < G.m && p != j ? W[i + ld * p] : xj[u];
+        }
+#pragma unroll
+        for (int u = 0; u < SU; ++u) {
+            const int i = i0 + BST * u;
+            if (i < G.m && p != j) {
+                W[i + ld * j] = xp[u];
+                W[i + ld * p] = xj[u];
+            }
+            if (i > j && i < G.m) s += xp[u] * xp[u];
         }
     }
     __syncthreads();
@@ -283,12 +298,6 @@ __global__ void __launch_bounds__(BST) big_step_kernel(BigArgs a, int j) {
         const int t = perm[j]; perm[j] = perm[p]; perm[p] = t;
         double tn = nrm[j]; nrm[j] = nrm[p]; nrm[p] = tn;
         tn = nrm0[j]; nrm0[j] = nrm0[p]; nrm0[p] = tn;
-    }
-    // reflector for W[j:, j]
-    T s = T(0);
-    for (int i = j + 1 + threadIdx.x; i < G.m; i += blockDim.x) {
-        const T v = W[i + ld * j];
-        s += v * v;
     }
     hs[threadIdx.x] = s;
     __syncthreads();
@@ -306,7 +315,14 @@ __global__ void __launch_bounds__(BST) big_step_kernel(BigArgs a, int j) {
     }
     __syncthreads();
     if (tau != T(0)) {
-        for (int i = j + 1 + threadIdx.x; i < G.m; i += blockDim.x) W[i + ld * j] *= scal;
+        for (int i0 = j + 1 + threadIdx.x; i0 < G.m; i0 += BST * SU) {
+            T x[SU];
+#pragma unroll
+            for (int u = 0; u < SU; ++u) x[u] = i0 + BST * u < G.m ? W[i0 + BST * u + ld * j] : T(0);
+#pragma unroll
+            for (int u = 0; u < SU; ++u)
+                if (i0 + BST * u < G.m) W[i0 + BST * u + ld * j] = x[u] * scal;
+        }
         if (threadIdx.x == 0) W[j + ld * j] = -copysign(sqrt(alpha * alpha + ss), alpha);
     }
     if (threadIdx.x == 0) {
@@ -316,8 +332,10 @@ __global__ void __launch_bounds__(BST) big_step_kernel(BigArgs a, int j) {
     }
 }
 
+// (U rows per lane are loaded before their FMAs: bytes in flight bound the
+// step.  n = 200, b != c, 64-bit: 234 -> 175 ms of updates, 128 of them FP64.)
 template <typename T>
-__global__ void __launch_bounds__(256) big_update_kernel(BigArgs a, int j) {
+__global__ void __launch_bounds__(256, 4) big_update_kernel(BigArgs a, int j) {
     const BigGroup G = a.groups[blockIdx.y];
     const BigState S = a.state[blockIdx.y];
     if (S.k != j + 1 || S.stop) return;
@@ -329,16 +347,40 @@ __global__ void __launch_bounds__(256) big_update_kernel(BigArgs a, int j) {
     T* col = W + ld * l;
     const T* v = W + ld * j;
     const T tau = (T)S.tau;
+    constexpr int U = 8;                 // rows in flight per lane
     T w = T(0);
     if (tau != T(0)) {
-        for (int i = j + 1 + lane; i < G.m; i += 32) w += v[i] * col[i];
+        int i = j + 1 + lane;
+        for (; i + 32 * (U - 1) < G.m; i += 32 * U) {
+            T x[U], y[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                x[u] = col[i + 32 * u];
+                y[u] = v[i + 32 * u];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) w += y[u] * x[u];
+        }
+        for (; i < G.m; i += 32) w += v[i] * col[i];
         w = warp_sum(w);
         w = (w + col[j]) * tau;
         __syncwarp();
         if (lane == 0) col[j] -= w;
     }
-    if (tau != T(0))
-        for (int i = j + 1 + lane; i < G.m; i += 32) col[i] -= w * v[i];
+    if (tau != T(0)) {
+        int i = j + 1 + lane;
+        for (; i + 32 * (U - 1) < G.m; i += 32 * U) {
+            T x[U], y[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                x[u] = col[i + 32 * u];
+                y[u] = v[i + 32 * u];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) col[i + 32 * u] = x[u] - w * y[u];
+        }
+        for (; i < G.m; i += 32) col[i] -= w * v[i];
+    }
     // the square of the new norm (see kNormKeep)
     double* nrm = a.nrm + G.vec_off + l;
     double* nrm0 = a.nrm0 + G.vec_off + l;
@@ -384,22 +426,49 @@ __global__ void bqp_start_kernel(BigArgs a, int ngroups) {
     S.pend = 0;
 }
 
-// one pivot of the panel (one CTA per group): argmax of the downdated norms,
-// column swap, the pivot column brought up to date, its reflector, and
-// g = V_panel^T v
+// distributed shared memory of a cluster
+__device__ __forceinline__ uint32_t cl_peer(const void* p, int rank) {
+    uint32_t out;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return out;
+}
+__device__ __forceinline__ void cl_store(uint32_t a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cl_store(uint32_t a, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cl_store(uint32_t a, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cl_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// one pivot of the panel: argmax of the downdated norms, column swap, the pivot
+// column brought up to date, its reflector, and g = V_panel^T v.  The rows of a
+// group are dealt to a cluster of `cl` CTAs (as many as leave two per SM): the
+// steps of a pivot are passes over the m rows of up to 32 columns, and between
+// two bqp_f launches nothing else runs.  Every CTA finds the pivot itself;
+// the cluster's barriers (the reflector's norm, g) follow, and rank 0 keeps the
+// group's state.  Measured on a GB300, 3D n = 32 (eight boxes of up to 1,968
+// columns and 28,000 rows): 55 us a pivot with one CTA per group, 35 with up to
+// eight; with clusters for four times as many groups (three waves) 47.
 constexpr int QPT = 512;   // threads of the pivot kernel
 
 template <typename T>
-__global__ void __launch_bounds__(QPT) bqp_pivot_kernel(BigArgs a, int step) {
-    const BigGroup G = a.groups[blockIdx.x];
-    BigState* S = a.state + blockIdx.x;
+__global__ void __launch_bounds__(QPT) bqp_pivot_kernel(BigArgs a, int step, int cl) {
+    const int gi = blockIdx.x / cl, rank = blockIdx.x % cl;
+    const BigGroup G = a.groups[gi];
+    BigState* S = a.state + gi;
     if (S->stop || S->pend) return;
     const int j = S->k, j0 = S->j0, jj = j - j0;
     const int nb = a.nb;
     if (jj >= nb) return;
     const int kmax = min(G.m, G.n);
+    const bool lead = rank == 0 && threadIdx.x == 0;
     if (j >= kmax) {
-        if (threadIdx.x == 0) S->stop = 1;
+        if (lead) S->stop = 1;
         return;
     }
     T* W = static_cast<T*>(a.YK) + G.y_off;
@@ -409,132 +478,147 @@ __global__ void __launch_bounds__(QPT) bqp_pivot_kernel(BigArgs a, int step) {
     double* nrm0 = a.nrm0 + G.vec_off;
     int* perm = a.perm + G.vec_off;
     T* F = static_cast<T*>(a.F) + G.vec_off * nb;
-    T* gq = static_cast<T*>(a.gv) + (int64_t)blockIdx.x * QPB;
-    __shared__ double redv[QPT];
-    __shared__ int redi[QPT];
-    __shared__ T hs[QPT];
-    __shared__ T fj[QPB];
-    __shared__ T part[QPT / 32][QPB];
+    T* gq = static_cast<T*>(a.gv) + (int64_t)gi * QPB;
+    constexpr int NW = QPT / 32;
+    __shared__ double redv[NW];
+    __shared__ int redi[NW], redo[NW];
+    __shared__ T hs[NW], fj[QPB], part[NW][QPB];
+    __shared__ T cs[8], calpha, cg[8][QPB];             // sent by the CTAs of the cluster
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     // pivot: largest downdated norm, ties to the lowest original column
+    auto better = [](double v2, int o2, int l2, double v, int o, int l) {
+        return l2 >= 0 && (l < 0 || v2 > v || (v2 == v && o2 < o));
+    };
     double best = -1.0;
     int bl = -1, bo = 1 << 30;
-    for (int l = j + threadIdx.x; l < n; l += blockDim.x) {
+    for (int l = j + threadIdx.x; l < n; l += QPT) {
         const double v = nrm[l];
         if (v > best || (v == best && perm[l] < bo)) { best = v; bo = perm[l]; bl = l; }
     }
-    redv[threadIdx.x] = best;
-    redi[threadIdx.x] = bl;
-    __syncthreads();
-    for (int s2 = blockDim.x / 2; s2 > 0; s2 >>= 1) {
-        if (threadIdx.x < s2) {
-            const double v2 = redv[threadIdx.x + s2], v1 = redv[threadIdx.x];
-            const int l2 = redi[threadIdx.x + s2], l1 = redi[threadIdx.x];
-            if (l2 >= 0 && (l1 < 0 || v2 > v1 || (v2 == v1 && perm[l2] < perm[l1]))) {
-                redv[threadIdx.x] = v2;
-                redi[threadIdx.x] = l2;
-            }
+    for (int q = 0; q < 2; ++q) {
+        for (int off = 16; off; off >>= 1) {
+            const double v2 = __shfl_xor_sync(0xffffffffu, best, off);
+            const int o2 = __shfl_xor_sync(0xffffffffu, bo, off), l2 = __shfl_xor_sync(0xffffffffu, bl, off);
+            if (better(v2, o2, l2, best, bo, bl)) { best = v2; bo = o2; bl = l2; }
         }
-        __syncthreads();
+        if (q == 0) {
+            if (lane == 0) { redv[wid] = best; redo[wid] = bo; redi[wid] = bl; }
+            __syncthreads();
+            best = lane < NW ? redv[lane] : -1.0;
+            bo = lane < NW ? redo[lane] : 1 << 30;
+            bl = lane < NW ? redi[lane] : -1;
+        }
     }
-    const double bnorm = sqrt(fmax(redv[0], 0.0));
-    const int p = redi[0];
+    const double bnorm = sqrt(fmax(best, 0.0));
+    const int p = bl;
     const double nu0 = j == 0 ? bnorm : S->nu0;
-    __syncthreads();
     // the rank test decides on exact norms: within a panel (downdated norms,
     // relative error up to ~sqrt(eps_T) in the square) a maximum near the
     // threshold ends the panel instead, and the next panel's first pivot,
     // on the recomputed norms, decides
     const double margin = sizeof(T) == 4 ? 1e-3 : 1e-7;
     if (jj > 0 && bnorm <= G.tol * nu0 * (1.0 + margin) && p >= j) {
-        if (threadIdx.x == 0) S->pend = 1;
+        if (lead) S->pend = 1;
         return;
     }
     if (bnorm <= G.tol * nu0 || bnorm == 0.0 || p < j) {
-        if (threadIdx.x == 0) {
+        if (lead) {
             S->stop = 1;
             if (j == 0) S->nu0 = bnorm;
         }
         return;
     }
-    if (p != j) {
-        for (int i = threadIdx.x; i < G.m; i += blockDim.x) {
+    // this CTA's rows [i0, i1) of j .. m - 1 (rank 0: also the finished rows
+    // above, which only swap)
+    const int per = (G.m - j + cl - 1) / cl;
+    const int i0 = min(G.m, j + rank * per), i1 = min(G.m, i0 + per);
+    if (cl > 1) cl_sync();                              // every CTA is there before the first remote store
+    if (threadIdx.x < jj) fj[threadIdx.x] = F[p + (int64_t)n * threadIdx.x];
+    if (rank == 0 && p != j)
+        for (int i = threadIdx.x; i < j; i += QPT) {
             const T t = W[i + ld * j];
             W[i + ld * j] = W[i + ld * p];
             W[i + ld * p] = t;
         }
-        for (int q = threadIdx.x; q < jj; q += blockDim.x) {
-            const T t = F[j + (int64_t)n * q];
-            F[j + (int64_t)n * q] = F[p + (int64_t)n * q];
-            F[p + (int64_t)n * q] = t;
-        }
-    }
     __syncthreads();
-    if (threadIdx.x == 0 && p != j) {
-        const int t = perm[j]; perm[j] = perm[p]; perm[p] = t;
-        double tn = nrm[j]; nrm[j] = nrm[p]; nrm[p] = tn;
-        tn = nrm0[j]; nrm0[j] = nrm0[p]; nrm0[p] = tn;
-    }
-    for (int q = threadIdx.x; q < jj; q += blockDim.x) fj[q] = F[j + (int64_t)n * q];
-    __syncthreads();
-    // rows j.. of the pivot column: W[i, j] -= sum_q W[i, j0 + q] F[j, q]
-    if (jj > 0)
-        for (int i = j + threadIdx.x; i < G.m; i += blockDim.x) {
-            T acc = W[i + ld * j];
-            for (int q = 0; q < jj; ++q) acc -= W[i + ld * (j0 + q)] * fj[q];
-            W[i + ld * j] = acc;
-        }
-    __syncthreads();
-    // reflector for W[j:, j]
+    // the pivot column up to date, W[i, j] = W[i, p] - sum_q W[i, j0 + q] F[p, q],
+    // and the sum of its squares below row j
     T ssum = T(0);
-    for (int i = j + 1 + threadIdx.x; i < G.m; i += blockDim.x) {
-        const T v = W[i + ld * j];
-        ssum += v * v;
+    for (int i = i0 + threadIdx.x; i < i1; i += QPT) {
+        T acc = W[i + ld * p];
+        if (p != j) W[i + ld * p] = W[i + ld * j];
+#pragma unroll 8
+        for (int q = 0; q < jj; ++q) acc -= W[i + ld * (j0 + q)] * fj[q];
+        W[i + ld * j] = acc;
+        if (i > j) ssum += acc * acc;
+        else for (int q = 0; q < cl; ++q) cl_store(cl_peer(&calpha, q), acc);
     }
-    hs[threadIdx.x] = ssum;
+    ssum = warp_sum(ssum);
+    if (lane == 0) hs[wid] = ssum;
     __syncthreads();
-    for (int k2 = blockDim.x / 2; k2 > 0; k2 >>= 1) {
-        if (threadIdx.x < k2) hs[threadIdx.x] += hs[threadIdx.x + k2];
-        __syncthreads();
+    if (wid == 0) {
+        ssum = warp_sum(lane < NW ? hs[lane] : T(0));
+        if (lane < cl) cl_store(cl_peer(&cs[rank], lane), ssum);
     }
-    const T ss = hs[0];
-    const T alpha = W[j + ld * j];
+    if (cl > 1) cl_sync();
+    else __syncthreads();
+    T ss = T(0);
+    for (int q = 0; q < cl; ++q) ss += cs[q];
+    const T alpha = calpha;
     T tau = T(0), scal = T(0), beta = alpha;
     if (ss != T(0)) {
         beta = -copysign(sqrt(alpha * alpha + ss), alpha);
         tau = (beta - alpha) / beta;
         scal = T(1) / (alpha - beta);
     }
-    __syncthreads();
-    if (tau != T(0)) {
-        for (int i = j + 1 + threadIdx.x; i < G.m; i += blockDim.x) W[i + ld * j] *= scal;
-        if (threadIdx.x == 0) W[j + ld * j] = beta;
-    }
-    __syncthreads();
-    // g[q] = sum_{i >= j} W[i, j0 + q] v_i, v_j = 1, v_i = W[i, j] below
-    if (jj > 0) {
-        T acc[QPB];
+    // v, and g[q] = sum_{i >= j} W[i, j0 + q] v_i, v_j = 1
+    T acc[QPB];
 #pragma unroll
-        for (int q = 0; q < QPB; ++q) acc[q] = T(0);
-        for (int i = j + threadIdx.x; i < G.m; i += blockDim.x) {
-            const T vi = i == j ? T(1) : W[i + ld * j];
-#pragma unroll
-            for (int q = 0; q < QPB; ++q)
-                if (q < jj) acc[q] += W[i + ld * (j0 + q)] * vi;
+    for (int q = 0; q < QPB; ++q) acc[q] = T(0);
+    for (int i = i0 + threadIdx.x; i < i1; i += QPT) {
+        T vi = T(1);
+        if (i > j) {
+            vi = W[i + ld * j];
+            if (tau != T(0)) {
+                vi *= scal;
+                W[i + ld * j] = vi;
+            }
         }
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+        for (int q = 0; q < QPB; ++q)
+            if (q < jj) acc[q] += W[i + ld * (j0 + q)] * vi;
+    }
+    if (jj > 0) {
 #pragma unroll
         for (int q = 0; q < QPB; ++q) {
+            if (q >= jj) break;
             const T v = warp_sum(acc[q]);
             if (lane == 0) part[wid][q] = v;
         }
         __syncthreads();
         if (threadIdx.x < jj) {
             T v = T(0);
-            for (int w = 0; w < QPT / 32; ++w) v += part[w][threadIdx.x];
-            gq[threadIdx.x] = v;
+            for (int w = 0; w < NW; ++w) v += part[w][threadIdx.x];
+            cl_store(cl_peer(&cg[rank][threadIdx.x], 0), v);
         }
     }
+    if (cl > 1) cl_sync();
+    else __syncthreads();
+    if (rank != 0) return;
+    if (threadIdx.x < jj) {
+        T v = T(0);
+        for (int q = 0; q < cl; ++q) v += cg[q][threadIdx.x];
+        gq[threadIdx.x] = v;
+        if (p != j) F[p + (int64_t)n * threadIdx.x] = F[j + (int64_t)n * threadIdx.x];
+        F[j + (int64_t)n * threadIdx.x] = fj[threadIdx.x];
+    }
     if (threadIdx.x == 0) {
+        if (p != j) {
+            const int t = perm[j]; perm[j] = perm[p]; perm[p] = t;
+            double tn = nrm[j]; nrm[j] = nrm[p]; nrm[p] = tn;
+            tn = nrm0[j]; nrm0[j] = nrm0[p]; nrm0[p] = tn;
+        }
+        if (tau != T(0)) W[j + ld * j] = beta;
         if (j == 0) S->nu0 = bnorm;
         S->tau = (double)tau;
         S->k = j + 1;
@@ -542,37 +626,65 @@ __global__ void __launch_bounds__(QPT) bqp_pivot_kernel(BigArgs a, int step) {
     }
 }
 
-// F[l, jj] for the trailing columns (a warp per column), the pivot row's
-// entry brought up to date, and the norm downdated
+// F[l, jj] for the trailing columns (a warp per two columns, which share the
+// reads of v), the pivot row's entry brought up to date, and the norm downdated.
+// Bound by the bytes in flight: with 16 rows of the columns per lane loaded
+// before their FMAs the 3D n = 32 launches went from 107 to 73 ms (4.8 TB/s).
 template <typename T>
-__global__ void __launch_bounds__(256) bqp_f_kernel(BigArgs a, int step) {
+__global__ void __launch_bounds__(256, 4) bqp_f_kernel(BigArgs a, int step) {
     const BigGroup G = a.groups[blockIdx.y];
     const BigState S = a.state[blockIdx.y];
     if (S.stop || S.last_step != step) return;
     const int j = S.k - 1, j0 = S.j0, jj = j - j0;
     const int nb = a.nb;
     const int lane = threadIdx.x & 31;
-    const int l = j + 1 + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (l >= G.n) return;
+    const int l0 = j + 1 + 2 * (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    if (l0 >= G.n) return;
     T* W = static_cast<T*>(a.YK) + G.y_off;
     const int64_t ld = G.ld;
     const int n = G.n;
     T* F = static_cast<T*>(a.F) + G.vec_off * nb;
     const T* gq = static_cast<const T*>(a.gv) + (int64_t)blockIdx.y * QPB;
     const T tau = (T)S.tau;
-    T* col = W + ld * l;
+    const bool two = l0 + 1 < n;
+    const T* c0 = W + ld * l0;
+    const T* c1 = two ? c0 + ld : c0;
     const T* v = W + ld * j;
-    T dot = T(0);
-    for (int i = j + 1 + lane; i < G.m; i += 32) dot += v[i] * col[i];
-    dot = warp_sum(dot);
-    if (lane == 0) {
-        dot += col[j];
+    T d0 = T(0), d1 = T(0);
+    int i = j + 1 + lane;
+    constexpr int U = sizeof(T) == 4 ? 8 : 4;       // rows in flight per lane and column
+    for (; i + 32 * (U - 1) < G.m; i += 32 * U) {
+        T vv[U], x0[U], x1[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            x0[u] = c0[i + 32 * u];
+            x1[u] = c1[i + 32 * u];
+            vv[u] = v[i + 32 * u];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            d0 += vv[u] * x0[u];
+            d1 += vv[u] * x1[u];
+        }
+    }
+    for (; i < G.m; i += 32) {
+        d0 += v[i] * c0[i];
+        d1 += v[i] * c1[i];
+    }
+    d0 = warp_sum(d0);
+    d1 = warp_sum(d1);
+    if (lane < (two ? 2 : 1)) {
+        const int l = l0 + lane;
+        T* col = W + ld * l;
+        const T dot = (lane == 0 ? d0 : d1) + col[j];
         T corr = T(0);
+#pragma unroll 4
         for (int q = 0; q < jj; ++q) corr += F[l + (int64_t)n * q] * gq[q];
         const T f = tau * (dot - corr);
         F[l + (int64_t)n * jj] = f;
         // pivot row: W[j, l] -= sum_{q < jj} W[j, j0 + q] F[l, q] + F[l, jj]
         T r = col[j] - f;
+#pragma unroll 4
         for (int q = 0; q < jj; ++q) r -= W[j + ld * (j0 + q)] * F[l + (int64_t)n * q];
         col[j] = r;
         double* nrm = a.nrm + G.vec_off;
@@ -664,11 +776,24 @@ cudaError_t big_qp_panel(const BigArgs& a, int ngroups, int max_n, int max_m, in
     if (a.nb < 1 || a.nb > QPB) return cudaErrorInvalidValue;
     note_launch();
     bqp_start_kernel<<<(ngroups + 127) / 128, 128, 0, st>>>(a, ngroups);
+    int cl = 1;
+    while (cl < 8 && 2 * cl * ngroups <= 2 * a.num_sms && max_m > 1024 * cl) cl *= 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(ngroups * cl));
+    cfg.blockDim = dim3(QPT);
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)cl;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = cl > 1 ? 1 : 0;
     for (int jj = 0; jj < a.nb; ++jj, ++step) {
         note_launch();
-        bqp_pivot_kernel<T><<<ngroups, QPT, 0, st>>>(a, step);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, bqp_pivot_kernel<T>, a, step, cl);
+        if (e != cudaSuccess) return e;
         note_launch();
-        bqp_f_kernel<T><<<dim3((max_n + 7) / 8, ngroups), 256, 0, st>>>(a, step);
+        bqp_f_kernel<T><<<dim3((max_n + 15) / 16, ngroups), 256, 0, st>>>(a, step);
     }
     note_launch();
     bqp_update_kernel<T><<<dim3((max_m + 63) / 64, (max_n + 63) / 64, ngroups), 256, 0, st>>>(a);
@@ -1179,24 +1304,6 @@ constexpr size_t kFactorSmemMax = 224 * 1024;
 template <typename T>
 size_t be_factor_smem(int r, int cl) {
     return (size_t)((r + cl - 1) / cl) * r * sizeof(T) + 2 * (size_t)r * sizeof(T) + 2 * (size_t)r * sizeof(int) + 64;
-}
-
-__device__ __forceinline__ uint32_t cl_peer(const void* p, int rank) {
-    uint32_t out;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    return out;
-}
-__device__ __forceinline__ void cl_store(uint32_t a, double v) {
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
-}
-__device__ __forceinline__ void cl_store(uint32_t a, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-}
-__device__ __forceinline__ void cl_store(uint32_t a, int v) {
-    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ void cl_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // largest v, then lowest pos, over the warp; id follows (-1: no candidate)

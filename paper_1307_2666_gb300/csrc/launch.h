@@ -171,6 +171,7 @@ struct BigArgs {
     void* gv;
     double* nrm0;
     int nb;
+    int num_sms;
 };
 
 template <typename T> cudaError_t big_ygen(const BigArgs&, int nbig, int64_t max_entries, cudaStream_t);
