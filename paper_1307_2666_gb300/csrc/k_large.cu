@@ -1296,7 +1296,8 @@ __global__ void be_probs_kernel(BatchElimArgs a, int op, TcGemmProb* out) {
 // the lowest position as they do there.  Output in position order: LU (L
 // strictly below the diagonal), or for LDL boxes L below, D, and D L^T above.
 // Measured on a GB300 against the one-CTA and panel kernels this replaces: a
-// 64-bit LDL block of 388 rows 60 -> 3 ms with all its stages.
+// 64-bit LDL block of 388 rows 60 -> 8 ms with all its stages, and 4 with the
+// searches on integers and one reciprocal per step.
 constexpr int FT = 512;
 constexpr int FCL = 8;                       // largest cluster
 constexpr size_t kFactorSmemMax = 224 * 1024;
@@ -1316,6 +1317,23 @@ __device__ __forceinline__ void warp_best(T& v, int& pos, int& id) {
     }
 }
 
+// |v| as an integer of the same order: comparing these costs no FP64 operation
+// (64 cycles of a scheduler each; the searches were half of a 64-bit step)
+__device__ __forceinline__ long long abs_key(double v) { return __double_as_longlong(v) & 0x7fffffffffffffffLL; }
+__device__ __forceinline__ long long abs_key(float v) { return __float_as_int(v) & 0x7fffffff; }
+template <typename T> constexpr long long kInfKey = sizeof(T) == 8 ? 0x7ff0000000000000LL : 0x7f800000LL;
+// largest key, then lowest pos, over the warp; id follows (-1: no candidate)
+__device__ __forceinline__ void warp_best_key(long long& v, int& pos, int& id) {
+    for (int o = 16; o; o >>= 1) {
+        const long long v2 = __shfl_xor_sync(0xffffffffu, v, o);
+        const int p2 = __shfl_xor_sync(0xffffffffu, pos, o), i2 = __shfl_xor_sync(0xffffffffu, id, o);
+        if (i2 >= 0 && (id < 0 || v2 > v || (v2 == v && p2 < pos))) { v = v2; pos = p2; id = i2; }
+    }
+}
+__device__ __forceinline__ void cl_store(uint32_t a, long long v) {
+    asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
+
 template <typename T>
 __global__ void __launch_bounds__(FT) be_factor_kernel(BatchElimArgs a, int cl) {
     const int e = blockIdx.x / cl, rank = blockIdx.x % cl;
@@ -1325,8 +1343,9 @@ __global__ void __launch_bounds__(FT) be_factor_kernel(BatchElimArgs a, int cl) 
     const int64_t ld = d.k + r;
     T* Ag = static_cast<T*>(a.ws) + d.ws_off;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ T cval[2][FCL];
-    __shared__ int cid[2][FCL], cpos[2][FCL];
+    __shared__ long long cval[2][FCL];
+    __shared__ int cid[2][FCL], cpos[2][FCL], cstat[2], spiv;
+    __shared__ T cinv[2], sinv;
     const int own = (r - rank + cl - 1) / cl;         // columns rank, rank + cl, ...
     T* A = reinterpret_cast<T*>(smem_raw);            // A[i + r * s]: column rank + cl * s
     T* col = A + (size_t)((r + cl - 1) / cl) * r;     // col[r * parity + i]
@@ -1341,18 +1360,17 @@ __global__ void __launch_bounds__(FT) be_factor_kernel(BatchElimArgs a, int cl) 
     for (int j = 0; j < r; ++j) {
         T* c = col + r * (j & 1);
         int p;
-        T inv;
         if (d.ldl) {
             // remaining diagonal entry of largest magnitude
             if (warp == 0) {
-                T v = T(-1);
+                long long v = -1;
                 int ps = 0, id = -1;
                 for (int s = lane; s < own; s += 32) {
                     const int q = rank + cl * s, pq = pos[q];
-                    const T x = fabs(A[q + r * s]);
-                    if (pq >= j && (id < 0 ? x == x : x > v || (x == v && pq < ps))) { v = x; ps = pq; id = q; }
+                    const long long x = abs_key(A[q + r * s]);
+                    if (pq >= j && x <= kInfKey<T> && (id < 0 || x > v || (x == v && pq < ps))) { v = x; ps = pq; id = q; }
                 }
-                warp_best(v, ps, id);
+                warp_best_key(v, ps, id);
                 if (lane < cl) {
                     cl_store(cl_peer(&cval[j & 1][rank], lane), v);
                     cl_store(cl_peer(&cpos[j & 1][rank], lane), ps);
@@ -1361,11 +1379,11 @@ __global__ void __launch_bounds__(FT) be_factor_kernel(BatchElimArgs a, int cl) 
             }
             if (cl > 1) cl_sync();
             else __syncthreads();
-            T v = T(-1);
+            long long v = -1;
             int ps = 0;
             p = -1;
             for (int q = 0; q < cl; ++q) {
-                const T x = cval[j & 1][q];
+                const long long x = cval[j & 1][q];
                 const int pq = cpos[j & 1][q], id = cid[j & 1][q];
                 if (id >= 0 && (p < 0 || x > v || (x == v && pq < ps))) { v = x; ps = pq; p = id; }
             }
@@ -1376,33 +1394,39 @@ __global__ void __launch_bounds__(FT) be_factor_kernel(BatchElimArgs a, int cl) 
                     const T x = pos[i] >= j ? src[i] : T(0);
                     for (int q = 0; q < cl; ++q) cl_store(cl_peer(c + i, q), x);
                 }
+                if (warp == 0) {                      // the pivot's test and reciprocal, for all
+                    long long cm = 0;
+                    for (int i = lane; i < r; i += 32)
+                        if (i != p && pos[i] >= j) cm = max(cm, abs_key(src[i]));
+                    for (int o = 16; o; o >>= 1) cm = max(cm, __shfl_xor_sync(0xffffffffu, cm, o));
+                    const T dp = src[p], m = sizeof(T) == 8 ? (T)__longlong_as_double(cm) : (T)__int_as_float((int)cm);
+                    const long long kd = abs_key(dp);
+                    const int st = kd == 0 || kd >= kInfKey<T> ? 2 : fabs(dp) >= (T)a.ldl_alpha * m ? 0 : 1;
+                    const T iv = T(1) / dp;
+                    if (lane < cl) {
+                        cl_store(cl_peer(&cstat[j & 1], lane), st);
+                        cl_store(cl_peer(&cinv[j & 1], lane), iv);
+                    }
+                }
             }
             if (cl > 1) cl_sync();
             else __syncthreads();
-            const T dp = c[p];
-            T cm = T(0);
-            for (int i = lane; i < r; i += 32)
-                if (i != p) cm = fmax(cm, fabs(c[i]));
-            for (int o = 16; o; o >>= 1) cm = fmax(cm, __shfl_xor_sync(0xffffffffu, cm, o));
-            if (dp == T(0) || !isfinite((double)dp)) {
-                if (rank == 0 && threadIdx.x == 0) atomicOr(a.status, (int)DEV_SINGULAR);
-                break;
-            }
-            if (!(fabs(dp) >= (T)a.ldl_alpha * cm)) {
+            const int st = cstat[j & 1];
+            if (st != 0) {
                 if (rank == 0 && threadIdx.x == 0) {
-                    atomicOr(a.status, (int)DEV_LDL_FALLBACK);
-                    a.ldl_fail[a.fail_idx[e]] = 1;
+                    atomicOr(a.status, st == 2 ? (int)DEV_SINGULAR : (int)DEV_LDL_FALLBACK);
+                    if (st == 1) a.ldl_fail[a.fail_idx[e]] = 1;
                 }
                 break;
             }
-            inv = T(1) / dp;
+            const T inv = cinv[j & 1];
             for (int s = warp; s < own; s += NW) {
                 const int q = rank + cl * s;
                 if (pos[q] < j || q == p) continue;
-                const T vq = c[q];
+                const T f = c[q] * inv;
                 T* x = A + (size_t)r * s;
                 for (int i = lane; i < r; i += 32)
-                    if (i != p) x[i] -= c[i] * vq * inv;
+                    if (i != p) x[i] -= c[i] * f;
             }
             if (p % cl == rank) {
                 T* x = A + (size_t)r * (p / cl);
@@ -1414,24 +1438,29 @@ __global__ void __launch_bounds__(FT) be_factor_kernel(BatchElimArgs a, int cl) 
             if (j % cl == rank) {
                 T* x = A + (size_t)r * (j / cl);
                 if (warp == 0) {
-                    T v = T(-1);
+                    long long v = -1;
                     int ps = 0, id = -1;
                     for (int i = lane; i < r; i += 32) {
-                        const T y = fabs(x[i]);
+                        const long long y = abs_key(x[i]);
                         const int pi = pos[i];
-                        if (pi >= j && (id < 0 ? y == y : y > v || (y == v && pi < ps))) { v = y; ps = pi; id = i; }
+                        if (pi >= j && y <= kInfKey<T> && (id < 0 || y > v || (y == v && pi < ps))) { v = y; ps = pi; id = i; }
                     }
-                    warp_best(v, ps, id);
+                    warp_best_key(v, ps, id);
                     if (id < 0) id = at[j];           // (all NaN: the pivot test below fails)
+                    const long long kd = abs_key(x[id]);
                     if (lane < cl) {
                         cl_store(cl_peer(&cid[j & 1][0], lane), id);
-                        cl_store(cl_peer(&cval[j & 1][0], lane), x[id]);
+                        cl_store(cl_peer(&cstat[j & 1], lane), kd == 0 || kd >= kInfKey<T> ? 2 : 0);
                     }
-                    if (lane == 0) cpos[0][1] = id;
+                    const T iv = T(1) / x[id];
+                    if (lane == 0) {
+                        spiv = id;
+                        sinv = iv;
+                    }
                 }
                 __syncthreads();
-                const int pp = cpos[0][1];
-                const T pinv = T(1) / x[pp];
+                const int pp = spiv;
+                const T pinv = sinv;
                 for (int i = threadIdx.x; i < r; i += FT) {
                     const bool on = pos[i] >= j && i != pp;
                     const T l = on ? x[i] * pinv : T(0);
@@ -1442,8 +1471,7 @@ __global__ void __launch_bounds__(FT) be_factor_kernel(BatchElimArgs a, int cl) 
             if (cl > 1) cl_sync();
             else __syncthreads();
             p = cid[j & 1][0];
-            const T dp = cval[j & 1][0];
-            if (dp == T(0) || !isfinite((double)dp)) {
+            if (cstat[j & 1] != 0) {
                 if (rank == 0 && threadIdx.x == 0) atomicOr(a.status, (int)DEV_SINGULAR);
                 break;
             }
