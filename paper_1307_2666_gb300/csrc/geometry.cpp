@@ -48,7 +48,7 @@ static void stable_bucket(const int64_t* key, int64_t n, int64_t nkeys, std::vec
     off.assign(nkeys + 1, 0);
     int nch = 1;
 #ifdef _OPENMP
-    nch = omp_get_max_threads();
+    nch = omp_in_parallel() ? 1 : omp_get_max_threads();
 #endif
     if (n < 65536 || (int64_t)nch * nkeys > ((int64_t)1 << 22)) nch = 1;
     if (nch == 1) {
@@ -460,7 +460,7 @@ void build_near_groups(const Tree& t, const double* x, int s, double proxy_radiu
     const int nb = p.nbox;
     int nthr = 1;
 #ifdef _OPENMP
-    nthr = omp_get_max_threads();
+    nthr = omp_in_parallel() ? 1 : omp_get_max_threads();     // (one problem of several, planned side by side)
 #endif
     std::vector<NearScratch> scr(nthr);
     if (cache) {
@@ -479,7 +479,7 @@ void build_near_groups(const Tree& t, const double* x, int s, double proxy_radiu
     // chunks of up to 16 boxes, but at least ~8 chunks per thread, so that the
     // few-box sublevels near the top spread over all threads
     const int chunk = std::max(1, std::min(16, nb / (8 * nthr)));
-#pragma omp parallel for schedule(dynamic, chunk)
+#pragma omp parallel for schedule(dynamic, chunk) num_threads(nthr)
     for (int b = 0; b < nb; ++b) {
         int tid = 0;
 #ifdef _OPENMP
@@ -706,10 +706,13 @@ void build_near_groups(const Tree& t, const double* x, int s, double proxy_radiu
             cache->epoch[q] = scr[q].epoch;
         }
     if (tr) {
+#pragma omp critical(hif_geometry_trace)
+        {
         g_geo_ms[0] += tb1 - tb0;                      // bins and set-up (wall)
         g_geo_ms[1] += now_ms() - tb2;                 // gather (wall)
         for (const NearScratch& S : scr)               // per-box phases (thread time)
             for (int q = 0; q < 4; ++q) g_geo_ms[2 + q] += S.ms[q];
+        }
     }
 }
 
