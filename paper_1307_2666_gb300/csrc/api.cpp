@@ -1749,7 +1749,7 @@ static void matvec_dev(hif_handle h, int trans, const double* x, int64_t ldx, do
                                              sg.tc_tmax.as<unsigned long long>(), sg.tc_rows.p, st));
                 }
                 h->tc_xb.ensure(tc_source_digits_bytes(sg.gn, h->dim, h->num_sms));
-                h->tc_xmax.ensure(8 * sizeof(unsigned long long));
+                h->tc_xmax.ensure(9 * sizeof(unsigned long long));
                 h->tc_status.ensure(sizeof(int));
                 HIF_CUDA(cudaMemsetAsync(h->tc_status.p, 0, sizeof(int), st));
                 {

@@ -58,13 +58,20 @@
 // built by threads from L2 (two loads, an add and a store per 16 bytes).
 // Measured on a GB300, whole matvec, before (one MMA quarter per source line,
 // 8-column padding, whole tiles per CTA) and after: n = 1024 x 8 right-hand
-// sides 458 -> 281 ms (classes 6, 5, 4: 357, 290, 248 -> 236, 208, 162 ms),
-// n = 512 x 8 30.8 -> 17.7 ms, n = 64 x 1 0.29 -> 0.15 ms, 3D n = 24 x 3
-// 2.8 -> 0.94 ms.
+// sides 458 -> 272 ms (classes 6, 5, 4: 357, 290, 248 -> 222, 190, 152 ms; with
+// two drains per slot, see below, 281, 236, 208 and 162), n = 512 x 8 30.8 ->
+// 17.5 ms, n = 64 x 1 0.29 -> 0.16 ms, 3D n = 24 x 3 2.8 -> 0.94 ms.
 //
-// A column sums at most 7 pairs x 64 sources x 2^15 < 2^24 products, exact in
-// FP32, so a slot fills the two accumulators in turn, 64 sources each, and
-// the epilogue drains one while the MMAs fill the other.
+// The epilogue's conversions of column sums to integers run at 16 per clock, so
+// how often a column is drained matters (a drain per 64 sources is 4,096
+// cycles a slot at 8 classes).  A column sums products of a table digit (at most
+// 128) and a folded source digit; over the 128 sources of a slot that is below
+// 2^24, exact in FP32, whenever the digits of every source chunk satisfy
+// sum_t sum_q |d_t[q]| <= 2^16 (kFullSlot).  Random digits do (mean 57,300 of 7
+// digits, spread 1,100); the digit kernel finds the largest sum, and the two
+// accumulators then take a slot each.  Otherwise (coherent sources) they take
+// half a slot each: 7 pairs x 64 sources x 2^15 < 2^24 for any digits.  The
+// epilogue drains one while the MMAs fill the other.
 //
 // The slots of all tiles form one sequence (tile, middle source coordinate,
 // source chunk, distance) that is cut into equal ranges, one per CTA, so
@@ -122,6 +129,10 @@ constexpr int PART = NGRP * 8 * NEPI;           // int64 values of one partial t
 constexpr long long WAIT_CYCLES = 4000000000LL; // ~2 s at GB300 clocks
 
 static_assert(7 * (KC / NACC) * 128 * 256 <= (1 << 24), "exact FP32 accumulation of half a slot");
+// largest sum of |digit| over a source chunk's digits (the first SUMT) for
+// which a whole slot is exact: two chunks are added, table digits are <= 128
+constexpr unsigned kFullSlot = (1u << 24) / 2 / 128;
+constexpr int SUMT = 7;                         // most digit pairs of a class
 // S[1] gains less than 2 x 2^24 x (2^24 + 2^17) per slot
 static_assert(4294967296.0 * 65536.0 * 2.1 * CARRY < 9.2e18, "64-bit class sums between carries");
 
@@ -175,7 +186,7 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
 struct Bars {
     uint64_t full[NST_MAX];     // both operands built (NBUILD arrivals)
     uint64_t mma_done[NST_MAX];
-    uint64_t acc_full[NACC];    // accumulator written (1 commit)
+    uint64_t acc_full[NACC];    // accumulator written (1 commit); taken in turn
     uint64_t acc_empty[NACC];   // accumulator drained (NEPI arrivals)
     uint64_t drain;
     uint32_t tmem;
@@ -236,37 +247,56 @@ __global__ void tc_table_rows_kernel(const double* table, int n, int64_t lines, 
 // use): element (digit t, rhs r, source q) of chunk ch at
 // (((ch * SX + t) * (KC/8) + q/8) * nrv + r) * 8 + q % 8 (BF16 units).
 __global__ void tc_source_digits_kernel(const double* v, int64_t N, int n, int64_t lines, int nc, int r0, int nr,
-                                        int lg, int sx, int xshift, const unsigned long long* xmax, uint4* XB) {
+                                        int lg, int sx, int xshift, const unsigned long long* xmax, uint4* XB,
+                                        unsigned* chunk_max) {
     const int64_t tot = (lines * nc * (KC / 8)) << lg;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(e & ((1 << lg) - 1));
-        const int kb = (int)((e >> lg) % (KC / 8));
-        const int64_t ch = (e >> lg) / (KC / 8);
-        const int64_t J = ch / nc;
-        const int c = (int)(ch % nc);
-        float d[8][8];                               // [source][digit]
-        const int ex = (r < nr ? scale_exp(xmax[r]) : 0) + xshift;
+    __shared__ unsigned sums[256];               // sum of |digit| per (chunk, rhs) of this block
+    unsigned most = 0;
+    for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x; e0 < tot; e0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = e0 + threadIdx.x;
+        sums[threadIdx.x] = 0;
+        __syncthreads();
+        if (e < tot) {
+            const int r = (int)(e & ((1 << lg) - 1));
+            const int kb = (int)((e >> lg) % (KC / 8));
+            const int64_t ch = (e >> lg) / (KC / 8);
+            const int64_t J = ch / nc;
+            const int c = (int)(ch % nc);
+            float d[8][8];                       // [source][digit]
+            const int ex = (r < nr ? scale_exp(xmax[r]) : 0) + xshift;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int64_t jl = (int64_t)KC * c + 8 * kb + q;
-            if (r < nr && jl < n) {
-                digits8(ldexp(v[J * n + jl + N * (r0 + r)], -ex), d[q]);
-            } else {
+            for (int q = 0; q < 8; ++q) {
+                const int64_t jl = (int64_t)KC * c + 8 * kb + q;
+                if (r < nr && jl < n) {
+                    digits8(ldexp(v[J * n + jl + N * (r0 + r)], -ex), d[q]);
+                } else {
 #pragma unroll
-                for (int t = 0; t < 8; ++t) d[q][t] = 0.f;
+                    for (int t = 0; t < 8; ++t) d[q][t] = 0.f;
+                }
             }
-        }
+            float sum = 0.f;
 #pragma unroll
-        for (int t = 0; t < SX; ++t) {
-            if (t >= sx) break;
-            uint4 w;
-            w.x = pack2(d[0][t], d[1][t]);
-            w.y = pack2(d[2][t], d[3][t]);
-            w.z = pack2(d[4][t], d[5][t]);
-            w.w = pack2(d[6][t], d[7][t]);
-            XB[(((ch * SX + t) * (KC / 8) + kb) << lg) + r] = w;
+            for (int t = 0; t < SX; ++t) {
+                if (t >= sx) break;
+                uint4 w;
+                w.x = pack2(d[0][t], d[1][t]);
+                w.y = pack2(d[2][t], d[3][t]);
+                w.z = pack2(d[4][t], d[5][t]);
+                w.w = pack2(d[6][t], d[7][t]);
+                XB[(((ch * SX + t) * (KC / 8) + kb) << lg) + r] = w;
+                if (t < SUMT)
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) sum += fabsf(d[q][t]);
+            }
+            // (chunk in the block, rhs): a chunk's 16 << lg threads are neighbours
+            atomicAdd(&sums[((threadIdx.x >> lg) / (KC / 8) << lg) + r], (unsigned)sum);
         }
+        __syncthreads();
+        most = max(most, sums[threadIdx.x]);
+        __syncthreads();
     }
+    for (int o = 16; o; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+    if (threadIdx.x % 32 == 0 && most > 0) atomicMax(chunk_max, most);
 }
 
 // ---- the tensor-core sum ----------------------------------------------------
@@ -275,7 +305,7 @@ struct TcConvArgs {
     const __nv_bfloat16* R;     // mirrored table digit rows
     const unsigned char* XB;    // source digit chunks
     const unsigned long long* tmax;
-    const unsigned long long* xmax;   // NR entries
+    const unsigned long long* xmax;   // NR entries, then the largest chunk sum of |digit|
     double* ybuf;               // N x nrhs, grid order
     long long* part;            // two partial tiles per CTA
     int64_t N;
@@ -413,6 +443,8 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
     const uint32_t tmem = bars->tmem;
     const int64_t first = range_start(a, blockIdx.x, gridDim.x);
     const int64_t count = range_start(a, blockIdx.x + 1, gridDim.x) - first;
+    // a whole slot per accumulator, or half of one
+    const bool whole = *reinterpret_cast<const unsigned*>(a.xmax + NR) <= kFullSlot;
 
     if (warp == NEPI / 32) {
         // ---------------------------------------------------------- issuer
@@ -423,6 +455,7 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
             int st = 0;
             uint32_t ph = 0;
             bool ok = true;
+            int64_t use = 0;                     // accumulators filled
             for (int64_t si = 0; si < (a.stall ? 0 : count); ++si) {
                 if (!wait_bounded(&bars->full[st], ph, abort)) {
                     ok = false;
@@ -434,30 +467,30 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
                 const uint32_t a_st = tc::smem_addr(smem + st * STAGE);
                 const uint64_t a0 = tc::sdesc(a_st, CM, CM);
                 const uint64_t b0 = tc::sdesc(a_st + A_BYTES, 128, (KC / 8) * 128);
-#pragma unroll
-                for (int h = 0; h < NACC; ++h) {
-                    if (si >= 1 && !wait_bounded(&bars->acc_empty[h], (uint32_t)((si - 1) & 1), abort)) {
-                        ok = false;
-                        break;
-                    }
+                // slice by slice: consecutive MMAs of one slice read
+                // overlapping Hankel windows and keep N and D fixed, which
+                // the tensor core streams faster than alternating slices
+                // (the first MMA, slice 0 with every column, initializes
+                // the accumulator; the others add into it)
+                auto fill = [&](int k0, int k1) {
+                    const int ab = (int)(use & 1);
+                    if (use >= NACC && !wait_bounded(&bars->acc_empty[ab], (uint32_t)((use / NACC - 1) & 1), abort))
+                        return false;
                     tc::tc_fence_after();
-                    // slice by slice: consecutive MMAs of one slice read
-                    // overlapping Hankel windows and keep N and D fixed, which
-                    // the tensor core streams faster than alternating slices
-                    // (the first MMA, slice 0 with every column, initializes
-                    // the accumulator; the others add into it)
 #pragma unroll
                     for (int s = 0; s < C::ST; ++s) {
                         const uint64_t as = a0 + (uint64_t)(s * A_SLICE / 16);
-                        const uint32_t dst = tmem + ACCB * h + coloff(s);
-#pragma unroll
-                        for (int kk = h * (KC / 16 / NACC); kk < (h + 1) * (KC / 16 / NACC); ++kk)
-                            tc::mma_bf16(dst, as + (uint64_t)(2 * CM * kk / 16), b0 + (uint64_t)(16 * kk),
-                                         tc::idesc_bf16_f32(TM, C::ncols(s)),
-                                         !(s == 0 && kk == h * (KC / 16 / NACC)));
+                        const uint32_t dst = tmem + ACCB * ab + coloff(s);
+#pragma unroll 4
+                        for (int kk = k0; kk < k1; ++kk)
+                            tc::mma_bf16(dst, as + (uint64_t)(2 * CM / 16) * kk, b0 + (uint64_t)16 * kk,
+                                         tc::idesc_bf16_f32(TM, C::ncols(s)), !(s == 0 && kk == k0));
                     }
-                    tc::mma_commit(&bars->acc_full[h]);
-                }
+                    tc::mma_commit(&bars->acc_full[ab]);
+                    ++use;
+                    return true;
+                };
+                ok = whole ? fill(0, KC / 16) : fill(0, KC / 32) && fill(KC / 32, KC / 16);
                 if (!ok) break;
                 tc::mma_commit(&bars->mma_done[st]);
                 if (++st == NST) {
@@ -571,7 +604,8 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
         const int quad = warp & 3, cg = warp >> 2;
         const int row = 32 * quad + lane;
         long long S[8][NGRP];
-        uint32_t ph = 0;
+        const int nh = whole ? 1 : NACC;
+        unsigned use = 0;                        // accumulators drained (mod 2^32)
         bool ok = true;
         const Tiles tl(a);
         Place pl(tl, first);
@@ -584,14 +618,14 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
                 for (int g = 0; g < NGRP; ++g) S[e][g] = 0;
             for (int s = 0; s < nsl && ok; ++s) {
 #pragma unroll 1                                // (unrolled, the sums spill)
-                for (int h = 0; h < NACC; ++h) {
+                for (int h = 0; h < nh; ++h, ++use) {
                     // (a warp gives up as one: the TMEM loads below are collective)
-                    if (!__all_sync(0xffffffffu, wait_bounded(&bars->acc_full[h], ph, abort))) {
+                    if (!__all_sync(0xffffffffu, wait_bounded(&bars->acc_full[use & 1], (uint32_t)(use >> 1) & 1, abort))) {
                         ok = false;
                         break;
                     }
                     tc::tc_fence_after();
-                    const uint32_t tbase = tmem + ACCB * h + 8 * cg + ((uint32_t)(32 * quad) << 16);
+                    const uint32_t tbase = tmem + ACCB * (use & 1) + 8 * cg + ((uint32_t)(32 * quad) << 16);
 #pragma unroll
                     for (int k = 0; k < KD; k += 2) {
                         float v[2][8];
@@ -607,9 +641,8 @@ __global__ void __launch_bounds__(NTHR, 1) tc_conv_kernel(TcConvArgs a) {
                             }
                     }
                     tc::tc_fence_before();
-                    tc::mbar_arrive(&bars->acc_empty[h]);
+                    tc::mbar_arrive(&bars->acc_empty[use & 1]);
                 }
-                ph ^= 1;
                 if (s % CARRY == CARRY - 1 || s == nsl - 1) {
 #pragma unroll
                     for (int e = 0; e < 8; ++e) carry(S[e]);
@@ -778,7 +811,7 @@ cudaError_t launch_direct_grid_tc(const GridDirectArgs& a, const void* R, const 
     while ((N >> xshift) > ((int64_t)1 << 24)) ++xshift;
     for (int r0 = 0; r0 < a.nrhs; r0 += NR) {
         const int nr = std::min(NR, a.nrhs - r0);
-        cudaError_t e = cudaMemsetAsync(xmax, 0, NR * sizeof(unsigned long long), st);
+        cudaError_t e = cudaMemsetAsync(xmax, 0, (NR + 1) * sizeof(unsigned long long), st);
         if (e != cudaSuccess) return e;
         note_launch();
         tc_maxabs_kernel<<<(int)std::min<int64_t>((N + 255) / 256, 1024), 256, 0, st>>>(a.vbuf + N * r0, N, nr, N,
@@ -789,7 +822,8 @@ cudaError_t launch_direct_grid_tc(const GridDirectArgs& a, const void* R, const 
         const int64_t items = (lines * nc * (KC / 8)) << lg;
         note_launch();
         tc_source_digits_kernel<<<(int)std::min<int64_t>((items + 255) / 256, 152 * 16), 256, 0, st>>>(
-            a.vbuf, N, a.n, lines, nc, r0, nr, lg, classes, xshift, xmax, (uint4*)XB);
+            a.vbuf, N, a.n, lines, nc, r0, nr, lg, classes, xshift, xmax, (uint4*)XB,
+            (unsigned*)(xmax + NR));
         TcConvArgs t{};
         t.R = (const __nv_bfloat16*)R;
         t.XB = (const unsigned char*)XB;

@@ -339,7 +339,7 @@ void grid_finish_kernel_launch(const GridDirectArgs&, int64_t N, int eb, cudaStr
 // same sum on the tensor cores in exact 8-bit digits (k_tcconv.cu):
 // R = mirrored table digit rows (tc_table_rows_bytes), built once per grid by
 // launch_tc_table with tmax its max |entry|; XB = tc_source_digits_bytes of
-// scratch, xmax 8 entries, status one int (set to 1 if a wait expired)
+// scratch, xmax 9 entries, status one int (set to 1 if a wait expired)
 size_t tc_table_rows_bytes(int n, int dim);
 size_t tc_source_digits_bytes(int n, int dim, int num_sms);
 cudaError_t launch_tc_table(const double* table, int n, int dim, unsigned long long* tmax, void* R,
