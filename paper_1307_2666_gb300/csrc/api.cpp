@@ -896,7 +896,7 @@ static void run_factor(hif_handle h) {
     SciHost sci;
     std::vector<char> active(N, 1);
     std::vector<int> box_of(N, -1);
-    DevMem d_boxes, d_groups, d_cols, d_near, Rws, GKws, GSws, Tws, Wws, Woff, perm_out, k_out;
+    DevMem d_boxes, d_groups, d_cols, d_near, Rws, GKws, GSws, GPws, Tws, Wws, Woff, perm_out, k_out;
     DevMem d_small_boxes, d_small_groups, d_small_sorted, id_counter;
     FactorScratch S;
     BigBuffers big, bigR;
@@ -1092,9 +1092,9 @@ static void run_factor(hif_handle h) {
         Rws.ensure(sizeof(T) * std::max<int64_t>(Roff, 1));
         // small boxes by width bucket, and the CTAs per box of each
         const bool grams = h->second_kind && any_sci;
-        struct Bucket { FoldArgs fa; int count, w, cpt, rc; size_t smem; };
+        struct Bucket { FoldArgs fa; int count, w, cpt, rc; size_t smem; int64_t gram_at; };
         std::vector<Bucket> buckets;
-        int max_split = 1;
+        int64_t gram_part = 0;              // values of the Grams of split boxes' ranks 1..
         {
             int64_t at = 0;
             const int widths[] = {32, 64, 96, 128, 160, 192, 224, 256, 512, 1024};
@@ -1109,7 +1109,7 @@ static void run_factor(hif_handle h) {
                 if (at == b0) continue;
                 const int cpt = fold_cpt(w, (int)sizeof(T));
                 if (cpt == 0) fail(HIF_EINVAL, "box too wide for the fold kernel");
-                Bucket bk{FoldArgs{}, (int)(at - b0), w, cpt, 0, 0};
+                Bucket bk{FoldArgs{}, (int)(at - b0), w, cpt, 0, 0, 0};
                 bk.fa.box_list = d_small_sorted.as<int>() + b0;
                 bk.smem = fold_smem_bytes(w, cpt, grams, true, sizeof(T));
                 bk.fa.R_in_smem = bk.smem <= 220 * 1024;
@@ -1119,14 +1119,17 @@ static void run_factor(hif_handle h) {
                                   ? fold_split(w, (pairs / bk.count + 31) / 32, bk.count, h->num_sms, (int)sizeof(T))
                                   : 1;
                 if (const int fs = env_int("HIF_FOLD_SPLIT", 0); fs > 0 && cpt == 1 && bk.fa.R_in_smem) bk.fa.split = fs;
-                max_split = std::max(max_split, bk.fa.split);
+                bk.fa.gram_size = (int64_t)w * w;
+                bk.gram_at = gram_part;
+                gram_part += 2 * (int64_t)(bk.fa.split - 1) * bk.count * bk.fa.gram_size;
                 buckets.push_back(bk);
             }
             if (at != (int64_t)small_boxes.size()) fail(HIF_EINVAL, "box too wide for the fold kernel");
         }
         if (grams) {
-            GKws.ensure(sizeof(T) * Roff * max_split);
-            GSws.ensure(sizeof(T) * Roff * max_split);
+            GKws.ensure(sizeof(T) * Roff);
+            GSws.ensure(sizeof(T) * Roff);
+            GPws.ensure(sizeof(T) * std::max<int64_t>(gram_part, 1));
         }
         Tws.ensure(sizeof(T) * std::max<int64_t>(Toff, 1));
         perm_out.ensure(sizeof(int) * std::max<size_t>(p.cols.size(), 1));
@@ -1160,7 +1163,8 @@ static void run_factor(hif_handle h) {
                     f.box_list = bk.fa.box_list;
                     f.R_in_smem = bk.fa.R_in_smem;
                     f.split = bk.fa.split;
-                    f.gram_stride = Roff;
+                    f.gram_size = bk.fa.gram_size;
+                    f.gram_part = grams ? GPws.as<T>() + bk.gram_at : nullptr;
                     bk.fa = f;
                 }
                 // autotune (synchronous, first sighting of a bucket only)

@@ -112,9 +112,12 @@ __global__ void __launch_bounds__(256, CPT == 1 ? 2 : 1) fold_kernel(FoldArgs ar
     T* CS = grams ? align_ptr<T>(sp, (size_t)RC * n) : nullptr;
     T* const Rglob = static_cast<T*>(args.Rws) + bx.R_off;
     T* const Rpack = args.R_in_smem ? align_ptr<T>(sp, (size_t)n * (n + 1) / 2) : nullptr;
-    // (each CTA of a split sums its own Grams; added up at the end)
-    T* GK = grams ? static_cast<T*>(args.GKws) + bx.R_off + rank * args.gram_stride : nullptr;
-    T* GS = grams ? static_cast<T*>(args.GSws) + bx.R_off + rank * args.gram_stride : nullptr;
+    // (each CTA of a split sums its own Grams, those of ranks 1.. in gram_part;
+    // added up at the end)
+    T* const part = static_cast<T*>(args.gram_part) +
+                    (int64_t)(blockIdx.x / nsplit) * (nsplit - 1) * 2 * args.gram_size;
+    T* GK = !grams ? nullptr : rank == 0 ? static_cast<T*>(args.GKws) + bx.R_off : part + (2 * rank - 2) * args.gram_size;
+    T* GS = !grams ? nullptr : rank == 0 ? static_cast<T*>(args.GSws) + bx.R_off : part + (2 * rank - 1) * args.gram_size;
 
     const double c0 = bx.ctr[0], c1 = bx.ctr[1], c2 = dim == 3 ? bx.ctr[2] : 0.0;
     // column data of this thread's columns
@@ -358,8 +361,8 @@ __global__ void __launch_bounds__(256, CPT == 1 ? 2 : 1) fold_kernel(FoldArgs ar
                 T* gs = static_cast<T*>(args.GSws) + bx.R_off + e;
                 T k = gk[0], v = gs[0];
                 for (int q = 1; q < nsplit; ++q) {
-                    k += gk[q * args.gram_stride];
-                    v += gs[q * args.gram_stride];
+                    k += part[(2 * q - 2) * args.gram_size + e];
+                    v += part[(2 * q - 1) * args.gram_size + e];
                 }
                 gk[0] = k;
                 gs[0] = v;

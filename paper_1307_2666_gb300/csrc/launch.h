@@ -23,7 +23,8 @@ struct FoldArgs {
     int second_kind;
     int R_in_smem;
     int split;                // CTAs (a cluster) per box, 1, 2, 4 or 8
-    int64_t gram_stride;      // between the Grams of the CTAs of a split
+    void* gram_part;          // Grams (K, S) of ranks 1.. of every box of the launch,
+    int64_t gram_size;        // gram_size values each
     void* Rws;
     void* GKws;
     void* GSws;
