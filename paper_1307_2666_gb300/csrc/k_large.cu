@@ -12,9 +12,9 @@
 //                    warp per remaining column applies it and brings the
 //                    column norm up to date in FP64 (kNormKeep);
 //  * big_T           T = R1^{-1} R2 and the skeleton / redundant order;
-//  * gemm / trsm / elimination helpers: Lemma 2.4 blocks, Lemma 2.1 LU
-//                    (blocked, multi-CTA) and the Schur update for one large
-//                    box at a time.
+//  * be_*            the batched elimination of medium and large boxes: Lemma
+//                    2.4 blocks, Lemma 2.1 LU or LDL, inverses and the Schur
+//                    update, one launch per stage for all of them.
 #include <algorithm>
 
 #include "hif_common.cuh"
@@ -948,171 +948,6 @@ cudaError_t big_finish(const BigArgs& a, int ngroups, int max_n, cudaStream_t st
     note_launch();
     big_T_kernel<T><<<g, 256, 0, st>>>(a);
     return cudaGetLastError();
-}
-
-// --------------------------------------------------- dense helpers ------
-
-// C (m x n) += alpha op(A) op(B); 64 x 64 tiles, K staged 16 at a time.
-template <typename T>
-__global__ void __launch_bounds__(256) gemm_kernel(int m, int n, int kk, T alpha, const T* A, int64_t lda, int tA,
-                                                   const T* B, int64_t ldb, int tB, T* C, int64_t ldc) {
-    __shared__ T As[16][64 + 1];
-    __shared__ T Bs[16][64 + 1];
-    const int i0 = blockIdx.x * 64, j0 = blockIdx.y * 64;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    T acc[4][4] = {};
-    for (int l0 = 0; l0 < kk; l0 += 16) {
-        for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-            const int r = e % 64, l = e / 64;           // A tile: rows i0+r, k l0+l
-            const int i = i0 + r, kx = l0 + l;
-            T v = T(0);
-            if (i < m && kx < kk) v = tA ? A[kx + lda * i] : A[i + lda * kx];
-            As[l][r] = v;
-            const int jj = j0 + r;                      // B tile: k l0+l, cols j0+r
-            T u = T(0);
-            if (jj < n && kx < kk) u = tB ? B[jj + ldb * kx] : B[kx + ldb * jj];
-            Bs[l][r] = u;
-        }
-        __syncthreads();
-        for (int l = 0; l < 16; ++l) {
-            T av[4], bv[4];
-            for (int q = 0; q < 4; ++q) av[q] = As[l][tx + 16 * q];
-            for (int q = 0; q < 4; ++q) bv[q] = Bs[l][ty + 16 * q];
-            for (int p = 0; p < 4; ++p)
-                for (int q = 0; q < 4; ++q) acc[p][q] += av[p] * bv[q];
-        }
-        __syncthreads();
-    }
-    for (int p = 0; p < 4; ++p)
-        for (int q = 0; q < 4; ++q) {
-            const int i = i0 + tx + 16 * p, jj = j0 + ty + 16 * q;
-            if (i < m && jj < n) C[i + ldc * jj] += alpha * acc[p][q];
-        }
-}
-
-template <typename T>
-cudaError_t gemm(int m, int n, int kk, T alpha, const T* A, int64_t lda, bool tA, const T* B, int64_t ldb, bool tB,
-                 T* C, int64_t ldc, cudaStream_t st) {
-    if (m == 0 || n == 0 || kk == 0) return cudaSuccess;
-    dim3 g((m + 63) / 64, (n + 63) / 64);
-    note_launch();
-    gemm_kernel<T><<<g, 256, 0, st>>>(m, n, kk, alpha, A, lda, tA ? 1 : 0, B, ldb, tB ? 1 : 0, C, ldc);
-    return cudaGetLastError();
-}
-
-template <typename T>
-__global__ void big_gather_kernel(GeomDev g, SciDev sci, const int* rd, int r, const int* sk, int k, T* A) {
-    const int n = k + r;
-    const int ref = r > 0 ? rd[0] : sk[0];
-    const int d = g.dim;
-    const double r0 = g.x[(int64_t)d * ref], r1 = g.x[(int64_t)d * ref + 1];
-    const double r2 = d == 3 ? g.x[(int64_t)d * ref + 2] : 0.0;
-    const int64_t tot = (int64_t)n * n;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-        const int p = (int)(e % n), q = (int)(e / n);
-        const int i = p < r ? rd[p] : sk[p - r];
-        const int j = q < r ? rd[q] : sk[q - r];
-        A[e] = entry<T>(g, sci, i, j, r0, r1, r2);
-    }
-}
-
-template <typename T>
-__global__ void big_T_assemble_kernel(const ElimGroup* eg, int ng, const T* Tws, int k, int r, T* Tm) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < k * r; e += gridDim.x * blockDim.x) Tm[e] = T(0);
-    __syncthreads();   // single-CTA launch
-    for (int gi = 0; gi < ng; ++gi) {
-        const ElimGroup G = eg[gi];
-        for (int e = threadIdx.x; e < G.kg * G.rg; e += blockDim.x) {
-            const int i = e % G.kg, jj = e / G.kg;
-            Tm[(G.ko + i) + (int64_t)k * (G.ro + jj)] = Tws[G.T_off + e];
-        }
-    }
-}
-
-// X (m x n) <- X U^{-1}, U upper with diagonal; one thread per row of X
-template <typename T>
-__global__ void trsm_right_upper_rows(int n, const T* U, int64_t ldu, T* X, int64_t ldx, int m) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
-    for (int j = 0; j < n; ++j) {
-        T v = X[i + ldx * j];
-        for (int l = 0; l < j; ++l) v -= X[i + ldx * l] * U[l + ldu * j];
-        X[i + ldx * j] = v / U[j + ldu * j];
-    }
-}
-
-// B (n x m) <- L^{-1} P B with LAPACK interchanges piv; one thread per column
-template <typename T>
-__global__ void piv_lower_cols(int n, const T* L, int64_t ldl, const int* piv, T* B, int64_t ldb, int m) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= m) return;
-    T* col = B + ldb * c;
-    for (int j = 0; j < n; ++j) {
-        const int p = piv[j];
-        if (p != j) { const T t = col[j]; col[j] = col[p]; col[p] = t; }
-    }
-    for (int i = 0; i < n; ++i) {
-        T v = col[i];
-        for (int l = 0; l < i; ++l) v -= L[i + ldl * l] * col[l];
-        col[i] = v;
-    }
-}
-
-// outputs of one eliminated large box (same layout as the one-CTA path)
-template <typename T>
-__global__ void big_elim_out_kernel(int k, int r, const T* A, int64_t ld, const T* Tm, T* pool, ElimDesc ed) {
-    const T* Arr = A;
-    const T* Asr = A + r;
-    const T* Ars = A + ld * r;
-    T* Dv = pool + ed.D_out;
-    T* LUo = pool + ed.LU_out;
-    T* Xo = pool + ed.X_out;
-    T* Yo = pool + ed.Y_out;
-    T* To = pool + ed.T_out;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    for (int64_t e = t0; e < r; e += stride) Dv[e] = Arr[e + ld * e];
-    for (int64_t e = t0; e < (int64_t)r * r; e += stride) {
-        const int i = (int)(e % r), j = (int)(e / r);
-        LUo[e] = i == j ? T(0) : (i < j ? Arr[i + ld * j] / Arr[i + ld * i] : Arr[i + ld * j]);
-    }
-    for (int64_t e = t0; e < (int64_t)k * r; e += stride) {
-        const int i = (int)(e % k), j = (int)(e / k);
-        Xo[e] = Asr[i + ld * j];
-        To[e] = Tm[e];
-    }
-    for (int64_t e = t0; e < (int64_t)r * k; e += stride) {
-        const int i = (int)(e % r), j = (int)(e / r);
-        Yo[e] = Ars[i + ld * j] / Arr[i + ld * i];
-    }
-}
-
-// inverses of the unit triangular factors stored in LU (one thread per column)
-template <typename T>
-__global__ void tri_inv_cols(int n, const T* A, T* out) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    const int64_t ld = n;
-    out[c + ld * c] = T(0);
-    for (int i = c + 1; i < n; ++i) {
-        T v = -A[i + ld * c];
-        for (int l = c + 1; l < i; ++l) v -= A[i + ld * l] * out[l + ld * c];
-        out[i + ld * c] = v;
-    }
-    for (int i = c - 1; i >= 0; --i) {
-        T v = -A[i + ld * c];
-        for (int l = i + 1; l < c; ++l) v -= A[i + ld * l] * out[l + ld * c];
-        out[i + ld * c] = v;
-    }
-}
-
-__global__ void piv_to_perm_kernel(const int* piv, int r, int* pm) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    for (int i = 0; i < r; ++i) pm[i] = i;
-    for (int j = 0; j < r; ++j) {
-        const int p = piv[j];
-        const int t = pm[j]; pm[j] = pm[p]; pm[p] = t;
-    }
 }
 
 // ---------------------------------------------- batched elimination ----
