@@ -1258,10 +1258,14 @@ __global__ void __launch_bounds__(FT) be_factor_kernel(BatchElimArgs a, int cl) 
             for (int s = warp; s < own; s += NW) {
                 const int q = rank + cl * s;
                 if (pos[q] < j || q == p) continue;
-                const T f = c[q] * inv;
+                // 64 bits: one multiplication less per entry, 64 cycles of a
+                // scheduler.  In 32 bits that gains nothing, and the rounding
+                // of c[q] * inv, common to the column, costs solve then apply
+                // 10-17% of its error (n = 512, 1024)
+                const T f = sizeof(T) == 8 ? c[q] * inv : c[q];
                 T* x = A + (size_t)r * s;
                 for (int i = lane; i < r; i += 32)
-                    if (i != p) x[i] -= c[i] * f;
+                    if (i != p) x[i] -= sizeof(T) == 8 ? c[i] * f : c[i] * f * inv;
             }
             if (p % cl == rank) {
                 T* x = A + (size_t)r * (p / cl);
@@ -1699,7 +1703,12 @@ __global__ void be_dinv_kernel(BatchElimArgs a) {
 // From the inverses of the diagonal blocks of size s to those of size 2 s:
 // with F = [F11 0; F21 F22] the block below is -inv(F22) (F21 inv(F11)).
 // PH 1: T = F21 inv(F11), into B_rr's work space (no longer needed); PH 2:
-// X21 = -inv(F22) T.  One CTA per 32 x 32 tile, pair of blocks and box, so a
+// X21 = -inv(F22) T.  An error of T reaches X21 times inv(F22), which block
+// substitution does not do, so one correction follows: PH 3: T += F22 X21, the
+// block of F X - I; PH 4: X21 -= inv(F22) T.  (32 bits, eps = 1e-6, solve then
+// apply, geometric mean of the relative error over 20 problems of n = 512: 9.3e-7
+// with block substitution, 1.0e-6 by doubling alone, 5.6e-7 with the correction;
+// 8 of n = 1024: 1.8e-6, 2.5e-6, 1.2e-6, for 1-5% of the factorization.)  One CTA per 32 x 32 tile, pair of blocks and box, so a
 // level fills the GPU.  (Block column by block column, each one a chain over
 // its blocks, the 3D n = 32 inverses took 39 ms, the n = 200 64-bit ones 21;
 // with the cluster panels the eliminations went from 123 to 46 and from 92 to
@@ -1726,6 +1735,8 @@ __global__ void __launch_bounds__(256) be_inv_level_kernel(BatchElimArgs a, int 
     auto inv_at = [&](int i, int j) -> T {
         return i < r && j < r ? (i == j ? T(1) : i > j ? *tri_x(X, r, xt, i, j) : T(0)) : T(0);
     };
+    // left operand F (PH 1, 3) or inv(F22); right operand X (PH 1, 3) or T
+    constexpr bool LF = PH == 1 || PH == 3;
     const int k0 = PH == 1 ? tj0 : 0, k1 = PH == 1 ? nt : ti0 + 1;
     for (int K = k0; K < k1; ++K) {
         const int g0 = (PH == 1 ? b : b + s) + IB * K;            // rows of the right operand
@@ -1734,15 +1745,16 @@ __global__ void __launch_bounds__(256) be_inv_level_kernel(BatchElimArgs a, int 
             const int u = q % IB, v = q / IB;
             {
                 // coalesced along the stored rows
-                const int i = (PH == 1 ? UP : xt) ? v : u, l = (PH == 1 ? UP : xt) ? u : v;
+                const int i = (LF ? UP : xt) ? v : u, l = (LF ? UP : xt) ? u : v;
                 const int gi = i0 + i, gl = g0 + l;
-                Ls[i][l] = PH == 1 ? (gi < r && gl < r ? tri_f<T, UP>(F, r, gi, gl) : T(0)) : inv_at(gi, gl);
+                if (LF) Ls[i][l] = gi < r && gl < gi ? tri_f<T, UP>(F, r, gi, gl) : T(gi < r && gl == gi);
+                else Ls[i][l] = inv_at(gi, gl);
             }
             {
-                const bool tr = PH == 1 && xt;
+                const bool tr = LF && xt;
                 const int l = tr ? v : u, c = tr ? u : v;
                 const int gl = g0 + l, gc = j0 + c;
-                Rs[l][c] = PH == 1 ? inv_at(gl, gc) : gl < r ? Tm[gl + ld * gc] : T(0);
+                Rs[l][c] = LF ? inv_at(gl, gc) : gl < r ? Tm[gl + ld * gc] : T(0);
             }
         }
         __syncthreads();
@@ -1759,7 +1771,9 @@ __global__ void __launch_bounds__(256) be_inv_level_kernel(BatchElimArgs a, int 
     for (int q = 0; q < 4; ++q) {
         const int gj = j0 + tj + 8 * q;
         if (PH == 1) Tm[gi + ld * gj] = acc[q];
-        else *tri_x(X, r, xt, gi, gj) = -acc[q];
+        if (PH == 2) *tri_x(X, r, xt, gi, gj) = -acc[q];
+        if (PH == 3) Tm[gi + ld * gj] += acc[q];
+        if (PH == 4) *tri_x(X, r, xt, gi, gj) -= acc[q];
     }
 }
 
@@ -2073,9 +2087,17 @@ cudaError_t big_elim_batch(const BatchElimArgs& a, int max_n, int max_k, int max
         note_launch();
         be_inv_level_kernel<T, false, 2><<<g, 256, 0, st>>>(a, s);
         note_launch();
+        be_inv_level_kernel<T, false, 3><<<g, 256, 0, st>>>(a, s);
+        note_launch();
+        be_inv_level_kernel<T, false, 4><<<g, 256, 0, st>>>(a, s);
+        note_launch();
         be_inv_level_kernel<T, true, 1><<<g, 256, 0, st>>>(a, s);
         note_launch();
         be_inv_level_kernel<T, true, 2><<<g, 256, 0, st>>>(a, s);
+        note_launch();
+        be_inv_level_kernel<T, true, 3><<<g, 256, 0, st>>>(a, s);
+        note_launch();
+        be_inv_level_kernel<T, true, 4><<<g, 256, 0, st>>>(a, s);
     }
     note_launch();
     be_finish_kernel<T><<<dim3((unsigned)std::clamp<int64_t>(((int64_t)max_k * max_r + 255) / 256, 1, 512), nb), 256,

@@ -64,3 +64,23 @@ def test_panel_elimination_matches_cluster(monkeypatch, n, dim, precision):
     for other in out[1:]:
         for p, q in zip(other, out[0]):
             assert float((p - q).abs().max()) <= tol * float(q.abs().max())
+
+
+@pytest.mark.parametrize("symmetric", [True, False])
+@pytest.mark.parametrize("seed", [1004, 1007, 1010])
+def test_fp32_solve_then_apply_returns_the_vector(symmetric, seed):
+    """F (F^{-1} f) = f up to the rounding of the FP32 factors alone.  Solve
+    and apply pass ~16 (sub)levels each; with one unit of rounding (2^-24 of
+    the vector) per level and pass the sum is at most 32 of them.  Triangular
+    inverses that amplify their own rounding miss this."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1307_2666_gb300 as P
+    pb = hi.volume_problem(512, 2, smooth_seed=seed, rhs_seed=1003, nrhs=2)
+    T = lambda v: torch.as_tensor(np.ascontiguousarray(v), dtype=torch.float64, device="cuda:0")
+    f = T(pb.f.T).t()
+    fac = P.Factorization(T(pb.points), T(pb.weights), T(pb.a), T(pb.b), T(pb.c), pb.kernel_id, 1e-6,
+                          precision="fp32", symmetric=symmetric, autotune=False)
+    err = float((fac.apply(fac.solve(f)) - f).norm() / f.norm())
+    fac.close()
+    assert err <= 32 * 2.0 ** -24
