@@ -411,17 +411,18 @@ __device__ inline int cta_argmax_v_o(double v, int o, int pos, double* wv, int* 
 // Column-pivoted Householder QR of W (mrow x ng; element (i, l) at
 // W[i * rs + l * cs], overwritten) to relative tolerance tol (Lemma 2.2 with
 // the adaptive rank of Sec. 2.2): pivot = largest remaining column 2-norm
-// (ties: lowest original index), norms kept in FP64 (kNormKeep), stop at the first step whose pivot norm is <= tol times the first
+// (ties: lowest original index), norms recomputed exactly in FP64 after every
+// step, stop at the first step whose pivot norm is <= tol times the first
 // one.  Writes k, the column order (skeletons in pivot order, then
 // redundants in ascending order) and T = R1^{-1} R2 (k x (ng-k),
 // column-major, columns in the redundant order).  Row-major W (cs = 1) makes
 // the per-column sweeps of the trailing update coalesced.  perm, rank_of: ng
 // ints; wv/wo/wp: 33 entries of scratch each.
 template <typename T>
-__device__ void cpqr_id(T* W, int rs, int cs, int mrow, int ng, double tol, double* nrm, double* nrm0, int* perm,
+__device__ void cpqr_id(T* W, int rs, int cs, int mrow, int ng, double tol, double* nrm, int* perm,
                         int* rank_of, double* wv, int* wo, int* wp, T* hh, T* Tout, int* pout, int* kout) {
     for (int l = threadIdx.x; l < ng; l += blockDim.x) perm[l] = l;
-    // ---- column-pivoted Householder QR
+    // ---- column-pivoted Householder QR with exact norm recomputation
     for (int l = threadIdx.x; l < ng; l += blockDim.x) {
         double s = 0.0;
         for (int i = 0; i < mrow; ++i) {
@@ -429,7 +430,6 @@ __device__ void cpqr_id(T* W, int rs, int cs, int mrow, int ng, double tol, doub
             s += v * v;
         }
         nrm[l] = s;
-        nrm0[l] = s;
     }
     __syncthreads();
     const int kmax = min(mrow, ng);
@@ -458,8 +458,7 @@ __device__ void cpqr_id(T* W, int rs, int cs, int mrow, int ng, double tol, doub
         __syncthreads();
         if (p != j && threadIdx.x == 0) {
             const int t = perm[j]; perm[j] = perm[p]; perm[p] = t;
-            double tn = nrm[j]; nrm[j] = nrm[p]; nrm[p] = tn;
-            tn = nrm0[j]; nrm0[j] = nrm0[p]; nrm0[p] = tn;
+            const double tn = nrm[j]; nrm[j] = nrm[p]; nrm[p] = tn;
         }
         // Householder reflector for W[j:, j]
         if (threadIdx.x < 32) {
@@ -499,16 +498,10 @@ __device__ void cpqr_id(T* W, int rs, int cs, int mrow, int ng, double tol, doub
                 col[j * rs] -= w;
                 for (int i = j + 1; i < mrow; ++i) col[i * rs] -= w * v[i * rs];
             }
-            // the square of the new norm (see kNormKeep)
-            const double rj = (double)col[j * rs];
-            double s = fmax(nrm[l] - rj * rj, 0.0);
-            if (!(s >= kNormKeep * nrm0[l])) {
-                s = 0.0;
-                for (int i = j + 1; i < mrow; ++i) {
-                    const double c = (double)col[i * rs];
-                    s += c * c;
-                }
-                nrm0[l] = s;
+            double s = 0.0;
+            for (int i = j + 1; i < mrow; ++i) {
+                const double c = (double)col[i * rs];
+                s += c * c;
             }
             nrm[l] = s;
         }
@@ -574,7 +567,7 @@ __device__ void id_group(const IdArgs& args, const int gidx) {
 
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned char* sp = smem;
-    double* nrm = align_ptr<double>(sp, 2 * (size_t)ng);
+    double* nrm = align_ptr<double>(sp, ng);
     int* perm = align_ptr<int>(sp, ng);
     int* rank_of = align_ptr<int>(sp, ng);
     double* redv = align_ptr<double>(sp, blockDim.x);
@@ -599,7 +592,7 @@ __device__ void id_group(const IdArgs& args, const int gidx) {
     double tol = rho * args.eps;
     if (tol < args.tol_floor) tol = args.tol_floor;
 
-    cpqr_id<T>(W, ldw, 1, mrow, ng, tol, nrm, nrm + ng, perm, rank_of, redv, redi, redi + 36, hh,
+    cpqr_id<T>(W, ldw, 1, mrow, ng, tol, nrm, perm, rank_of, redv, redi, redi + 36, hh,
                static_cast<T*>(args.Tws) + gd.T_off, args.perm_out + gd.perm_off, args.k_out + gidx);
 }
 
@@ -891,8 +884,8 @@ __global__ void __launch_bounds__(128) id_batched_kernel(const double* mats, con
     double* hh = align_ptr<double>(sp, 4);
     for (int e = threadIdx.x; e < mm * nn; e += blockDim.x) W[(e % mm) + (int64_t)ldw * (e / mm)] = M[e];
     __syncthreads();
-    cpqr_id<double>(W, 1, ldw, mm, nn, tol[b], nrm, W + (int64_t)ldw * nn, pm, rk, redv, redi, redi + 64, hh, T + toff[b],
-                    perm + poff[b], k + b);
+    cpqr_id<double>(W, 1, ldw, mm, nn, tol[b], nrm, pm, rk, redv, redi, redi + 64, hh, T + toff[b], perm + poff[b],
+                    k + b);
 }
 
 cudaError_t launch_id_batched(int count, const double* mats, const int64_t* off, const int* m, const int* n,
@@ -909,7 +902,7 @@ cudaError_t launch_id_batched(int count, const double* mats, const int64_t* off,
     int maxn = 1;
     for (int i = 0; i < count; ++i) {
         wso[i] = tot;
-        tot += (int64_t)(hm[i] | 1) * hn[i] + hn[i];          // the matrix and its columns' last exact norms
+        tot += (int64_t)(hm[i] | 1) * hn[i];
         maxn = std::max(maxn, hn[i]);
     }
     double* ws = nullptr;
@@ -956,7 +949,7 @@ size_t fold_smem_bytes(int n, int cpt, bool sci, bool R_in_smem, int elem) {
 }
 
 size_t id_smem_bytes(int ng, int mrow, bool W_in_smem, int elem) {
-    size_t b = (size_t)ng * 24 + 128 * 8 + 72 * 4 + 2 * (size_t)ng * elem + 4 * elem + 160;
+    size_t b = (size_t)ng * 16 + 128 * 8 + 72 * 4 + 2 * (size_t)ng * elem + 4 * elem + 160;
     if (W_in_smem) b += (size_t)mrow * ng * elem + 16;
     return b + 64;
 }
@@ -1138,7 +1131,7 @@ __global__ void __launch_bounds__(128) id_noalloc_kernel(unsigned char* scratch,
     double* ws = reinterpret_cast<double*>(scratch + kNoAllocOffBytes + kNoAllocFlagBytes);
     double* W = ws + reinterpret_cast<const int64_t*>(scratch)[b];
     const double* M = mats + off[b];
-    __shared__ double nrm[2 * kNoAllocMaxCols];
+    __shared__ double nrm[kNoAllocMaxCols];
     __shared__ int pm[kNoAllocMaxCols];
     __shared__ int rk[kNoAllocMaxCols];
     __shared__ double redv[128];
@@ -1146,8 +1139,8 @@ __global__ void __launch_bounds__(128) id_noalloc_kernel(unsigned char* scratch,
     __shared__ double hh[4];
     for (int e = threadIdx.x; e < mm * nn; e += blockDim.x) W[(e % mm) + (int64_t)ldw * (e / mm)] = M[e];
     __syncthreads();
-    cpqr_id<double>(W, 1, ldw, mm, nn, tol[b], nrm, nrm + nn, pm, rk, redv, redi, redi + 64, hh, T + toff[b],
-                    perm + poff[b], k + b);
+    cpqr_id<double>(W, 1, ldw, mm, nn, tol[b], nrm, pm, rk, redv, redi, redi + 64, hh, T + toff[b], perm + poff[b],
+                    k + b);
 }
 
 // Device address of the scratch array for the current device, looked up once
