@@ -338,8 +338,8 @@ struct BigBuffers {
 // The column-pivoted QR of all large groups of a sublevel: by panels of
 // HIF_BIG_QP_NB pivots (blocked, one trailing product per panel) or, at 1,
 // one launch pair per pivot.  Default: panels of 32 in FP32; one pivot per
-// step in FP64, whose norms (kNormKeep) keep the rank decisions of the
-// symmetric and full proxy matrices identical at eps = 1e-9 (the blocked
+// step in FP64, whose exact norms at every decision keep the rank decisions of
+// the symmetric and full proxy matrices identical at eps = 1e-9 (the blocked
 // update's rounding moved one decision at the threshold by one).
 template <typename T>
 static void run_big_pivoted_qr(BigArgs& a, BigBuffers& B, const std::vector<BigGroup>& bgv, int max_n, int maxk,

@@ -147,15 +147,6 @@ __device__ inline void y_pair(int kid, int rid, T rx0, T rx1, T rx2, T rb, T rwc
     }
 }
 
-// Squared column norms of the pivoted QRs (Lemma 2.2).  After a step the square
-// is the previous one less that of the new pivot row's entry; while it has
-// not fallen below kNormKeep of the last sum over the column, the subtractions
-// have cost it less than 1e-13 of its value, far below the rounding that the
-// column's own updates left in it, and it stands.  Then it is summed anew.
-// (Summed at every step, a third of the 64-bit steps' work, and most of the
-// 32-bit ones', were these sums.)
-constexpr double kNormKeep = 1e-2;
-
 __device__ inline double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;

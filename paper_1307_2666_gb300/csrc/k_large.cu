@@ -10,7 +10,7 @@
 //    big_update      launches per pivot step for all large groups at once: one
 //                    CTA per group picks the pivot and forms the reflector, a
 //                    warp per remaining column applies it and brings the
-//                    column norm up to date in FP64 (kNormKeep);
+//                    column norm up to date in FP64 (see kNormKeep);
 //  * big_T           T = R1^{-1} R2 and the skeleton / redundant order;
 //  * be_*            the batched elimination of medium and large boxes: Lemma
 //                    2.4 blocks, Lemma 2.1 LU or LDL, inverses and the Schur
@@ -222,6 +222,22 @@ __global__ void big_norm_init_kernel(BigArgs a) {
 
 constexpr int BST = 256;   // threads of the step kernel: one CTA walks the pivot column of m rows
 
+// Squared column norms of the pivot steps (Lemma 2.2).  In 64 bits the square
+// after a step is the previous one less that of the new pivot row's entry, until
+// it falls below kNormKeep of the last sum over the column and is summed anew
+// (summed at every step, a third of the 64-bit work of a step were these sums).
+// What a step decides, the pivot and the rank, it decides on sums: of the
+// columns whose carried square lies within kNormTie of the largest (several
+// of them, or one that close to the threshold) those not fresh are summed
+// first.  A carried square is off by at most 2^-53 of the last sum per
+// subtraction and by the rounding of the reflections, a few times m 2^-53 of
+// the square at worst: 1,000 steps on 10,000 rows cost at most 2e-7 of it at
+// the kNormKeep line, so no column outside that margin can be the largest.
+// A square is fresh while nrm0 > 0; a carried one has its last sum negated.
+// 32-bit columns, whose stored entries move by far more, are always summed.
+constexpr double kNormKeep = 1e-2;
+constexpr double kNormTie = 1e-6;
+
 template <typename T>
 __global__ void __launch_bounds__(BST) big_step_kernel(BigArgs a, int j) {
     const BigGroup G = a.groups[blockIdx.x];
@@ -240,25 +256,61 @@ __global__ void __launch_bounds__(BST) big_step_kernel(BigArgs a, int j) {
         if (threadIdx.x == 0) S->stop = 1;
         return;
     }
-    double best = -1.0;
-    int bl = -1, bo = 1 << 30;
-    for (int l = j + threadIdx.x; l < G.n; l += blockDim.x) {
-        const double v = nrm[l];
-        if (v > best || (v == best && perm[l] < bo)) { best = v; bo = perm[l]; bl = l; }
-    }
-    redv[threadIdx.x] = best;
-    redi[threadIdx.x] = bl;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            const double v2 = redv[threadIdx.x + s], v1 = redv[threadIdx.x];
-            const int l2 = redi[threadIdx.x + s], l1 = redi[threadIdx.x];
-            if (l2 >= 0 && (l1 < 0 || v2 > v1 || (v2 == v1 && perm[l2] < perm[l1]))) {
-                redv[threadIdx.x] = v2;
-                redi[threadIdx.x] = l2;
-            }
+    // largest square, ties to the lowest original column, in redv[0] and redi[0]
+    auto find_pivot = [&]() {
+        double best = -1.0;
+        int bl = -1, bo = 1 << 30;
+        for (int l = j + threadIdx.x; l < G.n; l += BST) {
+            const double v = nrm[l];
+            if (v > best || (v == best && perm[l] < bo)) { best = v; bo = perm[l]; bl = l; }
         }
+        redv[threadIdx.x] = best;
+        redi[threadIdx.x] = bl;
         __syncthreads();
+        for (int s = BST / 2; s > 0; s >>= 1) {
+            if (threadIdx.x < s) {
+                const double v2 = redv[threadIdx.x + s], v1 = redv[threadIdx.x];
+                const int l2 = redi[threadIdx.x + s], l1 = redi[threadIdx.x];
+                if (l2 >= 0 && (l1 < 0 || v2 > v1 || (v2 == v1 && perm[l2] < perm[l1]))) {
+                    redv[threadIdx.x] = v2;
+                    redi[threadIdx.x] = l2;
+                }
+            }
+            __syncthreads();
+        }
+    };
+    find_pivot();
+    {
+        // columns that could be the largest, and those of them not fresh
+        const double top = redv[0], line = (1.0 - kNormTie) * top;
+        int close = 0, carried = 0;
+        for (int l = j + threadIdx.x; l < G.n; l += BST)
+            if (nrm[l] >= line) {
+                ++close;
+                carried |= nrm0[l] < 0.0;
+            }
+        const bool several = __syncthreads_count(close > 0) > 1 || __syncthreads_or(close > 1);
+        const double th = j == 0 ? 0.0 : G.tol * S->nu0, th2 = th * th;
+        if (__syncthreads_or(carried) && (several || fabs(top - th2) <= kNormTie * th2)) {
+            const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+            for (int l0 = j + 32 * wid; l0 < G.n; l0 += BST) {
+                const int l = l0 + lane;
+                unsigned todo = __ballot_sync(0xffffffffu, l < G.n && nrm[l] >= line && nrm0[l] < 0.0);
+                for (; todo; todo &= todo - 1) {
+                    const int q = l0 + __ffs(todo) - 1;
+                    double sum = 0.0;
+#pragma unroll 8
+                    for (int i = j + lane; i < G.m; i += 32) {
+                        const double c = (double)W[i + ld * q];
+                        sum += c * c;
+                    }
+                    sum = warp_sum(sum);
+                    if (lane == 0) nrm[q] = nrm0[q] = sum;
+                }
+            }
+            __syncthreads();
+            find_pivot();
+        }
     }
     const double bnorm = sqrt(fmax(redv[0], 0.0));
     const int p = redi[0];
@@ -385,18 +437,18 @@ __global__ void __launch_bounds__(256, 4) big_update_kernel(BigArgs a, int j) {
     double* nrm = a.nrm + G.vec_off + l;
     double* nrm0 = a.nrm0 + G.vec_off + l;
     __syncwarp();
-    const double rj = (double)col[j];
-    double s = fmax(*nrm - rj * rj, 0.0);
+    const double rj = (double)col[j], last = fabs(*nrm0);
+    double s = fmax(*nrm - rj * rj, 0.0), sum = -last;
     __syncwarp();
-    if (!(s >= kNormKeep * *nrm0)) {
+    if (sizeof(T) == 4 || !(s >= kNormKeep * last)) {
         s = 0.0;
         for (int i = j + 1 + lane; i < G.m; i += 32) {
             const double c = (double)col[i];
             s += c * c;
         }
-        s = warp_sum(s);
-        if (lane == 0) *nrm0 = s;
+        sum = s = warp_sum(s);
     }
+    if (lane == 0) *nrm0 = sum;
     if (lane == 0) *nrm = s;
 }
 
