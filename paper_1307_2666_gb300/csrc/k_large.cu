@@ -1310,14 +1310,14 @@ __global__ void __launch_bounds__(FT) be_factor_kernel(BatchElimArgs a, int cl) 
             for (int s = warp; s < own; s += NW) {
                 const int q = rank + cl * s;
                 if (pos[q] < j || q == p) continue;
-                // 64 bits: one multiplication less per entry, 64 cycles of a
-                // scheduler.  In 32 bits that gains nothing, and the rounding
-                // of c[q] * inv, common to the column, costs solve then apply
-                // 10-17% of its error (n = 512, 1024)
-                const T f = sizeof(T) == 8 ? c[q] * inv : c[q];
+                // (c_i c_q) inv, which is the same for (i, q) and (q, i): the
+                // remaining block stays symmetric to the bit.  c_i (c_q inv)
+                // would save an operation, but its rounding of c_q inv is
+                // common to the column
+                const T f = c[q];
                 T* x = A + (size_t)r * s;
                 for (int i = lane; i < r; i += 32)
-                    if (i != p) x[i] -= sizeof(T) == 8 ? c[i] * f : c[i] * f * inv;
+                    if (i != p) x[i] -= c[i] * f * inv;
             }
             if (p % cl == rank) {
                 T* x = A + (size_t)r * (p / cl);
