@@ -188,7 +188,9 @@ __device__ __forceinline__ void product(const Team& tm, const Op<T>& A, int p, i
         for (int it = warp; it < mine * G; it += nw) {
             const int i0 = 32 * (tm.rank + tm.size * (it / G)) + R * (it % G);
             if (i0 >= p) continue;
-            const int lo = A.tri < 0 ? i0 + 1 : 0, hi = A.tri > 0 ? min(q, i0 + R - 1) : q;
+            // (lanes start from the tile's first row, not from i0: R depends on NC,
+            // the order of a row's sum must not)
+            const int lo = A.tri < 0 ? i0 / 32 * 32 + 1 : 0, hi = A.tri > 0 ? min(q, i0 + R - 1) : q;
             const T* col[R];
 #pragma unroll
             for (int u = 0; u < R; ++u) {
