@@ -1518,21 +1518,24 @@ static void sweep_one(hif_handle h, SubFactor& sf, int mode, T* xw, int nrhs, cu
     }
     if (!sf.nsmall) return;
     const int nc = sweep_nc(sf, nrhs, sizeof(T));
-    SweepArgs a{};
-    a.boxes = sf.sboxes.as<BoxFac>();
-    a.sk_ids = sf.sk.as<int>();
-    a.rd_ids = sf.rd.as<int>();
-    a.pool = sf.pool.p;
-    a.perm = sf.perm.as<int>();
-    a.x = xw;
-    a.ldx = nrhs;
-    a.nrhs = nrhs;
-    a.mode = mode;
-    a.cluster = sf.cluster;
-    a.gws = sf.global ? h->sweep_ws.p : nullptr;
-    a.gws_off = sf.global ? sf.gws_off.as<int64_t>() : nullptr;
     const size_t smem = sweep_smem_bytes(sf.global ? 0 : sf.max_kr2_small, nc, sf.threads, sizeof(T));
-    HIF_CUDA((launch_sweep<T>(a, sf.nsmall, nc, sf.threads, smem, st)));
+    const int most = 65535 * nc;                 // right-hand sides per launch (grid y)
+    for (int r0 = 0; r0 < nrhs; r0 += most) {
+        SweepArgs a{};
+        a.boxes = sf.sboxes.as<BoxFac>();
+        a.sk_ids = sf.sk.as<int>();
+        a.rd_ids = sf.rd.as<int>();
+        a.pool = sf.pool.p;
+        a.perm = sf.perm.as<int>();
+        a.x = xw + r0;
+        a.ldx = nrhs;
+        a.nrhs = std::min(most, nrhs - r0);
+        a.mode = mode;
+        a.cluster = sf.cluster;
+        a.gws = sf.global ? h->sweep_ws.p : nullptr;
+        a.gws_off = sf.global ? sf.gws_off.as<int64_t>() : nullptr;
+        HIF_CUDA((launch_sweep<T>(a, sf.nsmall, nc, sf.threads, smem, st)));
+    }
 }
 
 template <typename T>
