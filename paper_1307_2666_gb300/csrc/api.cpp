@@ -296,8 +296,11 @@ static void detect_grid(hif_handle h, Segment& sg) {
 }
 
 // The complex kernel on a full uniform grid: the table of its values by index
-// offset.  Only for points within rounding of the grid (the direct sum uses
-// the points themselves elsewhere); self: K_ii / w.
+// offset.  Only for points that lie on the grid to 1e-15 of its extent, so that
+// the table is off by no more than the sum's own rounding; the direct sum uses
+// the points themselves elsewhere, grids far from the origin among them (their
+// coordinates are rounded to the ulp of the distance: at 1e4 extents the table
+// would be off by 1e-11).  self: K_ii / w.
 static void detect_helmholtz_grid(hif_handle h, Segment& sg, double self_re, double self_im) {
     const int64_t np = sg.N / 2;
     std::vector<double> X(2 * (size_t)np), W((size_t)np);
@@ -312,11 +315,11 @@ static void detect_helmholtz_grid(hif_handle h, Segment& sg, double self_re, dou
     double hx = 0.0;
     if (!grid_layout(X.data(), W.data(), np, 2, 0, &n, &hx, point_of)) return;
     const double lo[2] = {X[2 * (size_t)point_of[0]], X[2 * (size_t)point_of[0] + 1]};
-    const double tol = 1e-15 * std::max({hx * n, std::fabs(lo[0]), std::fabs(lo[1])});
+    const double tol = 1e-15 * hx * n;
     for (int64_t g = 0; g < np; ++g)
         for (int k = 0; k < 2; ++k) {
-            const double at = lo[k] + hx * (double)(k == 0 ? g / n : g % n);
-            if (std::fabs(X[2 * (size_t)point_of[g] + k] - at) > tol) return;
+            const double at = X[2 * (size_t)point_of[g] + k] - lo[k];        // exact
+            if (std::fabs(at - hx * (double)(k == 0 ? g / n : g % n)) > tol) return;
         }
     upload(sg.dof_of, point_of, h->st);
     sg.table.ensure(sizeof(double) * 2 * (size_t)np);
