@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(BST) big_step_kernel(BigArgs a, int j) {
         }
     };
     find_pivot();
-    {
+    if constexpr (sizeof(T) == 8) {
         // columns that could be the largest, and those of them not fresh
         const double top = redv[0], line = (1.0 - kNormTie) * top;
         int close = 0, carried = 0;
@@ -292,14 +292,17 @@ __global__ void __launch_bounds__(BST) big_step_kernel(BigArgs a, int j) {
         const bool several = __syncthreads_count(close > 0) > 1 || __syncthreads_or(close > 1);
         const double th = j == 0 ? 0.0 : G.tol * S->nu0, th2 = th * th;
         if (__syncthreads_or(carried) && (several || fabs(top - th2) <= kNormTie * th2)) {
+            // (neighbours on different warps: the two columns of a complex
+            // unknown tie at every step)
             const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-            for (int l0 = j + 32 * wid; l0 < G.n; l0 += BST) {
-                const int l = l0 + lane;
+            constexpr int NW = BST / 32;
+            for (int l0 = j + wid; l0 < G.n; l0 += BST) {
+                const int l = l0 + NW * lane;
                 unsigned todo = __ballot_sync(0xffffffffu, l < G.n && nrm[l] >= line && nrm0[l] < 0.0);
                 for (; todo; todo &= todo - 1) {
-                    const int q = l0 + __ffs(todo) - 1;
+                    const int q = l0 + NW * (__ffs(todo) - 1);
                     double sum = 0.0;
-#pragma unroll 8
+#pragma unroll 16
                     for (int i = j + lane; i < G.m; i += 32) {
                         const double c = (double)W[i + ld * q];
                         sum += c * c;
