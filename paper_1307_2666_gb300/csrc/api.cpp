@@ -938,18 +938,29 @@ static void run_factor(hif_handle h) {
         p.box_off.assign(1, 0);
         p.near_off.assign(1, 0);
         p.grp_off.assign(1, 0);
-        // Four problems or more are planned side by side, one thread each
-        // (largest first); fewer one after the other, each with every thread.
-        // 24 problems of n <= 256, 16 Arm cores: plans of a factorization 88 ms
-        // one after the other.
+        // Large problems are planned one after the other, each with every
+        // thread, then the small ones side by side (plans_in_turn).  32-bit
+        // factorizations, 16 Arm cores, ms with one thread each from four
+        // problems on and now: 4 of n = 512 618 and 540, 4 of n = 1024 2,424 and
+        // 2,086, n = 1024 with three of n = 64 1,146 and 594, n = 512 with 100 of
+        // n = 64 451 and 329; 24 of n <= 240 336 and 336 (plans of 88 ms when all
+        // were made in turn).
         const int nseg = (int)h->segs.size();
         std::vector<SublevelPlan> plans(nseg);
         std::vector<double> ms(2 * (size_t)nseg, 0.0);
-        std::vector<int> order(nseg);
-        for (int q = 0; q < nseg; ++q) order[q] = q;
-        std::stable_sort(order.begin(), order.end(), [&](int u, int v) { return h->segs[u]->N > h->segs[v]->N; });
-        const bool across = nseg >= 4;
-        near_caches.resize(across ? (size_t)omp_get_max_threads() : 1);
+        std::vector<int64_t> act(nseg, 0), sizes;
+        std::vector<int> order;
+        for (int q = 0; q < nseg; ++q) {
+            const Segment& sg = *h->segs[q];
+            if (tau >= sg.kinds.size()) continue;
+            act[q] = std::count(active.begin() + sg.off, active.begin() + sg.off + sg.N, 1);
+            order.push_back(q);
+        }
+        std::stable_sort(order.begin(), order.end(), [&](int u, int v) { return act[u] > act[v]; });
+        for (int q : order) sizes.push_back(act[q]);
+        const int turns = plans_in_turn(sizes, omp_get_max_threads());
+        // (cache 0: all threads; the others: one thread each)
+        near_caches.resize(turns < (int)order.size() ? 1 + (size_t)omp_get_max_threads() : std::max<size_t>(near_caches.size(), 1));
         auto plan_one = [&](int q, NearCache* cache) {
             const Segment& sg = *h->segs[q];
             if (tau >= sg.kinds.size()) return;
@@ -968,23 +979,22 @@ static void run_factor(hif_handle h) {
             ms[2 * q] = std::chrono::duration<double, std::milli>(q1 - q0).count();
             ms[2 * q + 1] = std::chrono::duration<double, std::milli>(q2 - q1).count();
         };
-        if (across) {
-            std::exception_ptr failed;
+        // (in turn: not as a parallel region switched off, the regions inside
+        // would start new threads each time, n = 64 took 61 instead of 28 ms)
+        for (int z = 0; z < turns; ++z) plan_one(order[z], &near_caches[0]);
+        std::exception_ptr failed;
+        if (turns < (int)order.size()) {
 #pragma omp parallel for schedule(dynamic, 1)
-            for (int z = 0; z < nseg; ++z) {
+            for (int z = turns; z < (int)order.size(); ++z) {
                 try {
-                    plan_one(order[z], &near_caches[omp_get_thread_num()]);
+                    plan_one(order[z], &near_caches[1 + omp_get_thread_num()]);
                 } catch (...) {
 #pragma omp critical(hif_plan_failed)
                     failed = std::current_exception();
                 }
             }
-            if (failed) std::rethrow_exception(failed);
-        } else {
-            // (not as a parallel region switched off: the regions inside would
-            // start new threads each time, n = 64 took 61 instead of 28 ms)
-            for (int q = 0; q < nseg; ++q) plan_one(q, &near_caches[0]);
         }
+        if (failed) std::rethrow_exception(failed);
         for (int q = 0; q < nseg; ++q) {
             const Segment& sg = *h->segs[q];
             if (tau >= sg.kinds.size()) continue;

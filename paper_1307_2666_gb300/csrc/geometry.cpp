@@ -409,6 +409,29 @@ bool grid_layout(const double* X, const double* Wt, int64_t N, int d, int64_t of
     return true;
 }
 
+int plans_in_turn(const std::vector<int64_t>& active, int threads) {
+    const int n = (int)active.size();
+    if (threads < 2) return n;
+    const double start = 48.0 * threads, all = 0.7 * threads;
+    double rest = 0.0, turn = 0.0, least = 0.0;
+    for (int64_t a : active) rest += (double)a;
+    int best = 0;
+    for (int k = 0; k <= n; ++k) {
+        if (k != n - 1) {
+            const double t = turn + (k == n ? 0.0 : start + std::max((double)active[k], rest / all));
+            if (k == 0 || t < least) {
+                least = t;
+                best = k;
+            }
+        }
+        if (k < n) {
+            turn += start + (double)active[k] / all;
+            rest -= (double)active[k];
+        }
+    }
+    return n == 1 ? 1 : best;
+}
+
 void geometry_trace(bool on, double* ms) {
     if (ms)
         for (int q = 0; q < 6; ++q) ms[q] = g_geo_ms[q];
