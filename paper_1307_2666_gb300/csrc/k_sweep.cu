@@ -54,7 +54,10 @@ __host__ __device__ constexpr int ldl_mode(int m) {
 // one: 0.50 -> 0.16 ms.
 // Row tiles of 32 go to the CTAs of a cluster in turn.  The order of every sum
 // depends on the box and the launch shape of its sublevel only, not on the
-// number of right-hand sides.
+// number of right-hand sides: R and with it the first column that the lanes
+// take of a transposed triangular product do depend on it, but that only turns
+// the columns round the lanes, and the tree of exchanges (distances 16, 8, 4, 2,
+// 1) pairs the same sums however they are turned.
 
 namespace {
 
@@ -188,9 +191,7 @@ __device__ __forceinline__ void product(const Team& tm, const Op<T>& A, int p, i
         for (int it = warp; it < mine * G; it += nw) {
             const int i0 = 32 * (tm.rank + tm.size * (it / G)) + R * (it % G);
             if (i0 >= p) continue;
-            // (lanes start from the tile's first row, not from i0: R depends on NC,
-            // the order of a row's sum must not)
-            const int lo = A.tri < 0 ? i0 / 32 * 32 + 1 : 0, hi = A.tri > 0 ? min(q, i0 + R - 1) : q;
+            const int lo = A.tri < 0 ? i0 + 1 : 0, hi = A.tri > 0 ? min(q, i0 + R - 1) : q;
             const T* col[R];
 #pragma unroll
             for (int u = 0; u < R; ++u) {
