@@ -149,11 +149,7 @@ struct SubFactor {
     std::vector<BoxFac> hbox;
     DevMem boxes, sk, rd, pool, perm;
     int max_kr2 = 0;               // max over boxes of k + 2 r
-    // sweep plan: CTAs per box and CTA size; boxes whose vectors exceed shared
-    // memory use a global work space (offsets per right-hand side)
-    bool global = false;
-    DevMem gws_off;
-    int64_t gws_units = 0;
+    // sweep plan: CTAs per box and CTA size
     int threads = 256, cluster = 1;
     // boxes of the cluster sweep kernel (sboxes) and the wide boxes whose
     // passes run as stage launches over the whole GPU (wboxes, work space at
@@ -1507,7 +1503,7 @@ enum { SOLVE_UP = 0, SOLVE_DOWN = 1, APPLY_UP = 2, APPLY_DOWN = 3,
 // most 8, halved until the sublevel's largest box fits into shared memory.
 static int sweep_nc(const SubFactor& sf, int nrhs, size_t elem) {
     int nc = nrhs > 4 ? 8 : nrhs > 2 ? 4 : nrhs;
-    while (nc > 1 && !sf.global && sweep_smem_bytes(sf.max_kr2_small, nc, sf.threads, (int)elem) > kSweepSmemMax) nc /= 2;
+    while (nc > 1 && sweep_smem_bytes(sf.max_kr2_small, nc, sf.threads, (int)elem) > kSweepSmemMax) nc /= 2;
     return nc;
 }
 
@@ -1531,7 +1527,7 @@ static void sweep_one(hif_handle h, SubFactor& sf, int mode, T* xw, int nrhs, cu
     }
     if (!sf.nsmall) return;
     const int nc = sweep_nc(sf, nrhs, sizeof(T));
-    const size_t smem = sweep_smem_bytes(sf.global ? 0 : sf.max_kr2_small, nc, sf.threads, sizeof(T));
+    const size_t smem = sweep_smem_bytes(sf.max_kr2_small, nc, sf.threads, sizeof(T));
     const int most = 65535 * nc;                 // right-hand sides per launch (grid y)
     for (int r0 = 0; r0 < nrhs; r0 += most) {
         SweepArgs a{};
@@ -1545,8 +1541,6 @@ static void sweep_one(hif_handle h, SubFactor& sf, int mode, T* xw, int nrhs, cu
         a.nrhs = std::min(most, nrhs - r0);
         a.mode = mode;
         a.cluster = sf.cluster;
-        a.gws = sf.global ? h->sweep_ws.p : nullptr;
-        a.gws_off = sf.global ? sf.gws_off.as<int64_t>() : nullptr;
         HIF_CUDA((launch_sweep<T>(a, sf.nsmall, nc, sf.threads, smem, st)));
     }
 }
@@ -1562,7 +1556,7 @@ static void sweep_seq(hif_handle h, T* xw, int nrhs, int op, cudaStream_t st) {
 static void ensure_sweep_ws(hif_handle h, int nrhs, size_t elem) {
     int64_t need = 1;
     for (auto& sf : h->subs)
-        need = std::max({need, sf->gws_units * (std::max(nrhs, 1) + 7), sf->wws_units * std::min(std::max(nrhs, 1), 16)});
+        need = std::max(need, sf->wws_units * std::min(std::max(nrhs, 1), 16));
     h->sweep_ws.ensure(elem * (size_t)need);
 }
 
@@ -1616,8 +1610,8 @@ static void sweep_all(hif_handle h, T* xw, int nrhs, int op) {
     g_launches.fetch_add(g->kernels);
 }
 
-// After the factorization: the launch shape and the global work-space offsets
-// of every sublevel's sweep.
+// After the factorization: the launch shape of every sublevel's sweep and the
+// work-space offsets of its wide boxes.
 template <typename T>
 static void prepare_sweeps(hif_handle h) {
     const cudaStream_t st = h->st;
@@ -1630,11 +1624,12 @@ static void prepare_sweeps(hif_handle h) {
             sf.sweep_perm_ints += r;
             sf.sweep_vec_elems += k + r;
         }
-        // LU boxes above 8,192 rows take the stage path over the whole GPU
-        // (HIF_SWEEP_WIDE: another line).  The cluster kernel was the faster
-        // of the two at every width measured: 64-bit n = 200, boxes of up to
-        // 1,153 rows, 3.8 ms with every box above 768 rows on the stage path
-        // and 1.6 ms with none; 3D n = 32, up to 1,968 rows, 5.2 and 1.7 ms.
+        // LU boxes above 8,192 rows, and those whose vectors do not fit into
+        // shared memory, take the stage path over the whole GPU
+        // (HIF_SWEEP_WIDE: another line).  The cluster kernel was the faster of
+        // the two at every width measured: 64-bit n = 200, boxes of up to 1,153
+        // rows, 3.8 ms with every box above 768 rows on the stage path and 1.6 ms
+        // with none; 3D n = 32, up to 1,968 rows, 5.2 and 1.7 ms. 
         const int wide_min = env_int("HIF_SWEEP_WIDE", 8192);
         std::vector<BoxFac> sb, wb;
         std::vector<int64_t> woffs;
@@ -1642,7 +1637,9 @@ static void prepare_sweeps(hif_handle h) {
         int max_kr = 0;
         sf.wws_units = 0;
         for (const BoxFac& bf : sf.hbox) {
-            if (!bf.ldl && bf.k + bf.r > wide_min) {
+            const bool fits = sweep_smem_bytes(bf.k + 2 * bf.r, 1, 512, sizeof(T)) <= kSweepSmemMax;
+            if (bf.ldl && !fits) fail(HIF_EINVAL, "symmetric box too large for the sweep kernel");
+            if (!bf.ldl && (bf.k + bf.r > wide_min || !fits)) {
                 wb.push_back(bf);
                 woffs.push_back(sf.wws_units);
                 sf.wws_units += (int64_t)bf.k + 2 * (int64_t)bf.r;
@@ -1669,18 +1666,6 @@ static void prepare_sweeps(hif_handle h) {
         sf.threads = max_kr <= 96                                                               ? 128
                      : sf.cluster == 8 && max_kr > 512 && sf.cluster * sf.nsmall <= h->num_sms ? 512
                                                                                                 : 256;
-        sf.global = sweep_smem_bytes(sf.max_kr2_small, 1, sf.threads, sizeof(T)) > kSweepSmemMax;
-        if (sf.global) sf.cluster = 1;
-        sf.gws_units = 0;
-        if (!sf.global || !sf.nsmall) continue;
-        std::vector<int64_t> offs(sb.size());
-        int64_t tot = 0;
-        for (size_t q = 0; q < sb.size(); ++q) {
-            offs[q] = tot;
-            tot += (int64_t)(sb[q].k + 2 * sb[q].r);
-        }
-        upload(sf.gws_off, offs, st);
-        sf.gws_units = tot;
     }
 }
 

@@ -1063,9 +1063,9 @@ __global__ void be_T_kernel(BatchElimArgs a) {
     }
 }
 
-// the GEMMs of Lemma 2.4 and the Schur update, one op per launch:
+// the GEMMs of Lemma 2.4, one op per launch:
 // 0: B_sr = A_sr - A_ss T     1: B_rr -= T^T B_sr     2: B_rr -= A_rs T
-// 3: B_rs = A_rs - T^T A_ss   4: S = -X Z (into the SCI pool)
+// 3: B_rs = A_rs - T^T A_ss
 // TS x TS tiles: 64, or 32 where the boxes give few of them.
 template <typename T, int TS>
 __global__ void __launch_bounds__(256) be_gemm_kernel(BatchElimArgs a, int op) {
@@ -1086,17 +1086,12 @@ __global__ void __launch_bounds__(256) be_gemm_kernel(BatchElimArgs a, int op) {
     const T* Bm;
     T* C;
     int64_t lda, ldb, ldc;
-    bool tA = false, tB = false;
+    bool tA = false;
     switch (op) {
         case 0: m = k; n = r; kk = k; A = Ass; lda = ld; Bm = Bx.Tm; ldb = k; C = Asr; ldc = ld; break;
         case 1: m = r; n = r; kk = k; A = Bx.Tm; lda = k; tA = true; Bm = Asr; ldb = ld; C = Arr; ldc = ld; break;
         case 2: m = r; n = r; kk = k; A = Ars; lda = ld; Bm = Bx.Tm; ldb = k; C = Arr; ldc = ld; break;
-        case 3: if (d.ldl) return; m = r; n = k; kk = k; A = Bx.Tm; lda = k; tA = true; Bm = Ass; ldb = ld; C = Ars; ldc = ld; break;
-        default:
-            if (k == 0 || d.sci_out < 0) return;
-            m = k; n = k; kk = r; A = Asr; lda = ld; Bm = Ars; ldb = ld;
-            C = static_cast<T*>(a.sci_pool) + d.sci_out; ldc = k;
-            break;
+        default: if (d.ldl) return; m = r; n = k; kk = k; A = Bx.Tm; lda = k; tA = true; Bm = Ass; ldb = ld; C = Ars; ldc = ld; break;
     }
     const int i0 = blockIdx.x * TS, j0 = blockIdx.y * TS;
     if (i0 >= m || j0 >= n || kk == 0) return;
@@ -1111,7 +1106,7 @@ __global__ void __launch_bounds__(256) be_gemm_kernel(BatchElimArgs a, int op) {
             As[l][rr] = v;
             const int jj = j0 + rr;
             T u = T(0);
-            if (jj < n && kx < kk) u = tB ? Bm[jj + ldb * kx] : Bm[kx + ldb * jj];
+            if (jj < n && kx < kk) u = Bm[kx + ldb * jj];
             Bs[l][rr] = u;
         }
         __syncthreads();
@@ -1132,10 +1127,7 @@ __global__ void __launch_bounds__(256) be_gemm_kernel(BatchElimArgs a, int op) {
     for (int p = 0; p < Q; ++p)
         for (int q = 0; q < Q; ++q) {
             const int i = i0 + tx + 16 * p, jj = j0 + ty + 16 * q;
-            if (i < m && jj < n) {
-                if (op == 4) C[i + ldc * jj] = -acc[p][q];
-                else C[i + ldc * jj] -= acc[p][q];
-            }
+            if (i < m && jj < n) C[i + ldc * jj] -= acc[p][q];
         }
 }
 

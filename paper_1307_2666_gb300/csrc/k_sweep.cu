@@ -90,8 +90,7 @@ __device__ __forceinline__ void st_peer(uint32_t a, double v) {
 __device__ __forceinline__ void st_peer(uint32_t a, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
-// *p = v in every CTA of the team (p: this CTA's shared or, for a team of
-// one, global memory)
+// *p = v in every CTA of the team (p: this CTA's shared memory)
 template <typename T>
 __device__ __forceinline__ void put_all(const Team& tm, T* p, T v) {
     if (tm.size == 1) {
@@ -235,14 +234,12 @@ sweep_kernel(SweepArgs a) {
     constexpr int U = BIG ? 16 : 8;
     const Team tm{(int)(blockIdx.x % a.cluster), a.cluster};
     if (tm.size > 1) cluster_arrive();               // waited for before the first store to a peer
-    const int bi = blockIdx.x / a.cluster;
-    const BoxFac bf = a.boxes[bi];
+    const BoxFac bf = a.boxes[blockIdx.x / a.cluster];
     const int k = bf.k, r = bf.r, c0 = blockIdx.y * NC, nr = min(NC, a.nrhs - c0);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using V = Row<T, NC>;
     T* red = reinterpret_cast<T*>(smem_raw);
     V* xs = reinterpret_cast<V*>(red + (blockDim.x / 32) * 32 * NC);
-    if (a.gws) xs = static_cast<V*>(a.gws) + (a.gws_off[bi] * gridDim.y + (int64_t)blockIdx.y * (k + 2 * r));
     V* xr = xs + k;
     V* tmp = xr + r;
     T* x = static_cast<T*>(a.x) + c0;
@@ -372,7 +369,7 @@ cudaError_t launch_nc(const SweepArgs& a, int nbox, int threads, size_t smem, cu
 template <typename T>
 cudaError_t launch_sweep(const SweepArgs& a, int nbox, int nc, int threads, size_t smem, cudaStream_t st) {
     if (nbox == 0) return cudaSuccess;
-    if (threads < 32 || threads > 512 || threads % 32 || a.cluster < 1 || a.cluster > 8 || (a.gws && a.cluster > 1))
+    if (threads < 32 || threads > 512 || threads % 32 || a.cluster < 1 || a.cluster > 8)
         return cudaErrorInvalidValue;
     const bool big = threads > 256;
     switch (nc) {

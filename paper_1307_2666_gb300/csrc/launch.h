@@ -82,8 +82,6 @@ struct SweepArgs {
     int nrhs;
     int mode;               // see k_sweep.cu
     int cluster;            // CTAs per box (1, 2, 4, 8)
-    void* gws;              // non-null: per-box vectors in global memory at gws_off[box] * nrhs (rounded up
-    const int64_t* gws_off; // to the launch's nc; boxes too large for shared memory, one CTA each)
 };
 
 // ---- large boxes: unpivoted blocked QR to the n x n factor R (k_bigqr.cu)
@@ -239,7 +237,6 @@ template <typename T> cudaError_t launch_elim(const ElimArgs&, int nbox, int num
 // sweeps
 // nc: right-hand sides held per CTA (1, 2, 4, 8); threads: CTA size, a
 // multiple of 32 up to 512; smem: sweep_smem_bytes of the largest k + 2 r
-// (0 units of k + 2 r with gws)
 constexpr size_t kSweepSmemMax = 224 * 1024;
 size_t sweep_smem_bytes(int k2r, int nc, int threads, int elem);
 template <typename T>
