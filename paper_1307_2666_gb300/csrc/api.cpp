@@ -1629,7 +1629,12 @@ static void prepare_sweeps(hif_handle h) {
         // (HIF_SWEEP_WIDE: another line).  The cluster kernel was the faster of
         // the two at every width measured: 64-bit n = 200, boxes of up to 1,153
         // rows, 3.8 ms with every box above 768 rows on the stage path and 1.6 ms
-        // with none; 3D n = 32, up to 1,968 rows, 5.2 and 1.7 ms. 
+        // with none; 3D n = 32, up to 1,968 rows, 5.2 and 1.7 ms. One solve with
+        // 1, 8 and 16 right-hand sides, stage path / cluster, one box of r = 2,304:
+        // 1.46, 1.48, 1.51 / 0.43, 1.05, 1.06 ms (64-bit), 0.54, 0.56, 0.59 /
+        // 0.40, 0.47, 0.47 (32-bit); r = 4,096: 3.2, 3.3, 3.3 / 1.0, 1.5, 1.5;
+        // r = 8,100: 6.2, 6.3, 6.5 / 3.1, 2.9, 6.0 (64-bit) and 4.4, 4.5, 4.6 /
+        // 2.6, 2.6, 2.5 (32-bit); four boxes of 4,096: 6.8, 7.0, 7.1 / 1.3, 3.4, 5.0.
         const int wide_min = env_int("HIF_SWEEP_WIDE", 8192);
         std::vector<BoxFac> sb, wb;
         std::vector<int64_t> woffs;
