@@ -1635,6 +1635,8 @@ static void prepare_sweeps(hif_handle h) {
         // 0.40, 0.47, 0.47 (32-bit); r = 4,096: 3.2, 3.3, 3.3 / 1.0, 1.5, 1.5;
         // r = 8,100: 6.2, 6.3, 6.5 / 3.1, 2.9, 6.0 (64-bit) and 4.4, 4.5, 4.6 /
         // 2.6, 2.6, 2.5 (32-bit); four boxes of 4,096: 6.8, 7.0, 7.1 / 1.3, 3.4, 5.0.
+        // With 128: r = 4,096 20.8 / 7.0 and 7.6 / 2.2, r = 8,100 50.5 / 24.9 and
+        // 35.3 / 11.4, n = 200 35.3 / 18.8, 3D n = 32 28.4 / 5.8.
         const int wide_min = env_int("HIF_SWEEP_WIDE", 8192);
         std::vector<BoxFac> sb, wb;
         std::vector<int64_t> woffs;
