@@ -140,6 +140,17 @@ class ClockSampler:
 
 # --------------------------------------------------------------- GPU arm ---
 
+def conv_digit_flops(n, nrhs):
+    """BF16 digit products (2 flops each) of one full tc_conv_kernel launch on the
+    n x n grid: 1,024 columns of 128 x 128 per slot; a slot is a distance along
+    the slow axis, a chunk of 128 sources and one of 128 targets for a tile of 32
+    columns (target line, right-hand side), and the source lines on both sides
+    of the tile share it."""
+    lines = 32 // (1 << max(0, nrhs - 1).bit_length())
+    distances = sum(max(min(lo + lines, n) - 1, n - 1 - lo) + 1 for lo in range(0, n, lines))
+    return 2.0 * 128 * 1024 * 128 * distances * (-(-n // 128)) ** 2
+
+
 def alu_peaks(peaks):
     """FP32 and FP64 SIMT peaks from the unit counts and the measured maximum
     SM clock: 152 SMs x 128 FP32 lanes (one FMA = 2 flop per clock) and
@@ -301,9 +312,9 @@ def run_gpu(args):
     groups = -(-nrhs // 8)
     # algorithmic work of the method (Sec. 8 roofline of the direct sum):
     # 2 N^2 flops per right-hand side; the kernel forms them from exact 8-bit
-    # digit products, 256 BF16 MACs per (target, source) pair and 8 RHS
+    # digit products
     flops_launch = 2.0 * N * N * min(nrhs, 8)
-    digit_flops_launch = 512.0 * N * N * min(nrhs, 8) / 8.0
+    digit_flops_launch = conv_digit_flops(n, min(nrhs, 8))
     t_launch = (tc_ms / 1000.0 / tc_launches) if tc_launches else float("nan")
     achieved = flops_launch / t_launch / 1e12
     peak = peaks.get("bf16_tflops_sustained", 1700.0)
