@@ -235,6 +235,9 @@ constexpr int BST = 256;   // threads of the step kernel: one CTA walks the pivo
 // the kNormKeep line, so no column outside that margin can be the largest.
 // A square is fresh while nrm0 > 0; a carried one has its last sum negated.
 // 32-bit columns, whose stored entries move by far more, are always summed.
+// Pivot steps of n = 200, b != c, 203.5 ms, n = 64 8.2, Helmholtz n = 64, where
+// the two columns of an unknown tie at every step, 36.1; deciding on the carried
+// squares alone 202.1, 7.8 and 32.9; sums at every step cost n = 200 40 ms more.
 constexpr double kNormKeep = 1e-2;
 constexpr double kNormTie = 1e-6;
 
@@ -1178,8 +1181,9 @@ __global__ void be_probs_kernel(BatchElimArgs a, int op, TcGemmProb* out) {
 // the lowest position as they do there.  Output in position order: LU (L
 // strictly below the diagonal), or for LDL boxes L below, D, and D L^T above.
 // Measured on a GB300 against the one-CTA and panel kernels this replaces: a
-// 64-bit LDL block of 388 rows 60 -> 8 ms with all its stages, and 4 with the
-// searches on integers and one reciprocal per step.
+// 64-bit LDL block of 388 rows 60 -> 8 ms with all its stages; all eliminations of
+// n = 64 (it and four blocks of 348) 12 ms, with the searches on integers and one
+// reciprocal per step 8.7 (7.2 with the unsymmetric update below).
 constexpr int FT = 512;
 constexpr int FCL = 8;                       // largest cluster
 constexpr size_t kFactorSmemMax = 224 * 1024;
@@ -1307,8 +1311,8 @@ __global__ void __launch_bounds__(FT) be_factor_kernel(BatchElimArgs a, int cl) 
                 if (pos[q] < j || q == p) continue;
                 // (c_i c_q) inv, which is the same for (i, q) and (q, i): the
                 // remaining block stays symmetric to the bit.  c_i (c_q inv)
-                // would save an operation, but its rounding of c_q inv is
-                // common to the column
+                // would save an operation (1.5 ms at n = 64, 64 bits), but its
+                // rounding of c_q inv is common to the column
                 const T f = c[q];
                 T* x = A + (size_t)r * s;
                 for (int i = lane; i < r; i += 32)
