@@ -314,7 +314,7 @@ static void detect_helmholtz_grid(hif_handle h, Segment& sg, double self_re, dou
     const double tol = 1e-15 * hx * n;
     for (int64_t g = 0; g < np; ++g)
         for (int k = 0; k < 2; ++k) {
-            const double at = X[2 * (size_t)point_of[g] + k] - lo[k];        // exact
+            const double at = X[2 * (size_t)point_of[g] + k] - lo[k];   // off by an ulp of the extent at most
             if (std::fabs(at - hx * (double)(k == 0 ? g / n : g % n)) > tol) return;
         }
     upload(sg.dof_of, point_of, h->st);
